@@ -56,22 +56,17 @@ SMI_FIELDS = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.act
 IR_MODES = {"restart": 0, "continue": 1}
 # DRAM bytes (read + write) per launch of the dominant kernels from one ncu
 # capture (profiles/kv_f32_cg2_cantilever_120x60x30_full.md,
-# profiles/kv_f32_cg2_cantilever_256x128x150_full.md,
-# profiles/kv_f64_pcg_cantilever_256x128x150_full.md, the FP64 figure scaled from
-# 4,915,200 to 216,000 elements by the bytes it reads per element), cold caches,
-# each with a digest of the kernel's source files at capture time: when the
-# sources change the figure is reported as stale (null) until it is re-taken.
+# profiles/kv_f32_cg2_cantilever_256x128x150_full.md), cold caches, each with a
+# digest of the kernel's source files at capture time: when the sources change the figure is reported as stale (null) until it is re-taken.
 KERNEL_SOURCES = {
     "cg2_kv_kernel": ["kv_column.cuh", "pcg_f32.cu", "modes.cuh"],
-    "pcg_kv_tile_kernel<double>": ["kv_tile.cuh", "kv_tile.cu", "modes.cuh"],
+    "pcg_kv_col64_kernel": ["kv_column64.cuh", "kv_tile.cu", "modes.cuh"],
 }
 NCU_DRAM_BYTES = {
     ("cg2_kv_kernel<2>", WORKLOAD): (6.646272e6, "0c045bd0c8e8"),
     ("cg2_kv_kernel<3>", WORKLOAD): (6.649088e6, "0c045bd0c8e8"),
     ("cg2_kv_kernel<2>", "cantilever_256x128x150"): (143.325184e6 + 74.990592e6, "0c045bd0c8e8"),
     ("cg2_kv_kernel<3>", "cantilever_256x128x150"): (144.233472e6 + 74.192384e6, "0c045bd0c8e8"),
-    ("pcg_kv_tile_kernel<double>", WORKLOAD): ((293.127936e6 + 199.873024e6) * 216000 / 4915200,
-                                               "6e176c6f4f1e"),
 }
 
 
@@ -632,7 +627,7 @@ def gpu_bench(args, rank, local_rank, world):
     sm_mhz = clk["sm_mhz"] or 1950.0
     n_sm = torch.cuda.get_device_properties(local_rank).multi_processor_count
     if args.form == "mixed":
-        kname = ("pcg_kv_tile_kernel<float>" if args.inner_form == "f32"
+        kname = ("pcg_kv_block_kernel" if args.inner_form == "f32"
                  else f"pcg_kv_tc_kernel ({args.inner_form})")
         if args.inner_form == "f32" and not persistent:
             kbase = "cg2_kv_kernel" if args.cg_engine == 2 else "pcg_kv_col_kernel"
@@ -662,8 +657,8 @@ def gpu_bench(args, rank, local_rank, world):
         fp64_peak_tflops = n_sm * 2 * 2 * sm_mhz * 1e6 / 1e12   # 2 DFMA/clk/SM, measured clock
         roof = {"bound": "alu", "achieved": FLOP_PER_ELEM * m.n_elem / kv_avg_s / 1e12,
                 "peak": fp64_peak_tflops, "unit": "TFLOP/s",
-                "kernel": "pcg_kv_tile_kernel<double>",
-                "traffic": ncu_traffic("pcg_kv_tile_kernel<double>", WORKLOAD)[0],
+                "kernel": "pcg_kv_col64_kernel",
+                "traffic": ncu_traffic("pcg_kv_col64_kernel", WORKLOAD)[0],
                 "peak_source": f"FP64 FMA pipe, {n_sm} SMs x 2 DFMA/clk x 2 flop x "
                                f"{sm_mhz:.0f} MHz median SM clock under load",
                 "flop_per_elem": FLOP_PER_ELEM}

@@ -108,6 +108,7 @@ struct mfto_handle {
   int occ_col[2];           // ... of the FP32 column kernel kinds (kv_tile.cu)
   int col_nzc;              // node layers per z-chunk of the column kernels (0: automatic)
   int col_kind;             // column kernel kind (mfto_kv_autotune)
+  int col64_shape, col64_nzc;  // tile shape and z-chunk of the FP64 column K.v (kv_tile.cu)
   int tcol_nzc;             // node layers per z-chunk of the tensor-core column kernel (0: automatic)
   unsigned int* d_bar;      // tree grid-barrier counters of the persistent CG (zeroed)
   int occ_tc[12];           // ... of the tensor-core kernels, [2 * (2 kind + split) + pcg]

@@ -1,55 +1,36 @@
-// Launchers of the tiled mode-space K.v (kv_tile.cuh): plain y = K v and the
-// CG form that also forms p_new = z + beta p_old, q = K p_new and alpha.
+// Launchers of the mode-space K.v kernels (FP32: kv_column.cuh and the block
+// variant of kv_tile.cuh; FP64: kv_column64.cuh): plain y = K v and the CG form
+// that also forms p_new = z + beta p_old, q = K p_new and alpha.
 #include "common.cuh"
 #include "kv_column.cuh"
+#include "kv_column64.cuh"
 #include "kv_tile.cuh"
 
 namespace {
 
-constexpr int kTX = 16, kTY = 12;   // owned nodes per CTA in x, y; 256 threads
-using Shape = TileShape<kTX, kTY>;
-
-// FP64 runs the z-streaming ring variant (bound by the FP64 pipe, little halo
-// recompute); FP32 runs the one-element-per-thread block variant (bound by
-// memory latency otherwise, so it trades halo arithmetic for parallelism).
-template <typename T>
-struct UseBlock { static constexpr bool value = sizeof(T) == 4; };
-static_assert(Shape::NE <= MFTO_BLOCK && Shape::NV <= MFTO_BLOCK, "tile larger than the block");
-
-template <typename T, typename Load, typename Epi>
-__device__ __forceinline__ double tile_body(const T* E, const uint8_t* fixed, const ModeCoef<T>& K,
-                                            const Grid& g, int nzc, const Load& ld, const Epi& epi,
-                                            T* smem) {
-  if constexpr (UseBlock<T>::value)
-    return kv_block_body<T>(E, fixed, K, g, ld, epi, smem);
-  else
-    return kv_tile_body<T, kTX, kTY>(E, fixed, K, g, nzc, ld, epi, smem);
-}
-
-template <typename T>
+// FP32, variant 2: one element per thread in 8 x 8 x 4 blocks (kv_block_body).
 __global__ void __launch_bounds__(MFTO_BLOCK)
-kv_tile_kernel(const T* __restrict__ E, const T* __restrict__ v, T* __restrict__ y,
-               const uint8_t* __restrict__ fixed, ModeCoef<T> K, Grid g, int nzc) {
+kv_block_kernel(const float* __restrict__ E, const float* __restrict__ v, float* __restrict__ y,
+                const uint8_t* __restrict__ fixed, ModeCoef<float> K, Grid g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  tile_body<T>(E, fixed, K, g, nzc, TileLoadPlain<T>{v}, TileStore<T>{v, y},
-               reinterpret_cast<T*>(smem_raw));
+  kv_block_body<float>(E, fixed, K, g, TileLoadPlain<float>{v}, TileStore<float>{v, y},
+                       reinterpret_cast<float*>(smem_raw));
 }
 
-template <typename T>
 __global__ void __launch_bounds__(MFTO_BLOCK)
-pcg_kv_tile_kernel(const T* __restrict__ E, const T* __restrict__ z, const T* __restrict__ p_old,
-                   T* __restrict__ p_new, T* __restrict__ q, const uint8_t* __restrict__ fixed,
-                   ModeCoef<T> K, Grid g, int nzc, PcgScalars* s, double* partials) {
+pcg_kv_block_kernel(const float* __restrict__ E, const float* __restrict__ z,
+                    const float* __restrict__ p_old, float* __restrict__ p_new,
+                    float* __restrict__ q, const uint8_t* __restrict__ fixed, ModeCoef<float> K,
+                    Grid g, PcgScalars* s, double* partials) {
   if (*(volatile int32_t*)&s->done) return;  // uniform over the grid
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double sh[64];
-  const T beta = (T)s->beta;
+  const float beta = (float)s->beta;
   double red[1];
-  red[0] = tile_body<T>(E, fixed, K, g, nzc, TileLoadDirection<T>{z, p_old, beta},
-                        TilePcg<T>{p_new, q}, reinterpret_cast<T*>(smem_raw));
+  red[0] = kv_block_body<float>(E, fixed, K, g, TileLoadDirection<float>{z, p_old, beta},
+                                TilePcg<float>{p_new, q}, reinterpret_cast<float*>(smem_raw));
   double tot[1];
-  if (last_block_reduce<1, DotAcc<T>::kWarpReduced>(red, partials, &s->ticket_b, tot, sh) &&
-      threadIdx.x == 0) {
+  if (last_block_reduce<1, true>(red, partials, &s->ticket_b, tot, sh) && threadIdx.x == 0) {
     s->pq = tot[0];
     if (!(tot[0] > 0.0) || !isfinite(tot[0])) {
       s->done = 1;
@@ -59,6 +40,116 @@ pcg_kv_tile_kernel(const T* __restrict__ E, const T* __restrict__ z, const T* __
       s->alpha = s->rz / tot[0];
     }
   }
+}
+
+// FP64: column-streaming body (kv_column64.cuh), one tile per CTA.  Launch
+// bounds: 256 resident threads per SM are enough to keep the FP64 pipe busy
+// and leave each the registers of a whole element.
+template <int CX, int CY>
+__global__ void __launch_bounds__(CX * CY, 256 / (CX * CY))
+kv_col64_kernel(const double* __restrict__ E, const double* __restrict__ v,
+                double* __restrict__ y, const uint8_t* __restrict__ fixed, ModeCoef<double> K,
+                Grid g, Col64Tiling tl) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  kv_column64_body<CX, CY>(E, fixed, K, g, tl, blockIdx.x, Col64LoadPlain{v}, Col64Store{v, y},
+                           reinterpret_cast<double*>(smem_raw));
+}
+
+template <int CX, int CY>
+__global__ void __launch_bounds__(CX * CY, 256 / (CX * CY))
+pcg_kv_col64_kernel(const double* __restrict__ E, const double* __restrict__ z,
+                    const double* __restrict__ p_old, double* __restrict__ p_new,
+                    double* __restrict__ q, const uint8_t* __restrict__ fixed,
+                    ModeCoef<double> K, Grid g, Col64Tiling tl, PcgScalars* s,
+                    double* partials) {
+  if (*(volatile int32_t*)&s->done) return;  // uniform over the grid
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double sh[64];
+  double red[1];
+  red[0] = kv_column64_body<CX, CY>(E, fixed, K, g, tl, blockIdx.x,
+                                    Col64LoadDirection{z, p_old, s->beta}, Col64Pcg{p_new, q},
+                                    reinterpret_cast<double*>(smem_raw));
+  double tot[1];
+  if (last_block_reduce<1>(red, partials, &s->ticket_b, tot, sh) && threadIdx.x == 0) {
+    s->pq = tot[0];
+    if (!(tot[0] > 0.0) || !isfinite(tot[0])) {
+      s->done = 1;
+      s->status = MFTO_BREAKDOWN;
+      s->alpha = 0.0;
+    } else {
+      s->alpha = s->rz / tot[0];
+    }
+  }
+}
+
+// Calls f with the tile shape of index i (mfto_handle::col64_shape).
+constexpr int kCol64Shapes = 5;
+template <typename F>
+mfto_status col64_dispatch(int i, const F& f) {
+  switch (i) {
+    case 0: return f(Col64Shape<32, 8>{});
+    case 1: return f(Col64Shape<16, 16>{});
+    case 2: return f(Col64Shape<32, 4>{});
+    case 3: return f(Col64Shape<16, 8>{});
+    default: return f(Col64Shape<8, 16>{});
+  }
+}
+
+// Tile shape and z-chunk of the FP64 kernel for a mesh.  A CTA of NT threads
+// over nzc owned node layers executes (nzc + 1) element layers of NT / 32
+// warps, and an SM's FP64 pipe takes its CTAs one after another, so the time
+// is that of the SM with the most CTAs: ceil(tiles / SMs) x NT x (nzc + 1 +
+// about half a layer of prologue and tail).  Every shape and every balanced
+// chunk length is tried (host arithmetic, once per handle).
+void col64_choose(mfto_handle* h) {
+  const Grid g = make_grid(h->mesh);
+  double best = 0.0;
+  for (int i = 0; i < kCol64Shapes; ++i)
+    col64_dispatch(i, [&](auto shape) -> mfto_status {
+      using S = decltype(shape);
+      const int64_t txy = (int64_t)((g.nx + S::OX - 1) / S::OX) * ((g.ny + S::OY - 1) / S::OY);
+      for (int tz = 1; tz <= g.nz; ++tz) {
+        const int nzc = (g.nz + tz - 1) / tz;
+        if ((g.nz + nzc - 1) / nzc != tz) continue;       // not a balanced count
+        if (txy * tz > MFTO_RED_SLOTS && tz > 1) break;    // one partial per CTA
+        const double cost = (double)((txy * tz + h->num_sms - 1) / h->num_sms) * S::NT *
+                            (nzc + 1.5);
+        if (best == 0.0 || cost < best) {
+          best = cost;
+          h->col64_shape = i;
+          h->col64_nzc = nzc;
+        }
+      }
+      return MFTO_OK;
+    });
+}
+
+template <typename S>
+Col64Tiling col64_tiling(const mfto_handle* h) {
+  const Grid g = make_grid(h->mesh);
+  Col64Tiling t;
+  t.tx = (g.nx + S::OX - 1) / S::OX;
+  t.ty = (g.ny + S::OY - 1) / S::OY;
+  t.nzc = h->col64_nzc;
+  t.tz = (g.nz + t.nzc - 1) / t.nzc;
+  return t;
+}
+
+mfto_status col64_attrs(mfto_handle* h) {
+  for (int i = 0; i < kCol64Shapes; ++i) {
+    const mfto_status s = col64_dispatch(i, [&](auto shape) -> mfto_status {
+      using S = decltype(shape);
+      MFTO_CUDA(h, cudaFuncSetAttribute(kv_col64_kernel<S::CX, S::CY>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)S::template smem_bytes<1>()));
+      MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_col64_kernel<S::CX, S::CY>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)S::template smem_bytes<2>()));
+      return MFTO_OK;
+    });
+    if (s != MFTO_OK) return s;
+  }
+  return MFTO_OK;
 }
 
 // FP32, variant 0: column-streaming body (kv_column.cuh).  MINB: resident
@@ -261,44 +352,15 @@ pcg_kv_col_kernel(const float* __restrict__ E, const float* __restrict__ z,
 // CTAs per SM.
 constexpr int kColKinds = 2;
 
-template <typename T>
-dim3 tile_grid(const mfto_handle* h, int* nzc_out, int per_sm = 1) {
+// grid-stride over 7 x 7 x 3 node blocks; one wave of resident CTAs
+unsigned block_grid(const mfto_handle* h, int per_sm) {
   const Grid g = make_grid(h->mesh);
-  if (UseBlock<T>::value) {
-    // grid-stride over 7 x 7 x 3 node blocks; one wave of resident CTAs
-    const int64_t nb = (int64_t)((g.nx + 6) / 7) * ((g.ny + 6) / 7) * ((g.nz + 2) / 3);
-    int64_t grid = (int64_t)per_sm * h->num_sms;
-    if (grid > nb) grid = nb;
-    *nzc_out = 0;
-    return dim3((unsigned)grid, 1, 1);
-  }
-  const int tx = (g.nx + kTX - 1) / kTX, ty = (g.ny + kTY - 1) / kTY;
-  const int target = (sizeof(T) == 8 ? 2 : 4) * h->num_sms;
-  int zch = (target + tx * ty / 2) / (tx * ty);
-  if (zch < 1) zch = 1;
-  if (zch > g.nz) zch = g.nz;
-  int nzc = (g.nz + zch - 1) / zch;
-  if (nzc < 4) nzc = g.nz < 4 ? g.nz : 4;
-  int tz = (g.nz + nzc - 1) / nzc;
-  // the CG form reduces one partial per block
-  if ((int64_t)tx * ty * tz > MFTO_RED_SLOTS) return dim3(0, 0, 0);
-  *nzc_out = nzc;
-  return dim3(tx, ty, tz);
+  const int64_t nb = (int64_t)((g.nx + 6) / 7) * ((g.ny + 6) / 7) * ((g.nz + 2) / 3);
+  const int64_t grid = (int64_t)per_sm * h->num_sms;
+  return (unsigned)(grid > nb ? nb : grid);
 }
 
-template <typename T>
-size_t tile_smem() {
-  return UseBlock<T>::value ? BlockShape::smem_bytes<T>() : Shape::smem_bytes<T>();
-}
-
-template <typename T>
-mfto_status set_attrs(mfto_handle* h) {
-  const int smem = (int)tile_smem<T>();
-  MFTO_CUDA(h, cudaFuncSetAttribute(kv_tile_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_tile_kernel<T>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  return MFTO_OK;
-}
+constexpr size_t kBlockSmem = BlockShape::smem_bytes<float>();
 
 }  // namespace
 
@@ -317,9 +379,13 @@ ColTiling col_launch_tiling(const mfto_handle* h, int per_sm, int* grid) {
 }
 
 mfto_status kv_tile_init(mfto_handle* h) {
-  mfto_status s = set_attrs<double>(h);
-  if (s == MFTO_OK) s = set_attrs<float>(h);
+  col64_choose(h);
+  const mfto_status s = col64_attrs(h);
   if (s != MFTO_OK) return s;
+  MFTO_CUDA(h, cudaFuncSetAttribute(kv_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kBlockSmem));
+  MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_block_kernel,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlockSmem));
   const int csm = (int)kColSmem;
   MFTO_CUDA(h, cudaFuncSetAttribute(kv_col_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, csm));
   MFTO_CUDA(h, cudaFuncSetAttribute(kv_col_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, csm));
@@ -355,20 +421,13 @@ mfto_status kv_tile_init(mfto_handle* h) {
   for (int k = 0; k < kColKinds; ++k)
     if (h->occ_col[k] < 1) h->occ_col[k] = 1;
   MFTO_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                   &h->occ_kv32, kv_tile_kernel<float>, MFTO_BLOCK, tile_smem<float>()));
+                   &h->occ_kv32, kv_block_kernel, MFTO_BLOCK, kBlockSmem));
   MFTO_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                   &h->occ_pcg32, pcg_kv_tile_kernel<float>, MFTO_BLOCK, tile_smem<float>()));
+                   &h->occ_pcg32, pcg_kv_block_kernel, MFTO_BLOCK, kBlockSmem));
   if (h->occ_kv32 < 1) h->occ_kv32 = 1;
   if (h->occ_pcg32 < 1) h->occ_pcg32 = 1;
   return MFTO_OK;
 }
-
-template <typename T>
-static const ModeCoef<T>& coef(const mfto_handle* h);
-template <>
-const ModeCoef<double>& coef<double>(const mfto_handle* h) { return h->mc64; }
-template <>
-const ModeCoef<float>& coef<float>(const mfto_handle* h) { return h->mc32; }
 
 // One l1-Jacobi sweep on the FP32 operator fused with it (first: from x = 0,
 // writing x and A x; otherwise x -> xo).  Needs the column kernel (variant 0).
@@ -433,71 +492,81 @@ mfto_status gmg_cheb_col_launch(mfto_handle* h, int mode, const float* E, const 
   return MFTO_OK;
 }
 
-template <typename T>
-mfto_status kv_tile_launch(mfto_handle* h, const T* E, const T* v, T* y, cudaStream_t st) {
-  if (sizeof(T) == 4 && h->kv_variant == 0) {
+template <>
+mfto_status kv_tile_launch<double>(mfto_handle* h, const double* E, const double* v, double* y,
+                                   cudaStream_t st) {
+  const mfto_status s = col64_dispatch(h->col64_shape, [&](auto shape) -> mfto_status {
+    using S = decltype(shape);
+    const Col64Tiling tl = col64_tiling<S>(h);
+    kv_col64_kernel<S::CX, S::CY><<<tl.count(), S::NT, S::template smem_bytes<1>(), st>>>(
+        E, v, y, h->d_fixed, h->mc64, make_grid(h->mesh), tl);
+    return MFTO_OK;
+  });
+  MFTO_LAUNCH_CHECK(h);
+  return s;
+}
+
+template <>
+mfto_status kv_tile_launch<float>(mfto_handle* h, const float* E, const float* v, float* y,
+                                  cudaStream_t st) {
+  const Grid g = make_grid(h->mesh);
+  if (h->kv_variant == 0) {
     int grid = 0;
     const int kind = h->col_kind;
     const ColTiling tl = col_launch_tiling(h, h->occ_col[kind], &grid);
-    const Grid g = make_grid(h->mesh);
-    const float *Ef = (const float*)E, *vf = (const float*)v;
-    float* yf = (float*)y;
     const size_t sm = kColSmem;
     if (kind == 1)
-      kv_col_kernel<3><<<grid, MFTO_BLOCK, sm, st>>>(Ef, vf, yf, h->d_fixed, h->mc32, g, tl);
+      kv_col_kernel<3><<<grid, MFTO_BLOCK, sm, st>>>(E, v, y, h->d_fixed, h->mc32, g, tl);
     else
-      kv_col_kernel<2><<<grid, MFTO_BLOCK, sm, st>>>(Ef, vf, yf, h->d_fixed, h->mc32, g, tl);
-    MFTO_LAUNCH_CHECK(h);
-    return MFTO_OK;
+      kv_col_kernel<2><<<grid, MFTO_BLOCK, sm, st>>>(E, v, y, h->d_fixed, h->mc32, g, tl);
+  } else {
+    kv_block_kernel<<<block_grid(h, h->occ_kv32), MFTO_BLOCK, kBlockSmem, st>>>(
+        E, v, y, h->d_fixed, h->mc32, g);
   }
-  int nzc = 0;
-  const dim3 grid = tile_grid<T>(h, &nzc, h->occ_kv32);
-  if (grid.x == 0) return mfto_fail(h, MFTO_TOO_LARGE, "mesh too large for the K.v tiling");
-  kv_tile_kernel<T><<<grid, MFTO_BLOCK, tile_smem<T>(), st>>>(
-      E, v, y, h->d_fixed, coef<T>(h), make_grid(h->mesh), nzc);
   MFTO_LAUNCH_CHECK(h);
   return MFTO_OK;
 }
 
-template <typename T>
-mfto_status pcg_kv_tile_launch(mfto_handle* h, const T* E, const T* z, const T* p_old, T* p_new,
-                               T* q, PcgScalars* s, double* partials, cudaStream_t st) {
-  if (sizeof(T) == 4 && h->kv_variant == 0) {
+template <>
+mfto_status pcg_kv_tile_launch<double>(mfto_handle* h, const double* E, const double* z,
+                                       const double* p_old, double* p_new, double* q,
+                                       PcgScalars* s, double* partials, cudaStream_t st) {
+  const mfto_status r = col64_dispatch(h->col64_shape, [&](auto shape) -> mfto_status {
+    using S = decltype(shape);
+    const Col64Tiling tl = col64_tiling<S>(h);
+    if (tl.count() > MFTO_RED_SLOTS)
+      return mfto_fail(h, MFTO_TOO_LARGE, "mesh too large for the K.v tiling");
+    pcg_kv_col64_kernel<S::CX, S::CY><<<tl.count(), S::NT, S::template smem_bytes<2>(), st>>>(
+        E, z, p_old, p_new, q, h->d_fixed, h->mc64, make_grid(h->mesh), tl, s, partials);
+    return MFTO_OK;
+  });
+  MFTO_LAUNCH_CHECK(h);
+  return r;
+}
+
+template <>
+mfto_status pcg_kv_tile_launch<float>(mfto_handle* h, const float* E, const float* z,
+                                      const float* p_old, float* p_new, float* q, PcgScalars* s,
+                                      double* partials, cudaStream_t st) {
+  const Grid g = make_grid(h->mesh);
+  if (h->kv_variant == 0) {
     int grid = 0;
     const int kind = h->col_kind;
     const ColTiling tl = col_launch_tiling(h, h->occ_col[kind], &grid);
-    const Grid g = make_grid(h->mesh);
-    const float *Ef = (const float*)E, *zf = (const float*)z, *pf = (const float*)p_old;
-    float *pn = (float*)p_new, *qf = (float*)q;
     const size_t sm = kColSmem;
     if (kind == 1)
-      pcg_kv_col_kernel<3><<<grid, MFTO_BLOCK, sm, st>>>(Ef, zf, pf, pn, qf, h->d_fixed, h->mc32,
-                                                         g, tl, s, partials);
+      pcg_kv_col_kernel<3><<<grid, MFTO_BLOCK, sm, st>>>(E, z, p_old, p_new, q, h->d_fixed,
+                                                         h->mc32, g, tl, s, partials);
     else
-      pcg_kv_col_kernel<2><<<grid, MFTO_BLOCK, sm, st>>>(Ef, zf, pf, pn, qf, h->d_fixed, h->mc32,
-                                                         g, tl, s, partials);
-    MFTO_LAUNCH_CHECK(h);
-    return MFTO_OK;
+      pcg_kv_col_kernel<2><<<grid, MFTO_BLOCK, sm, st>>>(E, z, p_old, p_new, q, h->d_fixed,
+                                                         h->mc32, g, tl, s, partials);
+  } else {
+    pcg_kv_block_kernel<<<block_grid(h, h->occ_pcg32), MFTO_BLOCK, kBlockSmem, st>>>(
+        E, z, p_old, p_new, q, h->d_fixed, h->mc32, g, s, partials);
   }
-  int nzc = 0;
-  const dim3 grid = tile_grid<T>(h, &nzc, h->occ_pcg32);
-  if (grid.x == 0) return mfto_fail(h, MFTO_TOO_LARGE, "mesh too large for the K.v tiling");
-  pcg_kv_tile_kernel<T><<<grid, MFTO_BLOCK, tile_smem<T>(), st>>>(
-      E, z, p_old, p_new, q, h->d_fixed, coef<T>(h), make_grid(h->mesh), nzc, s, partials);
   MFTO_LAUNCH_CHECK(h);
   return MFTO_OK;
 }
-
-template mfto_status kv_tile_launch<double>(mfto_handle*, const double*, const double*, double*,
-                                            cudaStream_t);
-template mfto_status kv_tile_launch<float>(mfto_handle*, const float*, const float*, float*,
-                                           cudaStream_t);
-template mfto_status pcg_kv_tile_launch<double>(mfto_handle*, const double*, const double*,
-                                                const double*, double*, double*, PcgScalars*,
-                                                double*, cudaStream_t);
-template mfto_status pcg_kv_tile_launch<float>(mfto_handle*, const float*, const float*,
-                                               const float*, float*, float*, PcgScalars*,
-                                               double*, cudaStream_t);
 
 // Times the FP32 column K.v (as one inner CG iteration with the graph CG
 // engines, as a plain K.v otherwise) for every balanced chunk length along z
