@@ -109,6 +109,7 @@ struct mfto_handle {
   int col_nzc;              // node layers per z-chunk of the column kernels (0: automatic)
   int col_kind;             // column kernel kind (mfto_kv_autotune)
   int col64_shape, col64_nzc;  // tile shape and z-chunk of the FP64 column K.v (kv_tile.cu)
+  int energy_shape, energy_nzc;  // ... of the compliance kernel (simp.cu)
   int tcol_nzc;             // node layers per z-chunk of the tensor-core column kernel (0: automatic)
   unsigned int* d_bar;      // tree grid-barrier counters of the persistent CG (zeroed)
   int occ_tc[12];           // ... of the tensor-core kernels, [2 * (2 kind + split) + pcg]
@@ -671,6 +672,7 @@ mfto_status cg2_enqueue(mfto_handle* h, cudaStream_t st, const PcgVecs<float>& v
                         cudaEvent_t ev1);
 mfto_status pcg_persist_iterate(mfto_handle* h, const PcgVecs<float>& v, PcgScalars* host_s);
 mfto_status kv_tile_init(mfto_handle* h);
+mfto_status simp_init(mfto_handle* h);
 template <typename T>
 mfto_status kv_tile_launch(mfto_handle* h, const T* E, const T* v, T* y, cudaStream_t st);
 template <typename T>

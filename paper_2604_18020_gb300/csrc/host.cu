@@ -350,6 +350,7 @@ extern "C" mfto_status mfto_create(const mfto_mesh* mesh, const mfto_params* par
     return MFTO_CUDA_ERROR;
   }
   mfto_status s = kv_tile_init(h);
+  if (s == MFTO_OK) s = simp_init(h);
   if (s == MFTO_OK) s = pcg_persist_init(h);
   if (s == MFTO_OK) s = cg2_attrs(h);
   if (s == MFTO_OK) h->cg_engine = 2;

@@ -38,12 +38,15 @@ struct Col64Shape {
   static constexpr int OX = CX - 1, OY = CY - 1;           // owned nodes per layer
   static constexpr int ROW = 6 * CX;                       // one edge row: s, d x 3 components
   static_assert(NT % 32 == 0 && CX <= 32, "whole warps, x neighbours within a warp");
+  // shared memory of the node stream (ring, node edges) and, for the K.v, of
+  // the back edges [2][CY][ROW] and own values [3][3][NT]
+  template <int KSRC>
+  static constexpr size_t stream_bytes() {
+    return sizeof(double) * (size_t)(2 * 3 * KSRC * NV + 2 * (CY + 1) * ROW);
+  }
   template <int KSRC>
   static constexpr size_t smem_bytes() {
-    // ring [2][3 KSRC][NV], node edges [2][CY + 1][ROW], back edges
-    // [2][CY][ROW], own values [3][3][NT]
-    return sizeof(double) *
-           (size_t)(2 * 3 * KSRC * NV + 2 * (CY + 1) * ROW + 2 * CY * ROW + 9 * NT);
+    return stream_bytes<KSRC>() + sizeof(double) * (size_t)(2 * CY * ROW + 9 * NT);
   }
 };
 
@@ -86,6 +89,19 @@ struct Col64Face {
   double m[3][4];
 };
 
+// z stage: modes m = f + 4 (z difference) of the element between face modes lo
+// (below) and up (above).  Mode 0, a translation, is left 0.
+__device__ __forceinline__ void col64_modes(const Col64Face& lo, const Col64Face& up,
+                                            double (&X)[3][8]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      X[c][f] = f == 0 ? 0.0 : lo.m[c][f] + up.m[c][f];
+      X[c][f | 4] = up.m[c][f] - lo.m[c][f];
+    }
+}
+
 // Element layer between face modes lo_f (below) and up_f (above), unit mode
 // operator, modulus and undone z stage: up (in: the upper-face outputs of the
 // element below, out: this one's) and Ms = up_in + this element's lower-face
@@ -94,13 +110,7 @@ __device__ __forceinline__ void col64_element(const Col64Face& lo_f, const Col64
                                               double E, const ModeCoef<double>& K, Col64Face& up,
                                               Col64Face& Ms) {
   double X[3][8], Y[3][8];
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      X[c][f] = f == 0 ? 0.0 : lo_f.m[c][f] + up_f.m[c][f];
-      X[c][f | 4] = up_f.m[c][f] - lo_f.m[c][f];
-    }
+  col64_modes(lo_f, up_f, X);
 #pragma unroll
   for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -160,44 +170,54 @@ struct Col64Pcg {                     // CG: p_new stored, q = K p_new, p_new.q 
   }
 };
 
-// Tile `tile` of `tl`; returns this thread's share of the epilogue reduction.
-template <int CX, int CY, typename Load, typename Epi>
-__device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
-                                                   const uint8_t* __restrict__ fixed,
-                                                   const ModeCoef<double>& K, const Grid& g,
-                                                   const Col64Tiling& tl, int tile,
-                                                   const Load& ld, const Epi& epi, double* smem) {
+// The node layers of a tile of CX x CY element columns, streamed along z: raw
+// values copied asynchronously two layers ahead into a ring (each thread reads
+// only its own copies, so the ring needs no barrier), the x stage of every
+// edge row into shared memory, the y stage into registers.  fixed NULL: no
+// masks.
+template <int CX, int CY, typename Load>
+struct Col64Stream {
   using S = Col64Shape<CX, CY>;
-  constexpr int KS = Load::kSrc;
-  double* ring = smem;                                 // [2][3 KS][NV]
-  double* edges = ring + 2 * 3 * KS * S::NV;           // [2][CY + 1][6][CX], slot of layer k: k & 1
-  double* back = edges + 2 * (CY + 1) * S::ROW;        // [2][CY][6][CX], slot of layer k: k & 1
-  double* ownv = back + 2 * CY * S::ROW;               // [3][3][NT], slot of layer k: (k + 3) % 3
-  const int tid = threadIdx.x;
-  const int ex = tid % CX, ey = tid / CX;
-  const int bx = tile % tl.tx, by = (tile / tl.tx) % tl.ty, bz = tile / (tl.tx * tl.ty);
-  const int gi = bx * S::OX - 1 + ex, gj = by * S::OY - 1 + ey;   // element column and node
-  const int kb = bz * tl.nzc, ke = min(kb + tl.nzc, g.nz);        // owned node layers [kb, ke)
-  const int nxy = g.nx * g.ny, nexy = g.nelx * g.nely;
-  // the thread's nodes of a layer: its own, the tile's last column for the
-  // last thread of a row, the tile's last row for the threads of the last row
-  const bool re = ex == CX - 1, te = ey == CY - 1;
-  const bool in_x0 = gi >= 0 && gi < g.nx, in_x1 = gi + 1 < g.nx;
-  const bool in_y0 = gj >= 0 && gj < g.ny, in_y1 = gj + 1 < g.ny;
-  const bool in0 = in_x0 && in_y0, in1 = re && in_x1 && in_y0;
-  const bool in2 = te && in_x0 && in_y1, in3 = re && te && in_x1 && in_y1;
-  const int nb0 = gi + g.nx * gj;
-  const bool elem_in = gi >= 0 && gj >= 0 && gi < g.nelx && gj < g.nely;
-  const bool own_node = ex >= 1 && ey >= 1 && in0;
-  const bool warp_elem = __any_sync(0xffffffffu, elem_in);
-  const bool warp_own = __any_sync(0xffffffffu, own_node);
-  double red = 0.0;
+  static constexpr int KS = Load::kSrc;
+  // ring [2][3 KS][NV], node edges [2][CY + 1][6][CX]; slot of layer k: k & 1
+  static constexpr int kRing = 2 * 3 * KS * S::NV, kEdges = 2 * (CY + 1) * S::ROW;
+  static constexpr int kDoubles = kRing + kEdges;
+  double *ring, *edges;
+  const Load& ld;
+  const uint8_t* fixed;
+  const Grid& g;
+  int ex, ey, gi, gj, nb0, nxy, last;   // last: the topmost node layer to copy
+  bool re, te, in0, in1, in2, in3;
+  double eo[6];   // this column's lower-y edge of the node layer staged last
 
-  // copies of node layer L into ring slot L & 1 and the masks of its nodes
-  // (own | right << 8 | top << 16 | corner << 24); fm: the masks of L
-  auto issue = [&](int L) -> uint32_t {
+  // (i0, j0): element column and node of thread 0
+  __device__ __forceinline__ Col64Stream(double* smem, const Load& load, const uint8_t* fix,
+                                         const Grid& grid, int i0, int j0, int last_layer)
+      : ring(smem), edges(smem + kRing), ld(load), fixed(fix), g(grid) {
+    ex = threadIdx.x % CX;
+    ey = threadIdx.x / CX;
+    gi = i0 + ex;
+    gj = j0 + ey;
+    last = min(last_layer, g.nz - 1);
+    nxy = g.nx * g.ny;
+    nb0 = gi + g.nx * gj;
+    // the thread's nodes of a layer: its own, the tile's last column for the
+    // last thread of a row, the tile's last row for the threads of the last row
+    re = ex == CX - 1;
+    te = ey == CY - 1;
+    const bool in_x0 = gi >= 0 && gi < g.nx, in_x1 = gi + 1 < g.nx;
+    const bool in_y0 = gj >= 0 && gj < g.ny, in_y1 = gj + 1 < g.ny;
+    in0 = in_x0 && in_y0;
+    in1 = re && in_x1 && in_y0;
+    in2 = te && in_x0 && in_y1;
+    in3 = re && te && in_x1 && in_y1;
+  }
+
+  // copies node layer L into its ring slot; returns the masks of the thread's
+  // nodes (own | right << 8 | top << 16 | corner << 24)
+  __device__ __forceinline__ uint32_t issue(int L) {
     double* R = ring + (L & 1) * 3 * KS * S::NV;
-    const bool lay = L >= 0 && L < g.nz && L <= ke;
+    const bool lay = L >= 0 && L <= last;
     uint32_t fm = 0;
     auto one = [&](bool in, int node, int q, int shift) {
       in = in && lay;
@@ -207,7 +227,7 @@ __device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
 #pragma unroll
         for (int c = 0; c < 3; ++c)
           col64_cp8(R + (3 * s + c) * S::NV + q, ld.src(s) + 3 * n + c, in);
-      if (in) fm |= (uint32_t)fixed[node] << shift;
+      if (in && fixed != nullptr) fm |= (uint32_t)fixed[node] << shift;
     };
     const int base = nb0 + nxy * L, q = ey * S::NX + ex;
     one(in0, base, q, 0);
@@ -216,8 +236,9 @@ __device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
     if (re && te) one(in3, base + g.nx + 1, q + S::NX + 1, 24);
     col64_commit();
     return fm;
-  };
-  auto take = [&](int L, int q, uint32_t fm, double (&v)[3]) {
+  }
+
+  __device__ __forceinline__ void take(int L, int q, uint32_t fm, double (&v)[3]) const {
     const double* R = ring + (L & 1) * 3 * KS * S::NV + q;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -226,9 +247,11 @@ __device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
       for (int s = 0; s < KS; ++s) r[s] = R[(3 * s + c) * S::NV];
       v[c] = ((fm >> c) & 1) ? 0.0 : ld.combine(r);
     }
-  };
-  // x stage of one edge row: this thread's edge from its node and the next
-  auto edge = [&](const double (&a)[3], const double (&right)[3], double (&e)[6]) {
+  }
+
+  // x stage of one edge row: the edge from this thread's node to the next
+  __device__ __forceinline__ void edge(const double (&a)[3], const double (&right)[3],
+                                       double (&e)[6]) const {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       double b = __shfl_down_sync(0xffffffffu, a[c], 1);
@@ -236,20 +259,18 @@ __device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
       e[c] = a[c] + b;
       e[3 + c] = b - a[c];
     }
-  };
-  double eo[6];   // this column's lower-y edge of the node layer staged last
-  auto stage = [&](int L, uint32_t fm) {
+  }
+
+  // x stage of node layer L (its copies have landed); own: the thread's node
+  __device__ __forceinline__ void stage(int L, uint32_t fm, double (&own)[3]) {
     const int q = ey * S::NX + ex;
-    double own[3], right[3] = {0.0, 0.0, 0.0};
+    double right[3] = {0.0, 0.0, 0.0};
     take(L, q, fm, own);
     if (re) take(L, q + 1, fm >> 8, right);
     edge(own, right, eo);
     double* Eb = edges + (L & 1) * (CY + 1) * S::ROW + ey * S::ROW + ex;
 #pragma unroll
     for (int i = 0; i < 6; ++i) Eb[i * CX] = eo[i];
-    double* O = ownv + ((L + 3) % 3) * 3 * S::NT + tid;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) O[c * S::NT] = own[c];
     if (__any_sync(0xffffffffu, te)) {   // the tile's last edge row
       double top[3] = {0.0, 0.0, 0.0}, corner[3] = {0.0, 0.0, 0.0}, et[6];
       if (te) take(L, q + S::NX, fm >> 16, top);
@@ -260,9 +281,10 @@ __device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
         for (int i = 0; i < 6; ++i) Eb[S::ROW + i * CX] = et[i];
       }
     }
-  };
-  // y stage: face modes from this column's two edges
-  auto face = [&](int L, Col64Face& F) {
+  }
+
+  // y stage of node layer L, staged last, a barrier after its stage()
+  __device__ __forceinline__ void face(int L, Col64Face& F) const {
     const double* Eb = edges + (L & 1) * (CY + 1) * S::ROW + (ey + 1) * S::ROW + ex;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -272,6 +294,41 @@ __device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
       F.m[c][1] = eo[3 + c] + d1;
       F.m[c][3] = d1 - eo[3 + c];
     }
+  }
+};
+
+// Tile `tile` of `tl`; returns this thread's share of the epilogue reduction.
+// Iteration ez (element layer ez, between node layers ez and ez + 1) stages
+// node layer ez + 1, crosses the layer's barrier, finishes node layer ez - 1
+// and computes element layer ez.
+template <int CX, int CY, typename Load, typename Epi>
+__device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
+                                                   const uint8_t* __restrict__ fixed,
+                                                   const ModeCoef<double>& K, const Grid& g,
+                                                   const Col64Tiling& tl, int tile,
+                                                   const Load& ld, const Epi& epi, double* smem) {
+  using S = Col64Shape<CX, CY>;
+  using Stream = Col64Stream<CX, CY, Load>;
+  double* back = smem + Stream::kDoubles;              // [2][CY][6][CX], slot of layer k: k & 1
+  double* ownv = back + 2 * CY * S::ROW;               // [3][3][NT], slot of layer k: (k + 3) % 3
+  const int tid = threadIdx.x;
+  const int bx = tile % tl.tx, by = (tile / tl.tx) % tl.ty, bz = tile / (tl.tx * tl.ty);
+  const int kb = bz * tl.nzc, ke = min(kb + tl.nzc, g.nz);        // owned node layers [kb, ke)
+  Stream st(smem, ld, fixed, g, bx * S::OX - 1, by * S::OY - 1, ke);
+  const int ex = st.ex, ey = st.ey, gi = st.gi, gj = st.gj;
+  const int nexy = g.nelx * g.nely;
+  const bool elem_in = gi >= 0 && gj >= 0 && gi < g.nelx && gj < g.nely;
+  const bool own_node = ex >= 1 && ey >= 1 && st.in0;
+  const bool warp_elem = __any_sync(0xffffffffu, elem_in);
+  const bool warp_own = __any_sync(0xffffffffu, own_node);
+  double red = 0.0;
+
+  auto stage = [&](int L, uint32_t fm) {
+    double own[3];
+    st.stage(L, fm, own);
+    double* O = ownv + ((L + 3) % 3) * 3 * S::NT + tid;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) O[c * S::NT] = own[c];
   };
   double front[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};   // this column's share of its lower-y edge
   // owner's sum of node layer k: the shares of the columns at y - 1 (back
@@ -289,7 +346,7 @@ __device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
     if (own_node) {
       const double* O = ownv + ((k + 3) % 3) * 3 * S::NT + tid;
       const double pn[3] = {O[0], O[S::NT], O[2 * S::NT]};
-      epi(nb0 + nxy * k, acc, pn, (uint8_t)fm, red);
+      epi(st.nb0 + st.nxy * k, acc, pn, (uint8_t)fm, red);
     }
   };
 
@@ -300,13 +357,13 @@ __device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
 #pragma unroll
       for (int i = 0; i < 6; ++i) back[s * CY * S::ROW + ey * S::ROW + i * CX + ex] = 0.0;
   }
-  uint32_t fm_prev = 0, fm_cur = issue(kb - 1), fm_next = issue(kb);
+  uint32_t fm_prev = 0, fm_cur = st.issue(kb - 1), fm_next = st.issue(kb);
   col64_wait<1>();
   stage(kb - 1, fm_cur);
-  uint32_t fm_load = issue(kb + 1);
+  uint32_t fm_load = st.issue(kb + 1);
   __syncthreads();
   Col64Face F0, F1, U, Ms;
-  if (warp_elem) face(kb - 1, F0);
+  if (warp_elem) st.face(kb - 1, F0);
 #pragma unroll
   for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -320,11 +377,11 @@ __device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
     // into the slot it leaves
     col64_wait<1>();
     stage(ez + 1, fm_next);
-    const uint32_t fm_new = issue(ez + 3);
+    const uint32_t fm_new = st.issue(ez + 3);
     __syncthreads();
     if (ez - 1 >= kb) finish(ez - 1, fm_prev);
     if (warp_elem) {
-      face(ez + 1, Fup);
+      st.face(ez + 1, Fup);
       if (ez >= 0 && ez < g.nelz) {
         col64_element(Flo, Fup, Ee, K, U, Ms);
       } else {   // below or above the mesh: no element layer
@@ -357,4 +414,60 @@ __device__ __forceinline__ double kv_column64_body(const double* __restrict__ E,
   finish(ke - 1, fm_prev);
   col64_wait<0>();
   return red;
+}
+
+// Threads an SM holds at the kernels' launch bounds: registers for a whole
+// element in each (at most 168).
+constexpr int kCol64Threads = 384;
+
+// The tile shapes, by index, and the one (with its z-chunk) that a mesh gets.
+constexpr int kCol64Shapes = 5;
+template <typename F>
+mfto_status col64_dispatch(int i, const F& f) {
+  switch (i) {
+    case 0: return f(Col64Shape<32, 8>{});
+    case 1: return f(Col64Shape<16, 16>{});
+    case 2: return f(Col64Shape<32, 4>{});
+    case 3: return f(Col64Shape<16, 8>{});
+    default: return f(Col64Shape<8, 16>{});
+  }
+}
+
+// A CTA of NT threads over nzc layers executes (nzc + extra) layers of NT / 32
+// warps, and an SM's FP64 pipe takes its CTAs one after another, so the time is
+// that of the SM with the most CTAs: ceil(tiles / SMs) x NT x (nzc + extra), or
+// about half a CTA beyond the mean where there are more than are resident.
+// Few resident warps leave gaps: sweeps of shapes and chunks on seven meshes
+// (3,456 to 1,000,000 elements) gave 1.5 times the pipe's time with 4 warps on
+// an SM, 1.25 with 8 and 1.18 with 12, hence the factor 1.03 + 2 / warps.  Every
+// shape and every balanced chunk length is tried (host arithmetic, once per
+// handle).  halo: columns (in x and y) of a tile that it does not own; nx, ny,
+// nz: what the tiles own together; extra: the recomputed layer and about half a
+// layer of prologue and tail.
+static inline void col64_choose(int halo, int nx, int ny, int nz, double extra, int num_sms,
+                                int* shape_out, int* nzc_out) {
+  double best = 0.0;
+  for (int i = 0; i < kCol64Shapes; ++i)
+    col64_dispatch(i, [&](auto shape) -> mfto_status {
+      using S = decltype(shape);
+      const int ox = S::CX - halo, oy = S::CY - halo;
+      const int64_t txy = (int64_t)((nx + ox - 1) / ox) * ((ny + oy - 1) / oy);
+      for (int tz = 1; tz <= nz; ++tz) {
+        const int nzc = (nz + tz - 1) / tz;
+        if ((nz + nzc - 1) / nzc != tz) continue;          // not a balanced count
+        if (txy * tz > MFTO_RED_SLOTS && tz > 1) break;     // one partial per CTA
+        constexpr int resident = kCol64Threads / S::NT;
+        const double mean = (double)(txy * tz) / num_sms;
+        const int64_t ctas = (txy * tz + num_sms - 1) / num_sms;
+        const double busy = ctas > resident ? mean + 0.5 : (double)ctas;
+        const double warps = (double)(ctas > resident ? resident : ctas) * S::NT / 32;
+        const double cost = busy * S::NT * (nzc + extra) * (1.03 + 2.0 / warps);
+        if (best == 0.0 || cost < best) {
+          best = cost;
+          *shape_out = i;
+          *nzc_out = nzc;
+        }
+      }
+      return MFTO_OK;
+    });
 }

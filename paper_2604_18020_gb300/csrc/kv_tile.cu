@@ -42,11 +42,11 @@ pcg_kv_block_kernel(const float* __restrict__ E, const float* __restrict__ z,
   }
 }
 
-// FP64: column-streaming body (kv_column64.cuh), one tile per CTA.  Launch
-// bounds: 256 resident threads per SM are enough to keep the FP64 pipe busy
-// and leave each the registers of a whole element.
+// FP64: column-streaming body (kv_column64.cuh), one tile per CTA.  Held to
+// 168 registers, so that three CTAs of 128 threads share an SM (229 us at
+// 55 x 55 x 165; two, with 184 registers: 303 us).
 template <int CX, int CY>
-__global__ void __launch_bounds__(CX * CY, 256 / (CX * CY))
+__global__ void __launch_bounds__(CX * CY, kCol64Threads / (CX * CY))
 kv_col64_kernel(const double* __restrict__ E, const double* __restrict__ v,
                 double* __restrict__ y, const uint8_t* __restrict__ fixed, ModeCoef<double> K,
                 Grid g, Col64Tiling tl) {
@@ -56,7 +56,7 @@ kv_col64_kernel(const double* __restrict__ E, const double* __restrict__ v,
 }
 
 template <int CX, int CY>
-__global__ void __launch_bounds__(CX * CY, 256 / (CX * CY))
+__global__ void __launch_bounds__(CX * CY, kCol64Threads / (CX * CY))
 pcg_kv_col64_kernel(const double* __restrict__ E, const double* __restrict__ z,
                     const double* __restrict__ p_old, double* __restrict__ p_new,
                     double* __restrict__ q, const uint8_t* __restrict__ fixed,
@@ -80,48 +80,6 @@ pcg_kv_col64_kernel(const double* __restrict__ E, const double* __restrict__ z,
       s->alpha = s->rz / tot[0];
     }
   }
-}
-
-// Calls f with the tile shape of index i (mfto_handle::col64_shape).
-constexpr int kCol64Shapes = 5;
-template <typename F>
-mfto_status col64_dispatch(int i, const F& f) {
-  switch (i) {
-    case 0: return f(Col64Shape<32, 8>{});
-    case 1: return f(Col64Shape<16, 16>{});
-    case 2: return f(Col64Shape<32, 4>{});
-    case 3: return f(Col64Shape<16, 8>{});
-    default: return f(Col64Shape<8, 16>{});
-  }
-}
-
-// Tile shape and z-chunk of the FP64 kernel for a mesh.  A CTA of NT threads
-// over nzc owned node layers executes (nzc + 1) element layers of NT / 32
-// warps, and an SM's FP64 pipe takes its CTAs one after another, so the time
-// is that of the SM with the most CTAs: ceil(tiles / SMs) x NT x (nzc + 1 +
-// about half a layer of prologue and tail).  Every shape and every balanced
-// chunk length is tried (host arithmetic, once per handle).
-void col64_choose(mfto_handle* h) {
-  const Grid g = make_grid(h->mesh);
-  double best = 0.0;
-  for (int i = 0; i < kCol64Shapes; ++i)
-    col64_dispatch(i, [&](auto shape) -> mfto_status {
-      using S = decltype(shape);
-      const int64_t txy = (int64_t)((g.nx + S::OX - 1) / S::OX) * ((g.ny + S::OY - 1) / S::OY);
-      for (int tz = 1; tz <= g.nz; ++tz) {
-        const int nzc = (g.nz + tz - 1) / tz;
-        if ((g.nz + nzc - 1) / nzc != tz) continue;       // not a balanced count
-        if (txy * tz > MFTO_RED_SLOTS && tz > 1) break;    // one partial per CTA
-        const double cost = (double)((txy * tz + h->num_sms - 1) / h->num_sms) * S::NT *
-                            (nzc + 1.5);
-        if (best == 0.0 || cost < best) {
-          best = cost;
-          h->col64_shape = i;
-          h->col64_nzc = nzc;
-        }
-      }
-      return MFTO_OK;
-    });
 }
 
 template <typename S>
@@ -379,7 +337,8 @@ ColTiling col_launch_tiling(const mfto_handle* h, int per_sm, int* grid) {
 }
 
 mfto_status kv_tile_init(mfto_handle* h) {
-  col64_choose(h);
+  const Grid g = make_grid(h->mesh);
+  col64_choose(1, g.nx, g.ny, g.nz, 1.5, h->num_sms, &h->col64_shape, &h->col64_nzc);
   const mfto_status s = col64_attrs(h);
   if (s != MFTO_OK) return s;
   MFTO_CUDA(h, cudaFuncSetAttribute(kv_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
