@@ -67,8 +67,7 @@ struct MiscScalars {
   double sum[4];            // results of small reductions
   double lambda, change, volume;
   int32_t oc_steps;
-  int32_t oc_evals;         // candidate-volume evaluations (grid barriers) of the last OC
-  int32_t oc_kstar;         // its first-phase index k* (the next call's starting guess)
+  int32_t oc_evals;         // grid-wide sums of the last OC
   int32_t error;            // set by device code that gave up on a wait
   unsigned int ticket;
   unsigned int bar_count, bar_gen;
@@ -123,8 +122,7 @@ struct mfto_handle {
   double* d_filter_W;       // row sums W_e
   // PCG workspace (FP64)
   double *d_r, *d_z, *d_p0, *d_p1, *d_q, *d_dinv;
-  double* d_oc;             // [3][n_elem] OC bisection scratch (simp.cu)
-  int oc_hint;              // k* of the previous OC update (0: none), simp.cu
+  double* d_oc;             // [3][n_elem] scratch of the OC update (simp.cu) and the filter
   uint8_t* d_tile_fixed;    // column K.v xy tiles that stage a fixed node (kv_column.cuh)
   double* d_partials;       // [MFTO_RED_ROWS * MFTO_RED_SLOTS]
   double* d_partials2;      // [MFTO_RED_ROWS * MFTO_RED_SLOTS]

@@ -119,76 +119,91 @@ compliance_kernel(const double* __restrict__ rho, const double* __restrict__ u,
   }
 }
 
-// OC with bisection on lambda.  One cooperative grid of one CTA per SM.  A
-// first pass forms per element a_e = rho_e sqrt(max(0, -dc_e) n) and the
-// move-limit bounds, so that the candidate of a midpoint lambda is
-// a_e / sqrt(lambda) (the same value as rho_e sqrt(max(0, -dc_e) / (lambda / n))
-// up to rounding): each evaluation of the candidate volume is then one FP64
-// multiply and a clamp per element, on values kept in registers (G > 0: up
-// to G elements per thread) or re-read from the scratch arrays (G == 0,
-// larger meshes).  An evaluation sums the candidate field, crosses a
-// counting grid barrier (release-add of one arrival per CTA, acquire-polls
-// until every CTA has arrived; bounded), and warp 0 of every CTA adds the
-// per-CTA partials in the same order, so every CTA takes the same branch.
-// Partials are double-buffered by evaluation parity.
+// OC with bisection on lambda.  The candidate of a midpoint lambda is, per
+// element, a_e s clipped to its move limits [lo_e, hi_e], with s = 1/sqrt(lambda)
+// and a_e = rho_e sqrt(max(0, -dc_e) n) (the same value as rho_e sqrt(max(0,
+// -dc_e) / (lambda / n)) up to rounding).  Its volume is a nondecreasing,
+// piecewise linear function of s, which leaves little of the bisection's 60
+// to 80 volume evaluations to be done:
+//   1. a safeguarded Newton iteration in FP32 finds s* (where the volume is
+//      the target) to about 1e-7, on FP32 copies of a and rho;
+//   2. one FP64 pass classifies every element for all s within 1.5e-5 of that:
+//      clipped (its bound goes into a constant C), linear (its a into a slope
+//      A), or undecided (its breakpoint lies near; a few in 100,000);
+//   3. every CTA then holds volume(s) = C + A s + sum over the undecided for
+//      that window of s, in the same order of sums.  It confirms that the
+//      volume crosses the target within the window, narrows the window by
+//      Newton steps, and replays the bisection from [0, 1e9]: midpoints outside
+//      the window are decided by monotonicity, those inside by evaluation.
+// The replay takes the branches that the step by step bisection takes, so its
+// lambda and its last midpoint are the same.  A target below the sum of the
+// lower bounds, or above all that can be reached, decides every midpoint at
+// once.  Where the crossing is not confirmed (a volume that is flat there,
+// values beyond FP32's range, more undecided elements than the lists hold) the
+// bisection evaluates every midpoint over all elements.
 //
-// The bisection starts from [0, 1e9].  While its lower end is still 0, its
-// midpoints are lambda_k = 1e9 / 2^k (k = 1, 2, ...: each the previous one
-// halved, so exact down to the subnormal range), and it moves the upper end
-// down until the first k* whose candidate volume exceeds the target.  That
-// volume is nondecreasing in k (every step of its evaluation is monotone:
-// rounded products, clamps and fixed-order rounded sums), so k* is found by
-// a binary search over k, started at the previous call's k* (a hint that
-// leaves the result unchanged and normally settles it in two evaluations),
-// and the bisection then continues from exactly the state it would have
-// reached step by step.  The candidate of the last midpoint is written by a
-// final pass.
+// One cooperative grid; a grid barrier counts arrivals (release-add of one per
+// CTA, acquire-polls; bounded), and every CTA adds the per-CTA partials in the
+// same order, so that all take the same branches.  Bound by the FP64 pipe in
+// the first pass (a_e: about 30 operations) and by about ten grid barriers of
+// 2 to 3 us.  Measured on a GB300: 41 against 265 us at
+// 216,000 elements (a bisection of about 37 full evaluations), 325 against
+// 1,917 us at 4,915,200.
+constexpr int kOcThreads = 512;
+constexpr int kOcSeg = 64;        // undecided elements a CTA may list
+constexpr int kOcMine = 4;        // ... and a thread
+constexpr int kOcList = 1024;     // ... and the grid
+constexpr float kOcMargin = 3e-5f;
+constexpr double kOcWindow = 1.5e-5;
+
+struct OcElem {                   // an undecided element
+  double a, lo, hi;
+};
+
+struct OcUp {                     // the bisection whose every midpoint exceeds the target
+  double l1, l2, last;
+  int step;
+};
+
 template <int G>
-__global__ void __launch_bounds__(MFTO_BLOCK)
+__global__ void __launch_bounds__(kOcThreads, G > 0 ? 1 : 2)
 oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
-          double* __restrict__ rho_new, double* __restrict__ a_s, double* __restrict__ lo_s,
-          double* __restrict__ hi_s, int n, double volfrac, double move, MiscScalars* s,
-          double* partials, int k_end, int k_hint) {
+          double* __restrict__ rho_new, double* __restrict__ a_s, float2* __restrict__ f_s, int n,
+          double volfrac, double move, MiscScalars* s, double* partials, OcElem* list, int* counts,
+          int k_end, OcUp up) {
   __shared__ double sh[64];
+  __shared__ double s_tot[3];
+  __shared__ float s_f[3];
+  __shared__ int s_cnt, s_warp[32];
+  __shared__ OcElem s_list[kOcList];
   const double target = volfrac * (double)n;
   const int first = blockIdx.x * blockDim.x + threadIdx.x;
   const int stride = gridDim.x * blockDim.x;
-  double ra[G > 0 ? G : 1], rlo[G > 0 ? G : 1], rhi[G > 0 ? G : 1];
-  if constexpr (G > 0) {
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const int e = first + g * stride;
-      ra[g] = 0.0;
-      rlo[g] = 0.0;
-      rhi[g] = 0.0;
-      if (e < n) {
-        const double r = rho[e];
-        ra[g] = r * sqrt(fmax(0.0, -dc[e]) * (double)n);
-        rlo[g] = fmax(0.0, r - move);
-        rhi[g] = fmin(1.0, r + move);
-      }
-    }
-  } else {
-    for (int e = first; e < n; e += stride) {
-      const double r = rho[e];
-      a_s[e] = r * sqrt(fmax(0.0, -dc[e]) * (double)n);
-      lo_s[e] = fmax(0.0, r - move);
-      hi_s[e] = fmin(1.0, r + move);
-    }
-  }
-  // the candidate sum at the scale sc = 1 / sqrt(lambda)
-  auto volume = [&](double sc) {
-    double acc = 0.0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float movef = (float)move;
+  // per element a (FP64) and (a, rho) in FP32: in registers (G > 0: up to G
+  // elements per thread) or in scratch arrays (G == 0, larger meshes)
+  double ra[G > 0 ? G : 1];
+  float2 rf[G > 0 ? G : 1];
+  auto each = [&](auto&& f) {     // f(element, a, (a, rho) in FP32)
     if constexpr (G > 0) {
 #pragma unroll
       for (int g = 0; g < G; ++g)
-        if (first + g * stride < n) acc += fmax(rlo[g], fmin(rhi[g], ra[g] * sc));
+        if (first + g * stride < n) f(first + g * stride, ra[g], rf[g]);
     } else {
-      for (int e = first; e < n; e += stride) acc += fmax(lo_s[e], fmin(hi_s[e], a_s[e] * sc));
+      for (int e = first; e < n; e += stride) f(e, a_s[e], f_s[e]);
     }
-    return acc;
   };
-  unsigned int arrivals = 0;   // grid-barrier arrivals expected so far
+  auto each32 = [&](auto&& f) {   // f((a, rho) in FP32)
+    if constexpr (G > 0) {
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+        if (first + g * stride < n) f(rf[g]);
+    } else {
+      for (int e = first; e < n; e += stride) f(f_s[e]);
+    }
+  };
+  unsigned int arrivals = 0;      // grid-barrier arrivals expected so far
   auto grid_sync = [&]() {
     arrivals += gridDim.x;
     __syncthreads();
@@ -203,28 +218,118 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
     }
     __syncthreads();
   };
-  // 1 / sqrt(lambda) of each evaluation: formed once per CTA (the FP64 pipe
-  // runs 2 operations per clock per SM) and handed over in shared memory
-  __shared__ double s_sc, s_tot;
+  auto failed = [&]() { return *(volatile int32_t*)&s->error != 0; };
+  // grid totals of three block sums (valid in thread 0), identical in every
+  // thread: s_tot, and s_f in FP32 (s_f[0] less the target); partials
+  // double-buffered by parity, one grid barrier
   int evals = 0;
-  // the candidate volume at lambda, identical in every CTA
-  auto eval_total = [&](double lam) {
-    double* buf = partials + (evals & 1) * MFTO_RED_SLOTS;
+  auto totals = [&](double b0, double b1, double b2) {
+    double* buf = partials + (evals & 1) * 3 * MFTO_RED_SLOTS;
     ++evals;
-    if (threadIdx.x == 0) s_sc = 1.0 / sqrt(lam);
-    __syncthreads();
-    const double bs = block_sum(volume(s_sc), sh);
-    if (threadIdx.x == 0) buf[blockIdx.x] = bs;
+    if (threadIdx.x == 0) {
+      buf[blockIdx.x] = b0;
+      buf[MFTO_RED_SLOTS + blockIdx.x] = b1;
+      buf[2 * MFTO_RED_SLOTS + blockIdx.x] = b2;
+    }
     grid_sync();
-    if (threadIdx.x < 32) {
+    if (warp < 3) {
       double t = 0.0;
-      for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) t += __ldcg(&buf[b]);
+      for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(&buf[warp * MFTO_RED_SLOTS + b]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-      if (threadIdx.x == 0) s_tot = t;
+      if (lane == 0) {
+        s_tot[warp] = t;
+        s_f[warp] = (float)(warp == 0 ? t - target : t);
+      }
     }
     __syncthreads();
-    return s_tot;
+  };
+  // block sums of FP32 thread sums: warps in FP32, then one conversion each
+  auto block_f32 = [&](float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return block_sum_w0(lane == 0 ? (double)v : 0.0, sh);
+  };
+
+  // ---- a_e; sums of the lower bounds, of what each element can reach and of a
+  float sum_lo = 0.f, sum_hi = 0.f, sum_a = 0.f;
+  auto init = [&](int e, double& a, float2& f) {
+    const double r = rho[e];
+    a = r * sqrt(fmax(0.0, -dc[e]) * (double)n);
+    f = make_float2((float)a, (float)r);
+    const float lo = fmaxf(0.f, f.y - movef);
+    sum_lo += lo;
+    sum_hi += a > 0.0 ? fminf(1.f, f.y + movef) : lo;
+    sum_a += f.x;
+  };
+  if constexpr (G > 0) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      ra[g] = 0.0;
+      rf[g] = make_float2(0.f, 0.f);
+      if (first + g * stride < n) init(first + g * stride, ra[g], rf[g]);
+    }
+  } else {
+    for (int e = first; e < n; e += stride) {
+      double a;
+      float2 f;
+      init(e, a, f);
+      a_s[e] = a;
+      f_s[e] = f;
+    }
+  }
+  {
+    const double b0 = block_f32(sum_lo), b1 = block_f32(sum_hi);
+    totals(b0, b1, block_f32(sum_a));
+  }
+  // the volume exceeds the target at every midpoint, or at none (the FP32
+  // sums are good to far better than 1e-5)
+  const bool always = s_tot[0] * (1.0 - 1e-5) > target && move >= 0.0;
+  const bool never = s_tot[1] * (1.0 + 1e-5) < target && move >= 0.0;
+
+  // ---- 1. Newton in FP32, kept between the scales known to give too little
+  // (slo) and too much volume (shi); uniform over the grid
+  float sf = (float)target / s_f[2], slo = 0.f, shi = INFINITY;
+  bool found = false;
+  if (!always && !never && s_f[2] < INFINITY && sf > 1e-30f && sf < 1e30f) {
+    for (int it = 0; it < 24 && !failed(); ++it) {
+      float vol = 0.f, slope = 0.f;
+      each32([&](float2 f) {
+        const float t = f.x * sf;
+        const float lo = fmaxf(0.f, f.y - movef), hi = fminf(1.f, f.y + movef);
+        vol += fmaxf(lo, fminf(hi, t));
+        if (t > lo && t < hi) slope += f.x;
+      });
+      const double bv = block_f32(vol);
+      totals(bv, block_f32(slope), 0.0);
+      const float miss = s_f[0], A = s_f[1];
+      if (miss > 0.f) shi = sf; else slo = sf;
+      if (A > 0.f && fabsf(miss) <= 2e-6f * A * sf) { found = true; break; }
+      float next = A > 0.f ? sf - miss / A : -1.f;
+      if (!(next > slo && next < shi))    // outside what is known: halve in the logarithm
+        next = shi == INFINITY ? 4.f * sf : (slo > 0.f ? sqrtf(slo) * sqrtf(shi) : 0.25f * sf);
+      if (!(next > 1e-30f && next < 1e30f)) break;
+      sf = next;
+    }
+  }
+
+  // the bisection's state: bracket, last midpoint, its volume, steps
+  double l1 = 0.0, l2 = 1e9, total = 0.0, last = -1.0;
+  int step = 0;
+  bool done = false;
+  // the candidate volume at lambda over all elements
+  auto eval_total = [&](double lam) {
+    if (threadIdx.x == 0) sh[40] = 1.0 / sqrt(lam);
+    __syncthreads();
+    const double sc = sh[40];
+    double acc = 0.0;
+    each([&](int e, double a, float2) {
+      const double r = rho[e];
+      acc += fmax(fmax(0.0, r - move), fmin(fmin(1.0, r + move), a * sc));
+    });
+    __syncthreads();
+    totals(block_sum(acc, sh), 0.0, 0.0);
+    return s_tot[0];
   };
   // lambda_k = 1e9 halved k times (0 <= k <= k_end; exact for k <= 1083)
   auto lam_of = [](int k) {
@@ -233,71 +338,250 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
     for (int i = 1083; i < k; ++i) x = 0.5 * x;
     return x;
   };
-  const double target_v = target;
-  double l1 = 0.0, l2 = 1e9, total = 0.0, last = -1.0;
-  int step = 0, kstar = 0;
-  // the phase with lower end 0: k* = the first k in [1, k_end) whose volume
-  // exceeds the target (k_end: the first k with lambda_k = 0, where the
-  // step-by-step bisection stops); klo: volume known <= target (0: none
-  // evaluated), khi: volume known > target (k_end: none found yet)
-  if (k_end > 1) {
-    int klo = 0, khi = k_end;
-    double vlo = 0.0, vhi = 0.0;
-    auto probe = [&](int k) {
-      const double v = eval_total(lam_of(k));
-      if (v > target_v) { khi = k; vhi = v; } else { klo = k; vlo = v; }
-    };
-    if (k_hint >= 1 && k_hint < k_end) {
-      probe(k_hint);
-      if (khi == k_hint && k_hint - 1 >= 1) probe(k_hint - 1);
-      else if (klo == k_hint && k_hint + 1 < k_end) probe(k_hint + 1);
-    }
-    if (klo != k_end - 1 && khi == k_end) probe(k_end - 1);   // is there a k* at all?
-    while (khi - klo > 1 && !*(volatile int32_t*)&s->error) probe((klo + khi) / 2);
-    kstar = khi;
-    if (khi < k_end) {
-      l1 = lam_of(khi);
-      l2 = lam_of(khi - 1);
-      last = l1;
-      total = vhi;
-      step = khi;
-    } else {
-      l2 = lam_of(k_end - 1);
-      last = l2;
-      total = vlo;
-      step = k_end - 1;
-    }
+
+  if (always) {
+    l1 = up.l1;
+    l2 = up.l2;
+    last = up.last;
+    step = up.step;
+    total = eval_total(last);
+    done = true;
+  } else if (never && k_end > 1) {
+    // only the upper end ever moves, down to the last midpoint above 0
+    l2 = lam_of(k_end - 1);
+    last = l2;
+    step = k_end - 1;
+    total = eval_total(last);
+    done = true;
   }
-  // Stops at the relative bracket width 1e-10, or when the midpoint no
-  // longer lies strictly inside the bracket (lambda underflow when the target
-  // is unreachable from above), and after at most 4096 steps in any case.
-  while (l1 + l2 > 0.0 && (l2 - l1) / (l1 + l2) > 1e-10 && step < 4096) {
-    const double lmid = 0.5 * (l1 + l2);
-    if (!(l1 < lmid && lmid < l2)) break;   // uniform: every block holds the same l1, l2
-    total = eval_total(lmid);
-    last = lmid;
-    if (total > target) l1 = lmid; else l2 = lmid;
-    ++step;
-    if (*(volatile int32_t*)&s->error) break;
+
+  if (found) {
+    // ---- 2. classification for s in sf (1 -+ kOcWindow)
+    double cacc = 0.0, aacc = 0.0;
+    int mine = 0;
+    OcElem und[kOcMine];
+    each([&](int e, double a, float2 f) {
+      const float t = f.x * sf;
+      const float lo = fmaxf(0.f, f.y - movef), hi = fminf(1.f, f.y + movef);
+      if (t * (1.f + kOcMargin) < lo || a == 0.0) {
+        cacc += fmax(0.0, rho[e] - move);
+      } else if (t * (1.f - kOcMargin) > hi) {
+        cacc += fmin(1.0, rho[e] + move);
+      } else if (t * (1.f - kOcMargin) > lo && t * (1.f + kOcMargin) < hi && t > 1e-30f) {
+        aacc += a;
+      } else {
+        const double r = rho[e];
+        const OcElem u{a, fmax(0.0, r - move), fmin(1.0, r + move)};
+#pragma unroll
+        for (int i = 0; i < kOcMine; ++i)
+          if (i == mine) und[i] = u;
+        ++mine;
+      }
+    });
+    // the CTA's undecided elements, in thread order, into its list segment
+    int before = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, before, o);
+      if (lane >= o) before += v;
+    }
+    if (lane == 31) s_warp[warp] = before;
+    before -= mine;
+    int over = __syncthreads_or(mine > kOcMine);
+    if (threadIdx.x == 0) {
+      int t = 0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        const int c = s_warp[w];
+        s_warp[w] = t;
+        t += c;
+      }
+      s_cnt = t;
+    }
+    __syncthreads();
+    before += s_warp[warp];
+    if (s_cnt > kOcSeg) over = 1;
+    if (!over) {
+#pragma unroll
+      for (int i = 0; i < kOcMine; ++i)
+        if (i < mine) list[(size_t)blockIdx.x * kOcSeg + before + i] = und[i];
+    }
+    if (threadIdx.x == 0) counts[blockIdx.x] = over ? -1 : s_cnt;
+    const double bc = block_sum(cacc, sh);
+    totals(bc, block_sum(aacc, sh), 0.0);
+    const double C = s_tot[0], A = s_tot[1];
+    // every CTA's undecided elements, in CTA order, into shared memory
+    int have = 0, from = 0;
+    if (threadIdx.x < gridDim.x) have = __ldcg(&counts[threadIdx.x]);
+    over = __syncthreads_or(have < 0 || gridDim.x > blockDim.x);
+    int upto = have;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, upto, o);
+      if (lane >= o) upto += v;
+    }
+    if (lane == 31) s_warp[warp] = upto;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) from += s_warp[w];
+    from += upto - have;
+    over = __syncthreads_or(from + have > kOcList) || over;
+    if (!over) {
+      for (int i = 0; i < have; ++i) {
+        const double* p = &list[(size_t)threadIdx.x * kOcSeg + i].a;
+        s_list[from + i] = OcElem{__ldcg(p), __ldcg(p + 1), __ldcg(p + 2)};
+      }
+      if (threadIdx.x == blockDim.x - 1) s_cnt = from + have;
+    }
+    __syncthreads();
+
+    // ---- 3. the window, by warp 0 of every CTA alike
+    if (!over && warp == 0) {
+      const int nu = s_cnt;
+      double und_a = 0.0;   // slope of the undecided at the last evaluation
+      auto volume = [&](double sc) {
+        double v = 0.0, sl = 0.0;
+        for (int i = lane; i < nu; i += 32) {
+          const OcElem u = s_list[i];
+          const double t = u.a * sc;
+          v += fmax(u.lo, fmin(u.hi, t));
+          if (t > u.lo && t < u.hi) sl += u.a;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          v += __shfl_xor_sync(0xffffffffu, v, o);
+          sl += __shfl_xor_sync(0xffffffffu, sl, o);
+        }
+        und_a = sl;
+        return fma(A, sc, C) + v;
+      };
+      double wl = (double)sf * (1.0 - kOcWindow), wh = (double)sf * (1.0 + kOcWindow);
+      if (volume(wl) <= target && volume(wh) > target) {
+        // Newton steps towards the crossing, then a window of 2e-12 around it
+        double sc = (double)sf;
+        for (int it = 0; it < 6; ++it) {
+          const double v = volume(sc);
+          if (v > target) wh = fmin(wh, sc); else wl = fmax(wl, sc);
+          const double slope = A + und_a;
+          const double next = slope > 0.0 ? sc + (target - v) / slope : sc;
+          if (!(next > wl && next < wh) || fabs(next - sc) <= 1e-15 * sc) break;
+          sc = next;
+        }
+        const double nl = sc * (1.0 - 1e-12), nh = sc * (1.0 + 1e-12);
+        if (nl > wl && nl < wh && volume(nl) <= target) wl = nl;
+        if (nh > wl && nh < wh && volume(nh) > target) wh = nh;
+        // midpoints lambda below lam_h give too much volume, above lam_l not
+        // (a margin of a few roundings: those between are evaluated)
+        const double lam_l = 1.0 / (wl * wl) * (1.0 + 1e-15), lam_h = 1.0 / (wh * wh) * (1.0 - 1e-15);
+        // (compared as integers where both are positive: the FP64 pipe is the
+        // slow part of this serial chain)
+        auto less = [](double a, double b) {
+          return __double_as_longlong(a) < __double_as_longlong(b);
+        };
+        // while the lower end is 0 the midpoints are 1e9 halved k times: go
+        // straight to the last but one before the first that may exceed
+        const int k0 = ilogb(1e9 / lam_l) - 2;
+        if (k0 >= 1 && k0 < 1000) {
+          l2 = lam_of(k0);
+          last = l2;
+          step = k0;
+        }
+        bool known = false;
+        int fine = 0;
+        while (step < 4096) {
+          const double sum = l1 + l2;
+          // with the bracket at [l, 2 l] first, its relative width cannot have
+          // fallen to 1e-10 before 29 more halvings
+          if (!(sum > 0.0) || (l1 > 0.0 && ++fine > 29 && !((l2 - l1) / sum > 1e-10))) break;
+          const double lmid = 0.5 * sum;
+          if (!less(l1, lmid) || !less(lmid, l2)) break;
+          last = lmid;
+          known = !less(lmid, lam_h) && !less(lam_l, lmid);
+          bool above = less(lmid, lam_h);
+          if (known) {
+            total = volume(1.0 / sqrt(lmid));
+            above = total > target;
+          }
+          if (above) l1 = lmid; else l2 = lmid;
+          ++step;
+        }
+        if (last > 0.0 && !known) total = volume(1.0 / sqrt(last));
+        done = true;
+      }
+      if (lane == 0) {
+        sh[0] = l1;
+        sh[1] = l2;
+        sh[2] = total;
+        sh[3] = last;
+        s_cnt = done ? step : -1;
+      }
+    }
+    __syncthreads();
+    done = !over && s_cnt >= 0;
+    if (done) {
+      l1 = sh[0];
+      l2 = sh[1];
+      total = sh[2];
+      last = sh[3];
+      step = s_cnt;
+    }
+    __syncthreads();
+  }
+
+  if (!done) {
+    // every midpoint over all elements
+    // the phase with lower end 0: midpoints lambda_k, up to the first k in
+    // [1, k_end) whose volume exceeds the target, found by a binary search over
+    // k (the volume is nondecreasing in k; k_end: the first k with lambda_k =
+    // 0, where the step-by-step bisection stops); klo: volume known <= target
+    // (0: none evaluated), khi: volume known > target (k_end: none found yet)
+    if (k_end > 1) {
+      int klo = 0, khi = k_end;
+      double vlo = 0.0, vhi = 0.0;
+      auto probe = [&](int k) {
+        const double v = eval_total(lam_of(k));
+        if (v > target) { khi = k; vhi = v; } else { klo = k; vlo = v; }
+      };
+      probe(k_end - 1);   // is there such a k at all?
+      while (khi - klo > 1 && !failed()) probe((klo + khi) / 2);
+      if (khi < k_end) {
+        l1 = lam_of(khi);
+        l2 = lam_of(khi - 1);
+        last = l1;
+        total = vhi;
+        step = khi;
+      } else {
+        l2 = lam_of(k_end - 1);
+        last = l2;
+        total = vlo;
+        step = k_end - 1;
+      }
+    }
+    // Stops at the relative bracket width 1e-10, or when the midpoint no
+    // longer lies strictly inside the bracket (lambda underflow when the target
+    // is unreachable from above), and after at most 4096 steps in any case.
+    while (l1 + l2 > 0.0 && (l2 - l1) / (l1 + l2) > 1e-10 && step < 4096) {
+      const double lmid = 0.5 * (l1 + l2);
+      if (!(l1 < lmid && lmid < l2)) break;   // uniform: every block holds the same l1, l2
+      total = eval_total(lmid);
+      last = lmid;
+      if (total > target) l1 = lmid; else l2 = lmid;
+      ++step;
+      if (failed()) break;
+    }
   }
   // the candidate of the last midpoint (rho itself if no step ran), and
   // change = max |rho_new - rho|
-  const double sc = last > 0.0 ? 1.0 / sqrt(last) : 0.0;
+  if (threadIdx.x == 0) sh[40] = last > 0.0 ? 1.0 / sqrt(last) : 0.0;
+  __syncthreads();
+  const double sc = sh[40];
   double mx = 0.0;
-  auto write = [&](int e, double a, double lo, double hi) {
+  each([&](int e, double a, float2) {
     const double r = rho[e];
-    const double rn = last > 0.0 ? fmax(lo, fmin(hi, a * sc)) : r;
+    const double rn =
+        last > 0.0 ? fmax(fmax(0.0, r - move), fmin(fmin(1.0, r + move), a * sc)) : r;
     rho_new[e] = rn;
     mx = fmax(mx, fabs(rn - r));
-  };
-  if constexpr (G > 0) {
-#pragma unroll
-    for (int g = 0; g < G; ++g)
-      if (first + g * stride < n) write(first + g * stride, ra[g], rlo[g], rhi[g]);
-  } else {
-    for (int e = first; e < n; e += stride) write(e, a_s[e], lo_s[e], hi_s[e]);
-  }
-  double* buf = partials + 2 * MFTO_RED_SLOTS;
+  });
+  double* buf = partials + 6 * MFTO_RED_SLOTS;
   const double bm = block_max(mx, sh);
   if (threadIdx.x == 0) buf[blockIdx.x] = bm;
   grid_sync();
@@ -311,7 +595,6 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
       s->lambda = 0.5 * (l1 + l2);
       s->oc_steps = step;
       s->oc_evals = evals;
-      s->oc_kstar = kstar;
     }
   }
 }
@@ -367,20 +650,24 @@ mfto_status simp_init(mfto_handle* h) {
 
 mfto_status oc_launch(mfto_handle* h, const double* rho, const double* dc, double* rho_new,
                       mfto_iter_stats* st) {
-  // one CTA per SM (co-resident: the kernels use far fewer registers and no
-  // dynamic shared memory); elements in registers when they fit
+  // one CTA per SM with its elements in registers where they fit, two (and
+  // scratch arrays) on larger meshes; co-resident (cooperative launch)
   int blocks = h->num_sms;
-  const int need = (int)((h->n_elem + MFTO_BLOCK - 1) / MFTO_BLOCK);
-  const bool regs = h->n_elem <= (int64_t)blocks * MFTO_BLOCK * kOcRegs;
+  const int need = (int)((h->n_elem + kOcThreads - 1) / kOcThreads);
+  const bool regs = h->n_elem <= (int64_t)blocks * kOcThreads * kOcRegs;
   if (!regs) {
-    // larger meshes re-read the scratch arrays every step: more CTAs in flight
     int per_sm = 0;
     MFTO_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, oc_kernel<0>,
-                                                               MFTO_BLOCK, 0));
-    blocks = (per_sm < 4 ? (per_sm < 1 ? 1 : per_sm) : 4) * h->num_sms;
+                                                               kOcThreads, 0));
+    blocks = (per_sm < 2 ? (per_sm < 1 ? 1 : per_sm) : 2) * h->num_sms;
   }
   if (blocks > need) blocks = need;
   if (blocks < 1) blocks = 1;
+  // partial rows 0 .. 6, the list segments and counts behind them
+  static_assert(sizeof(OcElem) == 3 * sizeof(double), "list entries are three doubles");
+  const int64_t list_doubles = (int64_t)blocks * (3 * kOcSeg + 1);
+  if (list_doubles > (int64_t)(MFTO_RED_ROWS - 7) * MFTO_RED_SLOTS)
+    return mfto_fail(h, MFTO_UNSUPPORTED, "OC: more CTAs than the list segments hold");
   MFTO_CUDA(h, cudaMemsetAsync(&h->d_misc->error, 0, sizeof(int32_t), h->stream));
   MFTO_CUDA(h, cudaMemsetAsync(&h->d_misc->bar_count, 0, sizeof(unsigned int), h->stream));
   int n = (int)h->n_elem;
@@ -388,8 +675,9 @@ mfto_status oc_launch(mfto_handle* h, const double* rho, const double* dc, doubl
   MiscScalars* s = h->d_misc;
   double* partials = h->d_partials2;
   double* a_s = h->d_oc;
-  double* lo_s = h->d_oc + h->n_elem;
-  double* hi_s = h->d_oc + 2 * h->n_elem;
+  float2* f_s = reinterpret_cast<float2*>(h->d_oc + h->n_elem);
+  OcElem* list = reinterpret_cast<OcElem*>(partials + 7 * MFTO_RED_SLOTS);
+  int* counts = reinterpret_cast<int*>(list + (size_t)blocks * kOcSeg);
   // k_end: the first k at which 1e9 halved k times is 0 (the bisection's
   // midpoint with lower end 0 no longer lies inside its bracket)
   static const int k_end = [] {
@@ -401,18 +689,26 @@ mfto_status oc_launch(mfto_handle* h, const double* rho, const double* dc, doubl
     }
     return k;
   }();
-  int k_hint = h->oc_hint;
-  void* args[] = {(void*)&rho, (void*)&dc, (void*)&rho_new, &a_s, &lo_s, &hi_s, &n, &volfrac,
-                  &move, &s, &partials, (void*)&k_end, &k_hint};
+  static const OcUp up = [] {
+    OcUp u{0.0, 1e9, -1.0, 0};
+    while (u.l1 + u.l2 > 0.0 && (u.l2 - u.l1) / (u.l1 + u.l2) > 1e-10 && u.step < 4096) {
+      const double lmid = 0.5 * (u.l1 + u.l2);
+      if (!(u.l1 < lmid && lmid < u.l2)) break;
+      u.last = u.l1 = lmid;
+      ++u.step;
+    }
+    return u;
+  }();
+  void* args[] = {(void*)&rho, (void*)&dc, (void*)&rho_new, &a_s, &f_s, &n, &volfrac, &move, &s,
+                  &partials, &list, &counts, (void*)&k_end, (void*)&up};
   h->launches++;
   const void* fn = regs ? (const void*)oc_kernel<kOcRegs> : (const void*)oc_kernel<0>;
-  MFTO_CUDA(h, cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(MFTO_BLOCK), args, 0, h->stream));
+  MFTO_CUDA(h, cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kOcThreads), args, 0, h->stream));
   MFTO_CUDA(h, cudaMemcpyAsync(h->h_misc, h->d_misc, sizeof(MiscScalars), cudaMemcpyDeviceToHost,
                                h->stream));
   MFTO_CUDA(h, cudaStreamSynchronize(h->stream));
   if (h->h_misc->error)
     return mfto_fail(h, MFTO_CUDA_ERROR, "OC: a grid barrier wait gave up (bounded spin)");
-  h->oc_hint = (h->h_misc->oc_kstar >= 1 && h->h_misc->oc_kstar < k_end) ? h->h_misc->oc_kstar : 0;
   if (st) {
     st->change = h->h_misc->change;
     st->volume = h->h_misc->volume;
