@@ -112,7 +112,7 @@ struct mfto_handle {
   int tcol_nzc;             // node layers per z-chunk of the tensor-core column kernel (0: automatic)
   unsigned int* d_bar;      // tree grid-barrier counters of the persistent CG (zeroed)
   int occ_tc[12];           // ... of the tensor-core kernels, [2 * (2 kind + split) + pcg]
-  int occ_multi[3];         // ... of the multi-RHS kernels (F64 K.V, F32 K.V, F32 CG step)
+  int occ_multi;            // ... of the FP32 multi-RHS block CG step
   unsigned char* d_btc;     // tensor-core B operands: [kind][hi | lo]
   uint8_t* d_fixed;         // per-node mask
   // cone filter
@@ -673,6 +673,9 @@ mfto_status kv_tile_init(mfto_handle* h);
 mfto_status simp_init(mfto_handle* h);
 template <typename T>
 mfto_status kv_tile_launch(mfto_handle* h, const T* E, const T* v, T* y, cudaStream_t st);
+template <typename T>
+mfto_status kv_multi_col_launch(mfto_handle* h, const T* E, const T* V, T* Y, int nrhs,
+                                cudaStream_t st);
 template <typename T>
 mfto_status pcg_kv_tile_launch(mfto_handle* h, const T* E, const T* z, const T* p_old, T* p_new,
                                T* q, PcgScalars* s, double* partials, cudaStream_t st);

@@ -443,9 +443,9 @@ mfto_status col64_dispatch(int i, const F& f) {
 // shape and every balanced chunk length is tried (host arithmetic, once per
 // handle).  halo: columns (in x and y) of a tile that it does not own; nx, ny,
 // nz: what the tiles own together; extra: the recomputed layer and about half a
-// layer of prologue and tail.
+// layer of prologue and tail; copies: launches' worth of tiles in one grid.
 static inline void col64_choose(int halo, int nx, int ny, int nz, double extra, int num_sms,
-                                int* shape_out, int* nzc_out) {
+                                int* shape_out, int* nzc_out, int copies = 1) {
   double best = 0.0;
   for (int i = 0; i < kCol64Shapes; ++i)
     col64_dispatch(i, [&](auto shape) -> mfto_status {
@@ -457,8 +457,8 @@ static inline void col64_choose(int halo, int nx, int ny, int nz, double extra, 
         if ((nz + nzc - 1) / nzc != tz) continue;          // not a balanced count
         if (txy * tz > MFTO_RED_SLOTS && tz > 1) break;     // one partial per CTA
         constexpr int resident = kCol64Threads / S::NT;
-        const double mean = (double)(txy * tz) / num_sms;
-        const int64_t ctas = (txy * tz + num_sms - 1) / num_sms;
+        const double mean = (double)(txy * tz * copies) / num_sms;
+        const int64_t ctas = (txy * tz * copies + num_sms - 1) / num_sms;
         const double busy = ctas > resident ? mean + 0.5 : (double)ctas;
         const double warps = (double)(ctas > resident ? resident : ctas) * S::NT / 32;
         const double cost = busy * S::NT * (nzc + extra) * (1.03 + 2.0 / warps);

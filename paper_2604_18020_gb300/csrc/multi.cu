@@ -107,24 +107,6 @@ __device__ __forceinline__ void kv_block_multi(const T* __restrict__ E,
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(MFTO_BLOCK)
-kv_multi_kernel(const T* __restrict__ E, const T* __restrict__ V, T* __restrict__ Y,
-                const uint8_t* __restrict__ fixed, ModeCoef<T> K, Grid g, int nrhs, int n_dof) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  DotAcc<T> red[MFTO_MAX_RHS];
-  auto ld = [&](int r, int i) { return V[(size_t)r * n_dof + i]; };
-  auto epi = [&](int r, int node, const T (&acc)[3], const T (&pn)[3], uint8_t fm, DotAcc<T>&) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const size_t i = (size_t)r * n_dof + 3 * node + c;
-      Y[i] = ((fm >> c) & 1) ? V[i] : acc[c];
-    }
-  };
-  kv_block_multi<T>(E, fixed, K, g, nrhs, ld, epi, [](int) { return true; },
-                    reinterpret_cast<T*>(smem_raw), red);
-}
-
 // CG step A for every active case: p_new = z + beta p_old, q = K p_new, p.q
 __global__ void __launch_bounds__(MFTO_BLOCK)
 pcg_kv_multi(const float* __restrict__ E, const float* __restrict__ Z, const float* __restrict__ P0,
@@ -446,24 +428,11 @@ static unsigned multi_grid(const mfto_handle* h, int per_sm) {
 }
 
 mfto_status multi_init(mfto_handle* h) {
-  MFTO_CUDA(h, cudaFuncSetAttribute(kv_multi_kernel<double>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)block_smem(8)));
-  MFTO_CUDA(h, cudaFuncSetAttribute(kv_multi_kernel<float>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)block_smem(4)));
   MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_multi, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)block_smem(4)));
-  MFTO_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h->occ_multi[0],
-                                                             kv_multi_kernel<double>, MFTO_BLOCK,
-                                                             block_smem(8)));
-  MFTO_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h->occ_multi[1],
-                                                             kv_multi_kernel<float>, MFTO_BLOCK,
-                                                             block_smem(4)));
-  MFTO_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h->occ_multi[2], pcg_kv_multi,
+  MFTO_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h->occ_multi, pcg_kv_multi,
                                                              MFTO_BLOCK, block_smem(4)));
-  for (int i = 0; i < 3; ++i)
-    if (h->occ_multi[i] < 1) h->occ_multi[i] = 1;
+  if (h->occ_multi < 1) h->occ_multi = 1;
   MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_multi_col<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)kColSmem));
   MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_multi_col<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -473,21 +442,14 @@ mfto_status multi_init(mfto_handle* h) {
 
 static mfto_status kv_multi_launch(mfto_handle* h, mfto_form form, const void* E, const void* V,
                                    void* Y, int nrhs) {
-  const Grid g = make_grid(h->mesh);
-  h->launches++;
-  if (form == MFTO_FORM_F64) {
-    kv_multi_kernel<double><<<multi_grid(h, h->occ_multi[0]), MFTO_BLOCK, block_smem(8),
-                              h->stream>>>((const double*)E, (const double*)V, (double*)Y,
-                                           h->d_fixed, h->mc64, g, nrhs, (int)h->n_dof);
-  } else if (form == MFTO_FORM_F32) {
-    kv_multi_kernel<float><<<multi_grid(h, h->occ_multi[1]), MFTO_BLOCK, block_smem(4),
-                             h->stream>>>((const float*)E, (const float*)V, (float*)Y,
-                                          h->d_fixed, h->mc32, g, nrhs, (int)h->n_dof);
-  } else {
+  if (form != MFTO_FORM_F64 && form != MFTO_FORM_F32)
     return mfto_fail(h, MFTO_UNSUPPORTED, "mfto_kv_multi: forms F64 and F32 only");
-  }
-  MFTO_LAUNCH_CHECK(h);
-  return MFTO_OK;
+  h->launches++;
+  return form == MFTO_FORM_F64
+             ? kv_multi_col_launch<double>(h, (const double*)E, (const double*)V, (double*)Y, nrhs,
+                                           h->stream)
+             : kv_multi_col_launch<float>(h, (const float*)E, (const float*)V, (float*)Y, nrhs,
+                                          h->stream);
 }
 
 extern "C" mfto_status mfto_kv_multi(mfto_handle* h, mfto_form form, const void* E,
@@ -534,7 +496,7 @@ static mfto_status multi_chunk(mfto_handle* h, cudaStream_t st, int chunk, int n
           h->m_e32, p_new, h->m_q32, h->m_r32, h->m_z32, h->d_dinv32, (int)h->n_dof, h->m_pcg,
           h->d_partials2);
     } else {
-      pcg_kv_multi<<<multi_grid(h, h->occ_multi[2]), MFTO_BLOCK, block_smem(4), st>>>(
+      pcg_kv_multi<<<multi_grid(h, h->occ_multi), MFTO_BLOCK, block_smem(4), st>>>(
           h->d_E32, h->m_z32, p_old, p_new, h->m_q32, h->d_fixed, h->mc32, g, (int)h->n_dof,
           h->m_pcg, h->d_partials);
       pcg_update_multi<<<nb_node, MFTO_BLOCK, 0, st>>>(h->m_e32, p_new, h->m_q32, h->m_r32,
