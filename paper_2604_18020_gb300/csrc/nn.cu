@@ -276,14 +276,14 @@ mse_grad(const float* p, const float* __restrict__ t, const float* __restrict__ 
   }
 }
 
-// second pass (one block): loss = sum / count and 1 / count, in block order
-__global__ void mse_finish(double* partial) {
+// second pass (one block): loss = sum / count and 1 / count, one block's
+// partials per thread, a fixed tree
+__global__ void __launch_bounds__(kLossBlocks) mse_finish(double* partial) {
+  __shared__ double sh[64];
+  double s = block_sum(partial[threadIdx.x], sh);
+  __syncthreads();
+  double c = block_sum(partial[kLossBlocks + threadIdx.x], sh);
   if (threadIdx.x != 0) return;
-  double s = 0.0, c = 0.0;
-  for (int b = 0; b < kLossBlocks; ++b) {
-    s += partial[b];
-    c += partial[kLossBlocks + b];
-  }
   c = c > 1.0 ? c : 1.0;
   partial[2 * kLossBlocks] = s / c;
   partial[2 * kLossBlocks + 1] = 1.0 / c;
@@ -316,6 +316,8 @@ __global__ void to_bf16(const float* __restrict__ a, __nv_bfloat16* __restrict__
 }
 
 unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
+
+#include "nn_wgrad.cuh"
 
 // ---- 3x3x3 convolution on the tensor cores (implicit GEMM, tcgen05) ------
 //
@@ -655,24 +657,58 @@ int n_chunks(int V) {
   return c > 64 ? 64 : (c < 1 ? 1 : c);
 }
 
+// output channels per thread of the weight gradient: the width that pads the
+// layer's channels least (14 serves the default base's 14, 28, 56 and 112)
+int wgrad_co(int cout) {
+  int best = 16;
+  for (int co : {14, 8})
+    if (cdiv(cout, co) * co < cdiv(cout, best) * best) best = co;
+  return best;
+}
+
+mfto_status wgrad_launch(mfto_nn* n, const NnLayer& L, const float* in, const float* dout, Dims d) {
+  const int co = wgrad_co(L.cout);
+  // one wave: three CTAs per SM (shared memory)
+  const WgradPlan pl = wgrad_plan(L.cin, L.cout, d, co, 3 * n->num_sms, n->wpart_elems);
+  const size_t row = (size_t)L.cout * pl.pairs * 3;
+  if ((size_t)pl.tasks * row > n->wpart_elems)
+    return nfail(n, MFTO_INVALID_ARG, "weight partials too small");
+  const dim3 grid(pl.pblocks * pl.cblocks, pl.tasks);
+  n->launches += 2;
+  if (co == 14)
+    wgrad3<14><<<grid, 128, kWgSmem, n->stream>>>(in, L.cin, dout, L.cout, d, pl, n->wpart);
+  else if (co == 16)
+    wgrad3<16><<<grid, 128, kWgSmem, n->stream>>>(in, L.cin, dout, L.cout, d, pl, n->wpart);
+  else
+    wgrad3<8><<<grid, 128, kWgSmem, n->stream>>>(in, L.cin, dout, L.cout, d, pl, n->wpart);
+  NCUDA(n, cudaGetLastError());
+  wgrad_sum<<<cdiv(row, 32), 256, 0, n->stream>>>(n->wpart, L.cin, L.cout, pl, n->grad + L.w_off,
+                                                  n->grad + L.b_off);
+  NCUDA(n, cudaGetLastError());
+  return MFTO_OK;
+}
+
 // weight and bias gradients of one conv into n->grad; if din, the input
 // gradient, gated by `gate` (zero where gate <= 0) when gate is given
 mfto_status conv_backward(mfto_nn* n, const NnLayer& L, const float* in, const float* dout,
                           float* din, const float* gate, Dims d) {
   const int V = d.V();
-  const int KK = L.k * L.k * L.k;
-  const int chunks = n_chunks(V);
-  const int chunk = (V + chunks - 1) / chunks;
-  const size_t nw = (size_t)L.cout * L.cin * KK;
-  if ((size_t)chunks * nw > n->wpart_elems) return nfail(n, MFTO_INVALID_ARG, "weight partials too small");
-  n->launches += 4;
-  if (L.k == 3)
-    conv_bwd_weight<3><<<dim3(L.cout * L.cin, chunks), kNT, 0, n->stream>>>(in, L.cin, dout, L.cout, d, chunk, n->wpart);
-  else
+  if (L.k == 3) {
+    mfto_status s = wgrad_launch(n, L, in, dout, d);
+    if (s != MFTO_OK) return s;
+  } else {
+    const int KK = L.k * L.k * L.k;
+    const int chunks = n_chunks(V);
+    const int chunk = (V + chunks - 1) / chunks;
+    const size_t nw = (size_t)L.cout * L.cin * KK;
+    if ((size_t)chunks * nw > n->wpart_elems)
+      return nfail(n, MFTO_INVALID_ARG, "weight partials too small");
+    n->launches += 4;
     conv_bwd_weight<1><<<dim3(L.cout * L.cin, chunks), kNT, 0, n->stream>>>(in, L.cin, dout, L.cout, d, chunk, n->wpart);
-  sum_chunks<<<cdiv(nw, 256), 256, 0, n->stream>>>(n->wpart, (int)nw, chunks, n->grad + L.w_off);
-  bias_grad<<<dim3(L.cout, chunks), kNT, 0, n->stream>>>(dout, L.cout, V, chunk, n->wpart);
-  sum_chunks<<<cdiv(L.cout, 256), 256, 0, n->stream>>>(n->wpart, L.cout, chunks, n->grad + L.b_off);
+    sum_chunks<<<cdiv(nw, 256), 256, 0, n->stream>>>(n->wpart, (int)nw, chunks, n->grad + L.w_off);
+    bias_grad<<<dim3(L.cout, chunks), kNT, 0, n->stream>>>(dout, L.cout, V, chunk, n->wpart);
+    sum_chunks<<<cdiv(L.cout, 256), 256, 0, n->stream>>>(n->wpart, L.cout, chunks, n->grad + L.b_off);
+  }
   if (din && L.k == 3 && n->tc_conv && n->wpack_t) {
     // the data gradient as the adjoint convolution on the tensor cores
     const size_t li = (size_t)(&L - n->layers.data());
@@ -836,7 +872,7 @@ mfto_status check_dims(mfto_nn* n, int D, int H, int W, bool train) {
 mfto_status loss_and_grad(mfto_nn* n, const float* target, const float* mask, size_t cnt) {
   n->launches += 3;
   mse_grad<<<kLossBlocks, 256, 0, n->stream>>>(n->dpred, target, mask, n->dpred, cnt, n->lpart);
-  mse_finish<<<1, 32, 0, n->stream>>>(n->lpart);
+  mse_finish<<<1, kLossBlocks, 0, n->stream>>>(n->lpart);
   mse_scale<<<cdiv(cnt, 256), 256, 0, n->stream>>>(n->dpred, cnt, n->lpart);
   NCUDA(n, cudaGetLastError());
   return MFTO_OK;
@@ -878,6 +914,12 @@ extern "C" mfto_status mfto_nn_create(int32_t base, int32_t levels, int64_t max_
   n->max_vox = max_voxels;
   n->max_train_vox = max_train_voxels;
   n->stream = (cudaStream_t)stream;
+  n->num_sms = 152;
+  {
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+      cudaDeviceGetAttribute(&n->num_sms, cudaDevAttrMultiProcessorCount, dev);
+  }
   // layers in forward order (encoders, bottleneck, decoders, head)
   const int L = levels;
   size_t off = 0;
@@ -932,6 +974,15 @@ extern "C" mfto_status mfto_nn_create(int32_t base, int32_t levels, int64_t max_
       const int l = (i == n->layers.size() - 1) ? 0 : (bi < L ? bi : 2 * (L - 1) - bi);
       const size_t need = (size_t)n_chunks((int)(TV >> (3 * l))) * ((size_t)ly.cout * ly.cin * ly.k * ly.k * ly.k + ly.cout);
       wp = wp > need ? wp : need;
+      if (ly.k == 3) {
+        // the weight gradient's partials: one wave of CTAs, each 128 pairs x 3
+        // x its output channels; never more than one task per voxel
+        const size_t row = (size_t)ly.cout * (9 * ly.cin + 1) * 3;
+        const size_t wave = (size_t)(3 * n->num_sms) * 128 * 3 * 16;
+        const size_t most = row * (size_t)(TV >> (3 * l));
+        const size_t take = most < wave ? most : wave;
+        wp = wp > take + row ? wp : take + row;
+      }
     }
     n->wpart_elems = wp;
     A((void**)&n->wpart, sizeof(float) * wp);
@@ -958,10 +1009,6 @@ extern "C" mfto_status mfto_nn_create(int32_t base, int32_t levels, int64_t max_
     A((void**)&n->d_err, sizeof(int32_t));
     n->tc_conv = 1;
     n->wpack_dirty = true;
-    int dev = 0;
-    n->num_sms = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess)
-      cudaDeviceGetAttribute(&n->num_sms, cudaDevAttrMultiProcessorCount, dev);
   }
   if (!ok) {
     cudaGetLastError();
@@ -987,6 +1034,12 @@ extern "C" mfto_status mfto_nn_create(int32_t base, int32_t levels, int64_t max_
                            CtShape<16>::SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(conv3_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            CtShape<32>::SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(wgrad3<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem) !=
+          cudaSuccess ||
+      cudaFuncSetAttribute(wgrad3<14>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kWgSmem) != cudaSuccess ||
+      cudaFuncSetAttribute(wgrad3<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kWgSmem) != cudaSuccess ||
       cudaStreamSynchronize(n->stream) != cudaSuccess) {
     cudaGetLastError();
     free_nn(n);
