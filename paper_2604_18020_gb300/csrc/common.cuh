@@ -120,6 +120,7 @@ struct mfto_handle {
   int32_t* d_stencil_off;   // [3 * n_stencil]
   double* d_stencil_w;      // [n_stencil]
   double* d_filter_W;       // row sums W_e
+  int filter_shape, filter_nzc;  // tile width and z-chunk of the near filter (filter.cu)
   // PCG workspace (FP64)
   double *d_r, *d_z, *d_p0, *d_p1, *d_q, *d_dinv;
   double* d_oc;             // [3][n_elem] scratch of the OC update (simp.cu) and the filter
