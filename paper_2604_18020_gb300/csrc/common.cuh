@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include "kv_fixed.cuh"
 #include "../../include/mfto.h"
 
 // Mode-space coefficients for unit modulus; the 1/8 of the inverse transform
@@ -97,6 +98,8 @@ struct mfto_handle {
   float* d_ke32;
   double ke_diag;           // KE[l][l] (equal for every local DOF on a cube)
   ModeCoef<double> mc64;    // mode-space element operator (kv_tile.cuh)
+  FixOp fix;                // ... in fixed point (kv_fixed.cuh), where it fits
+  bool fix_ok;
   ModeCoef<float> mc32;
   int kv_variant;           // 0: tiled mode-space kernel, 1: node-centric dense KE
   int cg_engine;            // FP32 inner CG: 0 two kernels per iteration, 1 persistent,
@@ -671,6 +674,7 @@ mfto_status cg2_enqueue(mfto_handle* h, cudaStream_t st, const PcgVecs<float>& v
                         cudaEvent_t ev1);
 mfto_status pcg_persist_iterate(mfto_handle* h, const PcgVecs<float>& v, PcgScalars* host_s);
 mfto_status kv_tile_init(mfto_handle* h);
+void kv_tile_retile(mfto_handle* h);
 mfto_status simp_init(mfto_handle* h);
 template <typename T>
 mfto_status kv_tile_launch(mfto_handle* h, const T* E, const T* v, T* y, cudaStream_t st);

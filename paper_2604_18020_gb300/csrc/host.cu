@@ -158,6 +158,30 @@ mfto_status filter_rowsums(mfto_handle* h);  // filter.cu
 // Mode-space coefficients of the unit element operator (kv_tile.cuh): the
 // diagonal terms of mode_operator() and the off-diagonal couplings, with
 // the 1/8 of the inverse transform folded in.
+static FixConst scaled(long double c, int t) {   // c / 2^t
+  return fix_const((int64_t)(ldexpl(c, 62 - t) + 0.5L));
+}
+
+bool fixed_op(double nu, double h, FixOp* op) {
+  const double r = 2.0 * nu / (1.0 - 2.0 * nu), q = (r + 4.0) / 9.0;
+  if (!(nu >= 0.0) || !(r < 10.0)) return false;
+  op->k = 0;
+  while (8.0 * (3.0 * r + 2.0) * 1.01 >= (double)(64 << op->k)) ++op->k;
+  if (op->k > 2) return false;
+  const long double lnu = (long double)nu, lr = 2.0L * lnu / (1.0L - 2.0L * lnu);
+  int tr = 0, t3 = 0;
+  while (r >= (double)(1 << tr) * 0.999) ++tr;
+  while ((r / 3.0 > q ? r / 3.0 : q) >= (double)(1 << t3) * 0.999) ++t3;
+  op->r = scaled(lr, tr);
+  op->r3 = scaled(lr / 3.0L, t3);
+  op->third = scaled(1.0L / 3.0L, 0);
+  op->q = scaled((lr + 4.0L) / 9.0L, t3);
+  op->sr = tr + 2;
+  op->s3 = t3 + 2;
+  op->scale = (double)((long double)h / (2.0L * (1.0L + lnu)) / 16.0L);
+  return true;
+}
+
 void mode_coefficients(double nu, double hh, ModeCoef<double>* c64, ModeCoef<float>* c32) {
   const ModeOperator op = mode_operator(1.0, nu, hh);
   memset(c64, 0, sizeof(*c64));
@@ -191,6 +215,8 @@ static mfto_status upload_params(mfto_handle* h) {
     if (s != MFTO_OK) return s;
   }
   mode_coefficients(h->p.nu, h->mesh.h, &h->mc64, &h->mc32);
+  h->fix_ok = fixed_op(h->p.nu, h->mesh.h, &h->fix);
+  kv_tile_retile(h);
   MFTO_CUDA(h, cudaMemcpyAsync(h->d_ke64, ke, sizeof(ke), cudaMemcpyHostToDevice, h->stream));
   MFTO_CUDA(h, cudaMemcpyAsync(h->d_ke32, ke32, sizeof(ke32), cudaMemcpyHostToDevice, h->stream));
   return filter_setup(h);

@@ -24,6 +24,9 @@
 // transforms its 8 corners by itself.  The stages are pipelined over the
 // layers so that one barrier per layer is enough.
 //
+// The operators that kv_fixed.cuh holds (Poisson's ratios of 0 to 0.454) run
+// there; this kernel serves the others.
+//
 // Measured on a GB300, y = K v, against the kernel that transformed each
 // element's corners by itself in 16 x 12 node tiles: 229 against 394 us at
 // 55 x 55 x 165, 18.4 against 79.9 us at 24 x 12 x 12 (the operations above on
@@ -145,6 +148,7 @@ __device__ __forceinline__ void col64_element(const Col64Face& lo_f, const Col64
 
 // Epilogues: what the owner of a node does with its 3 sums.
 struct Col64Store {                   // plain K.v: y = sum, y_fixed = v
+  static constexpr bool kOwn = false;   // pn unused
   const double* v;
   double* y;
   __device__ __forceinline__ void operator()(int node, const double (&acc)[3],
@@ -155,6 +159,7 @@ struct Col64Store {                   // plain K.v: y = sum, y_fixed = v
   }
 };
 struct Col64Pcg {                     // CG: p_new stored, q = K p_new, p_new.q accumulated
+  static constexpr bool kOwn = true;
   double* p_new;
   double* q;
   __device__ __forceinline__ void operator()(int node, const double (&acc)[3],

@@ -1,0 +1,291 @@
+// FP64 K.v (Eq. matfree) evaluated in 64-bit fixed point, z-columns of elements
+// streamed as in kv_column64.cuh.
+//
+// The FP64 pipe runs 2 operations per clock and SM, the integer pipes 64; the
+// 153 FP64 operations per element of kv_column64.cuh are additions and products
+// by a few constants, so they are done on integers.  What floating point does
+// by the operation is done once per node, face and element here: a block of
+// values shares one exponent (that of its largest), and a block meets another
+// at the larger of the two exponents.
+//   node      3 components: |S| < 2^(57-k), one conversion by the FP64 pipe each
+//   face      4 nodes of a column at the exponent of the largest
+//   element   2 faces; mode operator, modulus (its mantissa as a 62-bit
+//             fraction, its exponent added to the block's)
+//   sum       with the element below, then over the 4 columns of a node;
+//             converted back to FP64 by its owner
+// Everything between is exact but for the products by constants and by the
+// modulus, which lose a few units of the last place, so the error of a block is
+// about 2^-57 of its largest input times the operator's norm: less than the
+// roundings of FP64 sums (2^-53 of every partial sum).  Against extended
+// precision (relative 2-norm; FP64 column kernel, then this): K u of a bending
+// field over graded moduli 3.3e-15, 5.6e-16, of a solved cantilever's u 5.8e-14,
+// 6.5e-15; the sensitivities 1.4e-15, 1.8e-16 and 2.3e-15, 4.3e-16.
+//
+// Measured on a GB300, y = K v, against the FP64 column kernel: 392 against
+// 1,973 us at 256 x 128 x 150, 54 against 232 at 55 x 55 x 165, 31 against 117 at
+// 120 x 60 x 30, 11 against 21 at 24 x 12 x 12 (cold L2).  About 1,100 instructions
+// per element and layer, issued on 55 % of the cycles; the rest waits for the
+// layer's barrier and for dependent results.
+#pragma once
+#include <math.h>
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define FIX_HD __host__ __device__ __forceinline__
+#else
+#define FIX_HD inline
+#endif
+
+// A constant 0 <= c < 1 as c 2^62 = hi 2^32 + lo (lo signed).
+struct FixConst {
+  int32_t hi, lo;
+};
+FIX_HD FixConst fix_const(int64_t c62) {
+  return {(int32_t)((c62 + 0x80000000ll) >> 32), (int32_t)(uint32_t)(uint64_t)c62};
+}
+
+// x c / 4 for |x| < 2^63: to within two units
+FIX_HD int64_t fix_mul(int64_t x, FixConst c) {
+  const uint32_t xl = (uint32_t)(uint64_t)x;
+  const int32_t xh = (int32_t)(x >> 32);
+  const int64_t low = (int64_t)((uint64_t)xl * (uint32_t)c.hi) + (int64_t)xh * c.lo;
+  return (int64_t)xh * c.hi + (low >> 32);
+}
+FIX_HD int64_t fix_shl(int64_t x, int s) { return (int64_t)((uint64_t)x << s); }
+
+// The element operator in units of h mu / 2: with r = lam / mu every
+// coefficient is an integer multiple of 1, 1/3, r, r/3 or (r + 4)/9.
+struct FixOp {
+  FixConst r;        // r / 2^(sr - 2)
+  FixConst r3;       // (r / 3) / 2^(s3 - 2)
+  FixConst third;    // 1 / 3
+  FixConst q;        // ((r + 4) / 9) / 2^(s3 - 2)
+  int sr, s3;
+  int k;             // input bits given up for the range of the result
+  double scale;      // h mu / 16: the unit, and the 8 of the mode transforms
+};
+
+// The operator for Poisson's ratio nu and element edge h; false where it does
+// not fit.  The largest sum anywhere is 8 (3 r + 2) times the largest input
+// (the row sum of the element matrix in these units), so k = 0 up to r = 1.97
+// (nu = 0.33), and r < 10 (nu < 0.454) keeps 55 bits of the inputs.  Negative
+// nu would need signed constants.
+bool fixed_op(double nu, double h, FixOp* op);   // host.cu
+
+FIX_HD int fix_min(int a, int b) { return a < b ? a : b; }
+FIX_HD int fix_max(int a, int b) { return a > b ? a : b; }
+
+// Exponents.  A node value is S 2^(e - 1079 + k), e the biased exponent of its
+// largest component, at least 64: what lies 64 or more below the exponent,
+// zeros and subnormals among it, becomes 0.  A value after the modulus is
+// Z 2^(e - 2099 + k).
+constexpr int kFixMinE = 64;
+constexpr int kFixNan = 1 << 14;          // a block with an infinity or a NaN
+constexpr int kFixEmpty = -(1 << 20);     // no contribution
+constexpr int kFixNanOut = 1 << 20;
+
+// four face modes (a + 2b) of three components and their exponent
+struct FixFace {
+  int64_t m[3][4];
+  int e;
+};
+
+// the value with these bits at exponent e, to the nearest: its mantissa shifted left
+// by `left` (4 - k), right by what its own exponent lacks, negated by the sign.
+// On the integer pipes: the conversion of the FP64 pipe, in front of the
+// layer's barrier, made the warps wait.
+FIX_HD int64_t fix_value(uint64_t bits, int e, int left) {
+  const int sh = fix_min(e - (int)((bits >> 52) & 0x7ff), 63);
+  const int64_t m =
+      (((int64_t)(((bits & 0xfffffffffffffull) | 0x10000000000000ull) << (left + 1)) >> sh) + 1) >>
+      1;
+  const int64_t sign = (int64_t)bits >> 63;
+  return (m ^ sign) - sign;
+}
+
+// (sum, difference) modes of a face from its nodes' values v[node][component]
+FIX_HD void fix_face(const int64_t (&v)[4][3], FixFace& F) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int64_t s0 = v[0][c] + v[1][c], d0 = v[1][c] - v[0][c];
+    const int64_t s1 = v[2][c] + v[3][c], d1 = v[3][c] - v[2][c];
+    F.m[c][0] = s0 + s1;
+    F.m[c][2] = s1 - s0;
+    F.m[c][1] = d0 + d1;
+    F.m[c][3] = d1 - d0;
+  }
+}
+
+// z stage: modes f + 4 (z difference) of the element between two faces shifted
+// right by dl and du; mode 0, a translation, is left out
+FIX_HD void fix_modes(const FixFace& lo, const FixFace& up, int dl, int du, int64_t (&X)[3][8]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      const int64_t a = lo.m[c][f] >> dl, b = up.m[c][f] >> du;
+      X[c][f] = f == 0 ? 0 : a + b;
+      X[c][f | 4] = b - a;
+    }
+}
+
+// The modulus: fraction in [1/2, 1) and exponent e (0: zero or below FP64's
+// normal range, taken as zero).
+struct FixModulus {
+  FixConst f;
+  int64_t f62;
+  int e;
+  bool negative;
+};
+FIX_HD FixModulus fix_modulus(uint64_t bits) {
+  FixModulus E;
+  E.negative = (bits >> 63) != 0;
+  E.e = (int)((bits >> 52) & 0x7ff);
+  E.f62 = E.e == 0 ? 0 : (int64_t)(((bits & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
+  E.f = fix_const(E.f62);
+  return E;
+}
+
+// Z = E Kt X / 4 in the units above
+FIX_HD void fix_operator(const int64_t (&X)[3][8], const FixOp& K, const FixModulus& E,
+                         int64_t (&Z)[3][8]) {
+  // constant strains: divergence and shears
+  const int64_t T = fix_shl(fix_mul(X[0][1] + X[1][2] + X[2][4], K.r), K.sr);
+  Z[0][1] = fix_mul(T + fix_shl(X[0][1], 1), E.f);
+  Z[1][2] = fix_mul(T + fix_shl(X[1][2], 1), E.f);
+  Z[2][4] = fix_mul(T + fix_shl(X[2][4], 1), E.f);
+  Z[0][2] = Z[1][1] = fix_mul(X[0][2] + X[1][1], E.f);
+  Z[0][4] = Z[2][1] = fix_mul(X[0][4] + X[2][1], E.f);
+  Z[1][4] = Z[2][2] = fix_mul(X[1][4] + X[2][2], E.f);
+  // strains linear in one axis
+  const int64_t Tx = fix_shl(fix_mul(X[1][3] + X[2][5], K.r3), K.s3);
+  Z[1][3] = fix_mul(Tx + X[1][3], E.f);
+  Z[2][5] = fix_mul(Tx + X[2][5], E.f);
+  const int64_t Ty = fix_shl(fix_mul(X[0][3] + X[2][6], K.r3), K.s3);
+  Z[0][3] = fix_mul(Ty + X[0][3], E.f);
+  Z[2][6] = fix_mul(Ty + X[2][6], E.f);
+  const int64_t Tz = fix_shl(fix_mul(X[0][5] + X[1][6], K.r3), K.s3);
+  Z[0][5] = fix_mul(Tz + X[0][5], E.f);
+  Z[1][6] = fix_mul(Tz + X[1][6], E.f);
+  const FixConst E3 = fix_const(fix_shl(fix_mul(E.f62, K.third), 2));
+  const int64_t S = X[0][6] + X[1][5] + X[2][3];
+  Z[0][6] = fix_mul(X[0][6] + S, E3);
+  Z[1][5] = fix_mul(X[1][5] + S, E3);
+  Z[2][3] = fix_mul(X[2][3] + S, E3);
+  // and bilinear ones
+  const FixConst Eq = fix_const(fix_shl(fix_mul(E.f62, K.q), 2));
+#pragma unroll
+  for (int c = 0; c < 3; ++c) Z[c][7] = fix_shl(fix_mul(X[c][7], Eq), K.s3 - 2);
+}
+
+// Undone z stage and the sum with the element below: Ms = upper outputs of the
+// element below (U) + this one's lower ones; U becomes this one's upper ones.
+FIX_HD void fix_join(const int64_t (&Z)[3][8], int e, FixFace& U, FixFace& Ms) {
+  const int em = fix_max(U.e, e), du = fix_min(em - U.e, 63), dz = fix_min(em - e, 63);
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      const int64_t s = f == 0 ? 0 : Z[c][f], d = Z[c][f | 4];
+      Ms.m[c][f] = (U.m[c][f] >> du) + ((s - d) >> dz);
+      U.m[c][f] = s + d;
+    }
+  Ms.e = em;
+  U.e = e;
+}
+
+// Shares of a column's four edges' nodes (a + 2b) from face modes.
+FIX_HD void fix_corners(const FixFace& M, int64_t (&w)[4][3]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int64_t s0 = M.m[c][0] - M.m[c][2], d0 = M.m[c][1] - M.m[c][3];
+    const int64_t s1 = M.m[c][0] + M.m[c][2], d1 = M.m[c][1] + M.m[c][3];
+    w[0][c] = s0 - d0;
+    w[1][c] = s0 + d0;
+    w[2][c] = s1 - d1;
+    w[3][c] = s1 + d1;
+  }
+}
+
+// A sum of squares in units of 2^64 (exact but for the squares of the low
+// words): 6 terms of |x| <= 2^61 or so fit.
+struct FixSquares {
+  int64_t h = 0, l = 0;
+  FIX_HD void add(int64_t x) {
+    const int32_t lo = (int32_t)(uint32_t)(uint64_t)x, hi = (int32_t)((x - lo) >> 32);
+    h += (int64_t)hi * hi;
+    l += (int64_t)hi * lo;
+  }
+  FIX_HD int64_t sum() const { return h + ((l + (1ll << 30)) >> 31); }
+};
+
+FIX_HD int fix_clz(uint32_t x) {
+#ifdef __CUDA_ARCH__
+  return __clz((int)x);
+#else
+  return x ? __builtin_clz(x) : 32;
+#endif
+}
+
+// x c / 4 to the nearest, for sums whose errors must not lean one way
+FIX_HD int64_t fix_mul_near(int64_t x, FixConst c) {
+  const uint32_t xl = (uint32_t)(uint64_t)x;
+  const int32_t xh = (int32_t)(x >> 32);
+  const int64_t low =
+      (int64_t)((uint64_t)xl * (uint32_t)c.hi + 0x80000000ull) + (int64_t)xh * c.lo;
+  return (int64_t)xh * c.hi + (low >> 32);
+}
+
+// X . Kt X in units of 2^(64 - 2 shift) (h mu / 2) of the modes' unit squared.
+// With the sums of fix_operator the 45 terms are 23 squares in five classes.
+// The sums are exact, and a rigid motion leaves none of them (a rotation
+// cancels in the shears), so all are shifted left by `shift` before they are
+// squared, the largest to about 2^60 (half of that with k > 0, where the
+// coefficients are larger): the energy keeps its precision however far the
+// strains lie below the displacements.
+FIX_HD int64_t fix_energy(const int64_t (&X)[3][8], const FixOp& K, int& shift) {
+  // normal strains, shears, those linear in one axis (two for each), twists
+  // and bilinear ones
+  int64_t v[18] = {X[0][1],           X[1][2],           X[2][4],
+                   X[0][2] + X[1][1], X[0][4] + X[2][1], X[1][4] + X[2][2],
+                   X[1][3],           X[2][5],           X[0][3],
+                   X[2][6],           X[0][5],           X[1][6],
+                   X[0][6],           X[1][5],           X[2][3],
+                   X[0][7],           X[1][7],           X[2][7]};
+  const int top = K.k > 0 ? 5 : 4;
+  shift = 0;
+  for (int pass = 0;; ++pass) {
+    uint32_t big = 0;
+#pragma unroll
+    for (int n = 0; n < 18; ++n) {
+      const int32_t hi = (int32_t)(v[n] >> 32);
+      big |= (uint32_t)(hi ^ (hi >> 31));
+    }
+    // high words all zero: the values are below 2^32 (at most three passes,
+    // the last for values of a few bits)
+    const int s = big != 0 ? fix_max(fix_clz(big) - top, 0) : 32 - top;
+#pragma unroll
+    for (int n = 0; n < 18; ++n) v[n] = fix_shl(v[n], s);
+    shift += s;
+    if (big != 0 || pass == 2) break;
+  }
+  FixSquares div, lin, own, one, third, bil;
+  div.add(v[0] + v[1] + v[2]);
+  lin.add(v[6] + v[7]);
+  lin.add(v[8] + v[9]);
+  lin.add(v[10] + v[11]);
+  third.add(v[12] + v[13] + v[14]);
+#pragma unroll
+  for (int n = 0; n < 3; ++n) {
+    own.add(v[n]);
+    third.add(v[12 + n]);
+    bil.add(v[15 + n]);
+  }
+#pragma unroll
+  for (int n = 3; n < 12; ++n) one.add(v[n]);
+  // the classes at most 24, 9, 12, 12 and 3 times 2^56 (a quarter with k > 0)
+  return one.sum() + 2 * own.sum() + fix_shl(fix_mul_near(div.sum(), K.r), K.sr) +
+         fix_shl(fix_mul_near(lin.sum(), K.r3), K.s3) +
+         fix_shl(fix_mul_near(third.sum(), K.third), 2) +
+         fix_shl(fix_mul_near(bil.sum(), K.q), K.s3);
+}

@@ -4,6 +4,7 @@
 #include "common.cuh"
 #include "kv_column.cuh"
 #include "kv_column64.cuh"
+#include "kv_column_fixed.cuh"
 #include "kv_tile.cuh"
 
 namespace {
@@ -42,6 +43,18 @@ pcg_kv_block_kernel(const float* __restrict__ E, const float* __restrict__ z,
   }
 }
 
+// alpha of a CG step from p.q
+__device__ __forceinline__ void pcg_alpha(PcgScalars* s, double pq) {
+  s->pq = pq;
+  if (!(pq > 0.0) || !isfinite(pq)) {
+    s->done = 1;
+    s->status = MFTO_BREAKDOWN;
+    s->alpha = 0.0;
+  } else {
+    s->alpha = s->rz / pq;
+  }
+}
+
 // FP64: column-streaming body (kv_column64.cuh), one tile per CTA.  Held to
 // 168 registers, so that three CTAs of 128 threads share an SM (229 us at
 // 55 x 55 x 165; two, with 184 registers: 303 us).
@@ -72,16 +85,48 @@ pcg_kv_col64_kernel(const double* __restrict__ E, const double* __restrict__ z,
                                     Col64LoadDirection{z, p_old, s->beta}, Col64Pcg{p_new, q},
                                     reinterpret_cast<double*>(smem_raw));
   double tot[1];
-  if (last_block_reduce<1>(red, partials, &s->ticket_b, tot, sh) && threadIdx.x == 0) {
-    s->pq = tot[0];
-    if (!(tot[0] > 0.0) || !isfinite(tot[0])) {
-      s->done = 1;
-      s->status = MFTO_BREAKDOWN;
-      s->alpha = 0.0;
-    } else {
-      s->alpha = s->rz / tot[0];
-    }
-  }
+  if (last_block_reduce<1>(red, partials, &s->ticket_b, tot, sh) && threadIdx.x == 0)
+    pcg_alpha(s, tot[0]);
+}
+
+// FP64 in fixed point (kv_column_fixed.cuh), the operator of nu in [0, 0.454).
+template <int CX, int CY>
+__global__ void __launch_bounds__(CX * CY, kFixThreads / (CX * CY))
+kv_fixed_kernel(const double* __restrict__ E, const double* __restrict__ v,
+                double* __restrict__ y, const uint8_t* __restrict__ fixed, FixOp K, Grid g,
+                Col64Tiling tl, int n_dof) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  v += (size_t)blockIdx.y * n_dof;   // grid row: load case
+  y += (size_t)blockIdx.y * n_dof;
+  kv_column_fixed_body<CX, CY>(E, fixed, K, g, tl, blockIdx.x, Col64LoadPlain{v}, Col64Store{v, y},
+                               reinterpret_cast<double*>(smem_raw));
+}
+
+template <int CX, int CY>
+__global__ void __launch_bounds__(CX * CY, kFixThreads / (CX * CY))
+pcg_kv_fixed_kernel(const double* __restrict__ E, const double* __restrict__ z,
+                    const double* __restrict__ p_old, double* __restrict__ p_new,
+                    double* __restrict__ q, const uint8_t* __restrict__ fixed, FixOp K, Grid g,
+                    Col64Tiling tl, PcgScalars* s, double* partials) {
+  if (*(volatile int32_t*)&s->done) return;  // uniform over the grid
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double sh[64];
+  double red[1];
+  red[0] = kv_column_fixed_body<CX, CY>(E, fixed, K, g, tl, blockIdx.x,
+                                        Col64LoadDirection{z, p_old, s->beta}, Col64Pcg{p_new, q},
+                                        reinterpret_cast<double*>(smem_raw));
+  double tot[1];
+  if (last_block_reduce<1>(red, partials, &s->ticket_b, tot, sh) && threadIdx.x == 0)
+    pcg_alpha(s, tot[0]);
+}
+
+template <int CX, int CY>
+constexpr size_t fixed_smem() {
+  return FixShape<CX, CY, Col64LoadPlain, Col64Store>::kBytes;
+}
+template <int CX, int CY>
+constexpr size_t pcg_fixed_smem() {
+  return FixShape<CX, CY, Col64LoadDirection, Col64Pcg>::kBytes;
 }
 
 template <typename S>
@@ -95,6 +140,14 @@ Col64Tiling col64_tiling(const mfto_handle* h, int nzc) {
   return t;
 }
 
+// tile shape and z-chunk of the FP64 column kernel in use
+void col64_tile(const mfto_handle* h, const Grid& g, int* shape, int* nzc, int copies) {
+  if (h->fix_ok)
+    fixed_choose(g.nx, g.ny, g.nz, h->num_sms, shape, nzc, copies);
+  else
+    col64_choose(1, g.nx, g.ny, g.nz, 1.5, h->num_sms, shape, nzc, copies);
+}
+
 mfto_status col64_attrs(mfto_handle* h) {
   for (int i = 0; i < kCol64Shapes; ++i) {
     const mfto_status s = col64_dispatch(i, [&](auto shape) -> mfto_status {
@@ -105,6 +158,12 @@ mfto_status col64_attrs(mfto_handle* h) {
       MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_col64_kernel<S::CX, S::CY>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)S::template smem_bytes<2>()));
+      MFTO_CUDA(h, cudaFuncSetAttribute(kv_fixed_kernel<S::CX, S::CY>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)fixed_smem<S::CX, S::CY>()));
+      MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_fixed_kernel<S::CX, S::CY>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)pcg_fixed_smem<S::CX, S::CY>()));
       return MFTO_OK;
     });
     if (s != MFTO_OK) return s;
@@ -114,15 +173,18 @@ mfto_status col64_attrs(mfto_handle* h) {
 
 // FP32, variant 0: column-streaming body (kv_column.cuh).  MINB: resident
 // CTAs per SM the register allocation is held to (2: up to 128 registers per
-// thread, 3: up to 80); mfto_kv_autotune picks one.
-template <int MINB>
+// thread, 3: up to 80); mfto_kv_autotune picks one.  MULTI: a grid row per load
+// case (a kernel of its own: the row offsets cost the single K.v 1.5 %).
+template <int MINB, bool MULTI>
 __global__ void __launch_bounds__(MFTO_BLOCK, MINB)
 kv_col_kernel(const float* __restrict__ E, const float* __restrict__ v, float* __restrict__ y,
               const uint8_t* __restrict__ fixed, ModeCoef<float> K, Grid g, ColTiling tl,
               int n_dof) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  v += (size_t)blockIdx.y * n_dof;   // grid row: load case
-  y += (size_t)blockIdx.y * n_dof;
+  if constexpr (MULTI) {
+    v += (size_t)blockIdx.y * n_dof;
+    y += (size_t)blockIdx.y * n_dof;
+  }
   kv_column_body(E, fixed, K, g, tl, ColLoadPlain{v}, ColStore{v, y},
                  reinterpret_cast<float*>(smem_raw));
 }
@@ -341,9 +403,12 @@ ColTiling col_launch_tiling(const mfto_handle* h, int per_sm, int* grid) {
   return tl;
 }
 
+// The FP64 column kernel's tiles, for the operator of the current parameters.
+void kv_tile_retile(mfto_handle* h) {
+  col64_tile(h, make_grid(h->mesh), &h->col64_shape, &h->col64_nzc, 1);
+}
+
 mfto_status kv_tile_init(mfto_handle* h) {
-  const Grid g = make_grid(h->mesh);
-  col64_choose(1, g.nx, g.ny, g.nz, 1.5, h->num_sms, &h->col64_shape, &h->col64_nzc);
   const mfto_status s = col64_attrs(h);
   if (s != MFTO_OK) return s;
   MFTO_CUDA(h, cudaFuncSetAttribute(kv_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -351,8 +416,14 @@ mfto_status kv_tile_init(mfto_handle* h) {
   MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_block_kernel,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlockSmem));
   const int csm = (int)kColSmem;
-  MFTO_CUDA(h, cudaFuncSetAttribute(kv_col_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, csm));
-  MFTO_CUDA(h, cudaFuncSetAttribute(kv_col_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, csm));
+  MFTO_CUDA(h, cudaFuncSetAttribute(kv_col_kernel<2, false>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, csm));
+  MFTO_CUDA(h, cudaFuncSetAttribute(kv_col_kernel<2, true>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, csm));
+  MFTO_CUDA(h, cudaFuncSetAttribute(kv_col_kernel<3, false>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, csm));
+  MFTO_CUDA(h, cudaFuncSetAttribute(kv_col_kernel<3, true>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, csm));
   MFTO_CUDA(h, cudaFuncSetAttribute(gmg_sweep_col_kernel<2, 0>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, csm));
   MFTO_CUDA(h, cudaFuncSetAttribute(gmg_sweep_col_kernel<2, 1>,
@@ -462,6 +533,12 @@ static mfto_status col64_launch(mfto_handle* h, const double* E, const double* v
   const mfto_status s = col64_dispatch(shape, [&](auto sh) -> mfto_status {
     using S = decltype(sh);
     const Col64Tiling tl = col64_tiling<S>(h, nzc);
+    if (h->fix_ok) {
+      kv_fixed_kernel<S::CX, S::CY>
+          <<<dim3(tl.count(), nrhs), S::NT, fixed_smem<S::CX, S::CY>(), st>>>(
+              E, v, y, h->d_fixed, h->fix, make_grid(h->mesh), tl, (int)h->n_dof);
+      return MFTO_OK;
+    }
     kv_col64_kernel<S::CX, S::CY>
         <<<dim3(tl.count(), nrhs), S::NT, S::template smem_bytes<1>(), st>>>(
             E, v, y, h->d_fixed, h->mc64, make_grid(h->mesh), tl, (int)h->n_dof);
@@ -475,12 +552,16 @@ static mfto_status col_launch(mfto_handle* h, const float* E, const float* v, fl
                               int kind, const ColTiling& tl, int grid, cudaStream_t st) {
   const Grid g = make_grid(h->mesh);
   const dim3 gr((unsigned)grid, (unsigned)nrhs);
-  if (kind == 1)
-    kv_col_kernel<3><<<gr, MFTO_BLOCK, kColSmem, st>>>(E, v, y, h->d_fixed, h->mc32, g, tl,
-                                                       (int)h->n_dof);
-  else
-    kv_col_kernel<2><<<gr, MFTO_BLOCK, kColSmem, st>>>(E, v, y, h->d_fixed, h->mc32, g, tl,
-                                                       (int)h->n_dof);
+  const int n_dof = (int)h->n_dof;
+#define MFTO_KV_COL(MINB, MULTI)                                                              \
+  kv_col_kernel<MINB, MULTI><<<gr, MFTO_BLOCK, kColSmem, st>>>(E, v, y, h->d_fixed, h->mc32,  \
+                                                               g, tl, n_dof)
+  if (kind == 1) {
+    if (nrhs > 1) MFTO_KV_COL(3, true); else MFTO_KV_COL(3, false);
+  } else {
+    if (nrhs > 1) MFTO_KV_COL(2, true); else MFTO_KV_COL(2, false);
+  }
+#undef MFTO_KV_COL
   MFTO_LAUNCH_CHECK(h);
   return MFTO_OK;
 }
@@ -514,7 +595,7 @@ mfto_status kv_multi_col_launch<double>(mfto_handle* h, const double* E, const d
                                         double* Y, int nrhs, cudaStream_t st) {
   const Grid g = make_grid(h->mesh);
   int shape = 0, nzc = 1;
-  col64_choose(1, g.nx, g.ny, g.nz, 1.5, h->num_sms, &shape, &nzc, nrhs);
+  col64_tile(h, g, &shape, &nzc, nrhs);
   return col64_launch(h, E, V, Y, nrhs, shape, nzc, st);
 }
 
@@ -558,6 +639,12 @@ mfto_status pcg_kv_tile_launch<double>(mfto_handle* h, const double* E, const do
     const Col64Tiling tl = col64_tiling<S>(h, h->col64_nzc);
     if (tl.count() > MFTO_RED_SLOTS)
       return mfto_fail(h, MFTO_TOO_LARGE, "mesh too large for the K.v tiling");
+    if (h->fix_ok) {
+      pcg_kv_fixed_kernel<S::CX, S::CY>
+          <<<tl.count(), S::NT, pcg_fixed_smem<S::CX, S::CY>(), st>>>(
+              E, z, p_old, p_new, q, h->d_fixed, h->fix, make_grid(h->mesh), tl, s, partials);
+      return MFTO_OK;
+    }
     pcg_kv_col64_kernel<S::CX, S::CY><<<tl.count(), S::NT, S::template smem_bytes<2>(), st>>>(
         E, z, p_old, p_new, q, h->d_fixed, h->mc64, make_grid(h->mesh), tl, s, partials);
     return MFTO_OK;
