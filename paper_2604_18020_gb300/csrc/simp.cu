@@ -4,6 +4,7 @@
 
 #include "common.cuh"
 #include "kv_column64.cuh"
+#include "kv_column_fixed.cuh"
 #include "simp_power.cuh"
 
 namespace {
@@ -50,6 +51,23 @@ __device__ __forceinline__ double mode_energy(const double (&X)[3][8],
   return fma(K.diag[0][7], sq[4], ce);
 }
 
+// What follows from an element's energy: its share of the compliance and of the
+// grayness sum, and its sensitivity.
+struct ElementEnergy {
+  double E0, Emin, penal;
+  const PowPlan& plan;
+  double* dc;
+  int e0, nexy;
+  double (&acc)[2];
+  __device__ __forceinline__ void operator()(double r, double ce, int ez) const {
+    double rp, rp1;
+    simp_powers<true>(r, penal, plan, rp, rp1);
+    acc[0] = fma(fma(E0 - Emin, rp, Emin), ce, acc[0]);
+    acc[1] += fma(-r, r, r);
+    if (dc) dc[e0 + nexy * ez] = -penal * (E0 - Emin) * rp1 * ce;
+  }
+};
+
 // ce_e = u_e^T KE u_e;  c = sum_e E_e ce_e;  dc_e = -p rho^(p-1) (E0-Emin) ce_e;
 // grayness sum 4 rho (1 - rho).  Fixed-order sums.
 //
@@ -87,6 +105,7 @@ compliance_kernel(const double* __restrict__ rho, const double* __restrict__ u,
   __syncthreads();
   Col64Face F0, F1;
   st.face(kb, F0);
+  const ElementEnergy element{E0, Emin, penal, plan, dc, e0, nexy, acc};
   auto layer = [&](int ez, const Col64Face& lo, Col64Face& up) {
     double r = 0.0;
     if (in) r = rho[e0 + nexy * ez];
@@ -99,13 +118,7 @@ compliance_kernel(const double* __restrict__ rho, const double* __restrict__ u,
     double X[3][8];
     col64_modes(lo, up, X);
     const double ce = mode_energy(X, K);
-    if (in) {
-      double rp, rp1;
-      simp_powers<true>(r, penal, plan, rp, rp1);
-      acc[0] = fma(fma(E0 - Emin, rp, Emin), ce, acc[0]);
-      acc[1] += fma(-r, r, r);
-      if (dc) dc[e0 + nexy * ez] = -penal * (E0 - Emin) * rp1 * ce;
-    }
+    if (in) element(r, ce, ez);
   };
   for (int ez = kb; ez < ke; ez += 2) {
     layer(ez, F0, F1);
@@ -117,6 +130,79 @@ compliance_kernel(const double* __restrict__ rho, const double* __restrict__ u,
     s->sum[0] = tot[0];
     s->sum[1] = 4.0 * tot[1];
   }
+}
+
+// The same on the fixed-point node stream (kv_column_fixed.cuh): the transforms
+// and the energy's squares on the integer pipes, about 12 FP64 operations per
+// element left (one conversion, powers and sums).  Measured on a GB300, p = 3,
+// against the kernel above, which serves the other Poisson's ratios: 303 against
+// 966 us at 256 x 128 x 150, 74 against 150 at 55 x 55 x 165, 49 against 76 at
+// 120 x 60 x 30 (the call, with its host round trip of about 25 us).
+template <int CX, int CY>
+__global__ void __launch_bounds__(CX * CY, kCol64Threads / (CX * CY))
+compliance_fixed_kernel(const double* __restrict__ rho, const double* __restrict__ u,
+                        double* __restrict__ dc, FixOp K, Grid g, Col64Tiling tl, double E0,
+                        double Emin, double penal, PowPlan plan, MiscScalars* s,
+                        double* partials) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double sh[64];
+  using St = FixStream<CX, CY, Col64LoadPlain, false>;
+  const int tile = blockIdx.x;
+  const int bx = tile % tl.tx, by = (tile / tl.tx) % tl.ty, bz = tile / (tl.tx * tl.ty);
+  const int kb = bz * tl.nzc, ke = min(kb + tl.nzc, g.nelz);   // element layers [kb, ke)
+  const Col64LoadPlain ld{u};
+  double* words = reinterpret_cast<double*>(smem_raw);
+  St st(words, reinterpret_cast<int*>(words + St::kWords), ld, nullptr, g, bx * CX, by * CY, ke,
+        K.k);
+  const int gi = bx * CX + threadIdx.x % CX, gj = by * CY + threadIdx.x / CX;
+  const bool in = gi < g.nelx && gj < g.nely;
+  const bool warp_in = __any_sync(0xffffffffu, in);
+  const int e0 = gi + g.nelx * gj, nexy = g.nelx * g.nely;
+  double acc[2] = {0.0, 0.0};
+  const ElementEnergy element{E0, Emin, penal, plan, dc, e0, nexy, acc};
+  st.issue(kb);
+  st.issue(kb + 1);
+  col64_wait<1>();
+  st.stage(kb, 0u);
+  st.issue(kb + 2);
+  double r_next = in ? rho[e0 + nexy * kb] : 0.0;
+  __syncthreads();
+  FixFace F0, F1;
+  st.face(kb, F0);
+  auto layer = [&](int ez, const FixFace& lo, FixFace& up) {
+    const double r = r_next;
+    if (in && ez + 1 < ke) r_next = rho[e0 + nexy * (ez + 1)];
+    col64_wait<1>();
+    st.stage(ez + 1, 0u);
+    st.issue(ez + 3);
+    __syncthreads();
+    if (!warp_in) return;
+    st.face(ez + 1, up);
+    const int em = max(lo.e, up.e);
+    int64_t X[3][8];
+    fix_modes(lo, up, min(em - lo.e, 63), min(em - up.e, 63), X);
+    int shift;
+    const double e = __ll2double_rn(fix_energy(X, K, shift));
+    const double ce = em >= kFixNan ? __longlong_as_double(0x7ff8000000000000ll)
+                                    : fix_scaled(e, 2 * (em - 1079 + K.k - shift) + 64, K);
+    if (in) element(r, ce, ez);
+  };
+  for (int ez = kb; ez < ke; ez += 2) {
+    layer(ez, F0, F1);
+    if (ez + 1 < ke) layer(ez + 1, F1, F0);
+  }
+  col64_wait<0>();
+  double tot[2];
+  if (last_block_reduce<2>(acc, partials, &s->ticket, tot, sh) && threadIdx.x == 0) {
+    s->sum[0] = tot[0];
+    s->sum[1] = 4.0 * tot[1];
+  }
+}
+
+template <typename S>
+constexpr size_t energy_smem() {
+  using St = FixStream<S::CX, S::CY, Col64LoadPlain, false>;
+  return 8 * (size_t)St::kWords + 4 * (size_t)St::kExp;
 }
 
 // OC with bisection on lambda.  The candidate of a midpoint lambda is, per
@@ -616,6 +702,12 @@ mfto_status compliance_launch(mfto_handle* h, const double* rho, const double* u
     tl.tz = (g.nelz + tl.nzc - 1) / tl.nzc;
     if (tl.count() > MFTO_RED_SLOTS)
       return mfto_fail(h, MFTO_TOO_LARGE, "mesh too large for the compliance tiling");
+    if (h->fix_ok) {
+      compliance_fixed_kernel<S::CX, S::CY><<<tl.count(), S::NT, energy_smem<S>(), h->stream>>>(
+          rho, u, dc, h->fix, g, tl, h->p.E0, h->p.Emin, h->p.penal, pow_plan(h->p.penal),
+          h->d_misc, h->d_partials);
+      return MFTO_OK;
+    }
     compliance_kernel<S::CX, S::CY>
         <<<tl.count(), S::NT, S::template stream_bytes<1>(), h->stream>>>(
             rho, u, dc, h->mc64, g, tl, h->p.E0, h->p.Emin, h->p.penal, pow_plan(h->p.penal),
@@ -641,6 +733,9 @@ mfto_status simp_init(mfto_handle* h) {
       MFTO_CUDA(h, cudaFuncSetAttribute(compliance_kernel<S::CX, S::CY>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)S::template stream_bytes<1>()));
+      MFTO_CUDA(h, cudaFuncSetAttribute(compliance_fixed_kernel<S::CX, S::CY>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)energy_smem<S>()));
       return MFTO_OK;
     });
     if (s != MFTO_OK) return s;
