@@ -3,14 +3,19 @@
 // one persistent launch over all instances, and the inner CG chunks are
 // captured into one CUDA graph.
 //
-// Work list: each instance is cut into element blocks (BX x BY x BZ elements,
-// the owned nodes are the (BX-1) x (BY-1) x (BZ-1) interior); the blocks of
-// all instances are numbered consecutively, instance by instance.  A
-// persistent grid (resident CTAs x SMs) walks this list; a CTA maps a global
-// block number to its instance by binary search over the instances' first
-// block numbers.  Per-instance sums (CG dot products, residual norms) are
-// formed per block and reduced per instance, in block order, by the last CTA
-// to finish -- deterministic and without atomics on the data.
+// The FP32 inner CG runs on the row tiles of batch_cg.cuh, two kernels per
+// iteration, every CTA summing its own instance's dot products; the outer FP64
+// residual on the fixed-point column kernel (kv_column_fixed.cuh), a tile list
+// over the instances.
+//
+// Plain K.V and the outer residual's sums: each instance is cut into element
+// blocks (BX x BY x BZ elements, the owned nodes are the (BX-1) x (BY-1) x
+// (BZ-1) interior); the blocks of all instances are numbered consecutively,
+// instance by instance.  A persistent grid (resident CTAs x SMs) walks this
+// list; a CTA maps a global block number to its instance by binary search over
+// the instances' first block numbers.  Per-instance residual norms are formed
+// per block and reduced per instance, in block order, by the last CTA to
+// finish -- deterministic and without atomics on the data.
 //
 // The block shape is a template parameter; mfto_batch_autotune times the
 // candidates on the batch itself and keeps the fastest.
@@ -20,6 +25,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "kv_column_fixed.cuh"
 #include "kv_tile.cuh"
 
 #define MFTO_BATCH_MAX 256
@@ -32,19 +38,25 @@ struct BatchInst {
   int up_blk0, up_nblk;      // node blocks of the vector kernels
 };
 
-struct BatchScal {
-  double rz, pq, alpha, beta, rr, ff, rtol2ff;
-  int32_t it, done, status, pad;
-};
+#include "batch_cg.cuh"
 
 struct BatchCtl {
-  int32_t count, all_done, maxit, pad;
-  unsigned int ticket_a, ticket_b, ticket_c, ticket_d;
+  int32_t all_done;
+  unsigned int ticket_d;
 };
+
+// FP64 tiles of an instance: the shape below, z-chunks of nzc node layers
+struct BatchTiles64 {
+  Grid g;
+  Col64Tiling tl;
+  int tile0;
+};
+using BatchShape64 = Col64Shape<16, 8>;
 
 struct BatchGraph {
   int chunk = 0;
-  int shape = -1;
+  int maxit = 0;          // what the captured launches hold
+  double rtol = 0.0;
   cudaGraphExec_t exec = nullptr;
 };
 
@@ -60,19 +72,27 @@ struct mfto_batch {
   int shape;
   int kv_total[MFTO_BATCH_SHAPES];
   int up_total;
-  int occ_kv64[MFTO_BATCH_SHAPES], occ_kv32[MFTO_BATCH_SHAPES], occ_pcg[MFTO_BATCH_SHAPES];
+  int occ_kv64[MFTO_BATCH_SHAPES], occ_kv32[MFTO_BATCH_SHAPES];
   BatchInst* d_inst[MFTO_BATCH_SHAPES];
   uint8_t* d_fixed;
   ModeCoef<double> mc64;
   ModeCoef<float> mc32;
+  FixOp fix;                       // FP64 operator in fixed point, where it fits
+  bool fix_ok;
   double ke_diag;
+  // tiles and update CTAs of the inner CG, FP64 tiles
+  BatchTiles* d_tiles;
+  int *d_tile_inst, *d_up_inst, *d_tile64_inst;
+  BatchTiles64* d_tiles64;
+  int cg_tiles, cg_updates, tiles64;
   float *r32, *z32, *p0, *p1, *q32, *e32, *dinv32, *E32;
   double* q64;
-  BatchScal* d_scal;
+  BatchScal* d_scal;               // [2][count], by the iteration's parity
   BatchScal* h_scal;
   BatchCtl* d_ctl;
   BatchCtl* h_ctl;
-  double *d_part_a, *d_part_b;     // [2][max blocks]
+  double* d_part_a;                // [2][max blocks]
+  float2 *d_share_a, *d_share_b;   // inner CG: [cg_tiles], [2][cg_updates]
   double* d_res;                   // [2 * count] outer residual sums
   int* d_mask;                     // [count] 1 = instance converged/stopped
   double* d_rzp;                   // [count] r.z of a continued direction (0: p = z)
@@ -257,52 +277,19 @@ batch_kv_kernel(const T* __restrict__ E, const T* __restrict__ V, T* __restrict_
   }
 }
 
-// inner CG step A over all live instances
-template <int S>
-__global__ void __launch_bounds__(MFTO_BLOCK)
-batch_pcg_kv(const float* __restrict__ E, const float* __restrict__ Z, const float* __restrict__ P0,
-             float* __restrict__ P1, float* __restrict__ Q, const uint8_t* __restrict__ fixed,
-             ModeCoef<float> K, const BatchInst* __restrict__ inst, BatchScal* sc, BatchCtl* ctl,
-             double* part, int total) {
-  if (*(volatile int32_t*)&ctl->all_done) return;
+// FP64 in fixed point: one tile of one instance per CTA
+__global__ void __launch_bounds__(BatchShape64::NT, kFixThreads / BatchShape64::NT)
+batch_kv_fixed(const double* __restrict__ E, const double* __restrict__ V, double* __restrict__ Y,
+               const uint8_t* __restrict__ fixed, FixOp K, const BatchInst* __restrict__ inst,
+               const BatchTiles64* __restrict__ tiles, const int* __restrict__ tile_inst) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int first[MFTO_BATCH_MAX];
-  __shared__ double sh[64];
-  const int count = ctl->count;
-  for (int i = threadIdx.x; i < count; i += blockDim.x) first[i] = inst[i].kv_blk0;
-  __syncthreads();
-  for (int gb = blockIdx.x; gb < total; gb += gridDim.x) {
-    const int i = find_inst(first, count, gb);
-    const BatchInst in = inst[i];
-    double pq = 0.0;
-    if (!sc[i].done) {                       // uniform over the CTA
-      const float beta = (float)sc[i].beta;
-      const long long o = 3 * in.node_off;
-      DotAcc<float> red;
-      batch_block<float, S>(E + in.elem_off, fixed + in.node_off, K, in, gb - in.kv_blk0,
-                            TileLoadDirection<float>{Z + o, P0 + o, beta},
-                            TilePcg<float>{P1 + o, Q + o}, reinterpret_cast<float*>(smem_raw), red);
-      pq = block_sum_w0(red.finish(), sh);
-    }
-    if (threadIdx.x == 0) part[gb] = pq;
-  }
-  if (batch_last_cta(&ctl->ticket_b)) {
-    __shared__ double tot[MFTO_BATCH_MAX];
-    per_instance_sums<1>(part, 0, inst, count, true, tot);
-    __syncthreads();
-    for (int i = threadIdx.x; i < count; i += blockDim.x) {
-      if (sc[i].done) continue;
-      sc[i].pq = tot[i];
-      if (!(tot[i] > 0.0) || !isfinite(tot[i])) {
-        sc[i].done = 1;
-        sc[i].status = MFTO_BREAKDOWN;
-        sc[i].alpha = 0.0;
-      } else {
-        sc[i].alpha = sc[i].rz / tot[i];
-      }
-    }
-    if (threadIdx.x == 0) ctl->ticket_b = 0u;
-  }
+  const int i = tile_inst[blockIdx.x];
+  const BatchTiles64 t = tiles[i];
+  const long long node = inst[i].node_off;
+  const double* v = V + 3 * node;
+  kv_column_fixed_body<BatchShape64::CX, BatchShape64::CY>(
+      E + inst[i].elem_off, fixed + node, K, t.g, t.tl, blockIdx.x - t.tile0, Col64LoadPlain{v},
+      Col64Store{v, Y + 3 * node}, reinterpret_cast<double*>(smem_raw));
 }
 
 // node-block walk of the vector kernels: calls f(i, node) for each node
@@ -314,136 +301,6 @@ __device__ __forceinline__ void for_instance_nodes(const int* first, const Batch
   const int n_node = in.nx * in.ny * in.nz;
   const int local = (gb - in.up_blk0) * MFTO_BLOCK + threadIdx.x;
   f(i, local < n_node ? in.node_off + local : -1LL);
-}
-
-// inner CG step B over all live instances
-__global__ void __launch_bounds__(MFTO_BLOCK)
-batch_update(float* __restrict__ U, const float* __restrict__ P, const float* __restrict__ Q,
-             float* __restrict__ R, float* __restrict__ Z, const float* __restrict__ dinv,
-             const BatchInst* __restrict__ inst, BatchScal* sc, BatchCtl* ctl, double* part,
-             int total, int stride) {
-  if (*(volatile int32_t*)&ctl->all_done) return;
-  __shared__ int first[MFTO_BATCH_MAX];
-  __shared__ double sh[64];
-  const int count = ctl->count;
-  for (int i = threadIdx.x; i < count; i += blockDim.x) first[i] = inst[i].up_blk0;
-  __syncthreads();
-  for (int gb = blockIdx.x; gb < total; gb += gridDim.x) {
-    DotAcc<float> d0, d1;
-    int inst_i = 0;
-    for_instance_nodes(first, inst, count, gb, [&](int i, long long node) {
-      inst_i = i;
-      if (node < 0 || sc[i].done) return;
-      const float alpha = (float)sc[i].alpha;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const long long k = 3 * node + c;
-        U[k] += alpha * P[k];
-        const float ri = R[k] - alpha * Q[k];
-        const float zi = ri * dinv[k];
-        R[k] = ri;
-        Z[k] = zi;
-        d0.add_prod(ri, zi);
-        d1.add_prod(ri, ri);
-      }
-    });
-    (void)inst_i;
-    const double a = block_sum_w0(d0.finish(), sh);
-    const double b = block_sum_w0(d1.finish(), sh);
-    if (threadIdx.x == 0) {
-      part[gb] = a;
-      part[stride + gb] = b;
-    }
-  }
-  if (batch_last_cta(&ctl->ticket_c)) {
-    __shared__ double tot[2 * MFTO_BATCH_MAX];
-    per_instance_sums<2>(part, stride, inst, count, false, tot);
-    __syncthreads();
-    for (int i = threadIdx.x; i < count; i += blockDim.x) {
-      BatchScal& s = sc[i];
-      if (s.done) continue;
-      s.it += 1;
-      s.rr = tot[2 * i + 1];
-      s.beta = tot[2 * i] / s.rz;
-      s.rz = tot[2 * i];
-      if (!isfinite(tot[2 * i]) || !isfinite(tot[2 * i + 1])) {
-        s.done = 1;
-        s.status = MFTO_BREAKDOWN;
-      } else if (tot[2 * i + 1] <= s.rtol2ff) {
-        s.done = 1;
-        s.status = MFTO_OK;
-      } else if (s.it >= ctl->maxit) {
-        s.done = 1;
-        s.status = MFTO_NOT_CONVERGED;
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int all = 1;
-      for (int i = 0; i < count; ++i) all &= sc[i].done;
-      ctl->all_done = all;
-      ctl->ticket_c = 0u;
-    }
-  }
-}
-
-// inner solve start: r = rhs (in place), z = r / d, r.z and r.r per instance
-__global__ void __launch_bounds__(MFTO_BLOCK)
-batch_init(float* R, float* __restrict__ Z, const float* __restrict__ dinv,
-           const BatchInst* __restrict__ inst, BatchScal* sc, BatchCtl* ctl, double* part,
-           int total, int stride, double rtol, int maxit, int count,
-           const double* __restrict__ rz_prev) {
-  __shared__ int first[MFTO_BATCH_MAX];
-  __shared__ double sh[64];
-  for (int i = threadIdx.x; i < count; i += blockDim.x) first[i] = inst[i].up_blk0;
-  __syncthreads();
-  for (int gb = blockIdx.x; gb < total; gb += gridDim.x) {
-    DotAcc<float> d0, d1;
-    for_instance_nodes(first, inst, count, gb, [&](int, long long node) {
-      if (node < 0) return;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const long long k = 3 * node + c;
-        const float ri = R[k];
-        const float zi = ri * dinv[k];
-        Z[k] = zi;
-        d0.add_prod(ri, zi);
-        d1.add_prod(ri, ri);
-      }
-    });
-    const double a = block_sum_w0(d0.finish(), sh);
-    const double b = block_sum_w0(d1.finish(), sh);
-    if (threadIdx.x == 0) {
-      part[gb] = a;
-      part[stride + gb] = b;
-    }
-  }
-  if (batch_last_cta(&ctl->ticket_a)) {
-    __shared__ double tot[2 * MFTO_BATCH_MAX];
-    per_instance_sums<2>(part, stride, inst, count, false, tot);
-    __syncthreads();
-    for (int i = threadIdx.x; i < count; i += blockDim.x) {
-      BatchScal& s = sc[i];
-      s.rz = tot[2 * i];
-      s.rr = tot[2 * i + 1];
-      s.ff = s.rr;
-      s.rtol2ff = rtol * rtol * s.ff;
-      s.alpha = 0.0;
-      s.beta = rz_prev[i] > 0.0 ? s.rz / rz_prev[i] : 0.0;   // continued direction
-      s.it = 0;
-      s.status = MFTO_OK;
-      s.done = s.ff == 0.0 ? 1 : 0;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int all = 1;
-      for (int i = 0; i < count; ++i) all &= sc[i].done;
-      ctl->count = count;
-      ctl->maxit = maxit;
-      ctl->all_done = all;
-      ctl->ticket_a = 0u;
-    }
-  }
 }
 
 // outer FP64 residual: R32 = F - KU (zero for masked instances), r.r, f.f
@@ -520,6 +377,9 @@ batch_accumulate(double* __restrict__ U, const float* __restrict__ e, long long 
     U[i] += (double)e[i];
 }
 
+constexpr size_t kBatch64Smem =
+    FixShape<BatchShape64::CX, BatchShape64::CY, Col64LoadPlain, Col64Store>::kBytes;
+
 mfto_status bfail(mfto_batch* b, mfto_status code, const char* msg) {
   if (b) snprintf(b->msg, sizeof(b->msg), "%s", msg);
   return code;
@@ -547,17 +407,12 @@ mfto_status shape_attrs(mfto_batch* b) {
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem<double>()));
   BCUDA(b, cudaFuncSetAttribute(batch_kv_kernel<float, S>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem<float>()));
-  BCUDA(b, cudaFuncSetAttribute(batch_pcg_kv<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)batch_smem<float>()));
   BCUDA(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->occ_kv64[S], batch_kv_kernel<double, S>,
                                                          MFTO_BLOCK, batch_smem<double>()));
   BCUDA(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->occ_kv32[S], batch_kv_kernel<float, S>,
                                                          MFTO_BLOCK, batch_smem<float>()));
-  BCUDA(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->occ_pcg[S], batch_pcg_kv<S>,
-                                                         MFTO_BLOCK, batch_smem<float>()));
   if (b->occ_kv64[S] < 1) b->occ_kv64[S] = 1;
   if (b->occ_kv32[S] < 1) b->occ_kv32[S] = 1;
-  if (b->occ_pcg[S] < 1) b->occ_pcg[S] = 1;
   return MFTO_OK;
 }
 
@@ -578,17 +433,13 @@ mfto_status launch_kv(mfto_batch* b, int S, const T* E, const T* V, T* Y, cudaSt
   return MFTO_OK;
 }
 
-mfto_status launch_pcg_kv(mfto_batch* b, cudaStream_t st, const float* P0, float* P1) {
-  const int S = b->shape;
-  const unsigned grid = persistent_grid(b, b->occ_pcg[S], b->kv_total[S]);
-  const size_t smem = batch_smem<float>();
+// FP64 K.V: the fixed-point tiles where the operator fits, else the blocks of
+// the current shape.
+mfto_status launch_kv64(mfto_batch* b, const double* E, const double* V, double* Y) {
+  if (!b->fix_ok) return launch_kv<double>(b, b->shape, E, V, Y, b->stream, b->mc64);
   b->launches++;
-  switch (S) {
-    case 0: batch_pcg_kv<0><<<grid, MFTO_BLOCK, smem, st>>>(b->E32, b->z32, P0, P1, b->q32, b->d_fixed, b->mc32, b->d_inst[0], b->d_scal, b->d_ctl, b->d_part_a, b->kv_total[0]); break;
-    case 1: batch_pcg_kv<1><<<grid, MFTO_BLOCK, smem, st>>>(b->E32, b->z32, P0, P1, b->q32, b->d_fixed, b->mc32, b->d_inst[1], b->d_scal, b->d_ctl, b->d_part_a, b->kv_total[1]); break;
-    case 2: batch_pcg_kv<2><<<grid, MFTO_BLOCK, smem, st>>>(b->E32, b->z32, P0, P1, b->q32, b->d_fixed, b->mc32, b->d_inst[2], b->d_scal, b->d_ctl, b->d_part_a, b->kv_total[2]); break;
-    default: batch_pcg_kv<3><<<grid, MFTO_BLOCK, smem, st>>>(b->E32, b->z32, P0, P1, b->q32, b->d_fixed, b->mc32, b->d_inst[3], b->d_scal, b->d_ctl, b->d_part_a, b->kv_total[3]); break;
-  }
+  batch_kv_fixed<<<b->tiles64, BatchShape64::NT, kBatch64Smem, b->stream>>>(
+      E, V, Y, b->d_fixed, b->fix, b->d_inst[0], b->d_tiles64, b->d_tile64_inst);
   BCUDA(b, cudaGetLastError());
   return MFTO_OK;
 }
@@ -599,25 +450,29 @@ int part_stride(const mfto_batch* b) {
   return m;
 }
 
-mfto_status enqueue_chunk(mfto_batch* b, cudaStream_t st, int chunk) {
-  const unsigned ug = persistent_grid(b, 8, b->up_total);
+mfto_status enqueue_chunk(mfto_batch* b, cudaStream_t st, int chunk, double rtol, int maxit) {
   for (int it = 0; it < chunk; ++it) {
-    float* p_old = (it & 1) ? b->p1 : b->p0;
-    float* p_new = (it & 1) ? b->p0 : b->p1;
-    mfto_status s = launch_pcg_kv(b, st, p_old, p_new);
-    if (s != MFTO_OK) return s;
-    b->launches++;
-    batch_update<<<ug, MFTO_BLOCK, 0, st>>>(b->e32, p_new, b->q32, b->r32, b->z32, b->dinv32,
-                                            b->d_inst[b->shape], b->d_scal, b->d_ctl, b->d_part_b,
-                                            b->up_total, part_stride(b));
-    BCUDA(b, cudaGetLastError());
+    const int par = it & 1;
+    BatchScal* prev = b->d_scal + (par ^ 1) * b->count;
+    BatchScal* cur = b->d_scal + par * b->count;
+    float* p_old = par ? b->p1 : b->p0;
+    float* p_new = par ? b->p0 : b->p1;
+    const BatchCgArgs a{b->E32,     b->z32,         p_old, p_new, b->q32,       b->d_fixed,
+                        b->d_inst[0], b->d_tiles,   b->d_tile_inst, prev, cur, b->d_share_b,
+                        b->d_share_a, b->cg_updates, maxit, rtol * rtol};
+    batch_cg_kv<<<b->cg_tiles, MFTO_BLOCK, kBatchCgSmem, st>>>(a, b->mc32);
+    batch_cg_update<<<b->cg_updates, MFTO_BLOCK, 0, st>>>(
+        b->e32, p_new, b->q32, b->r32, b->z32, b->dinv32, b->d_inst[0], b->d_tiles, b->d_up_inst,
+        cur, b->d_share_a, b->d_share_b, b->cg_updates);
   }
+  batch_cg_done<<<1, MFTO_BLOCK, 0, st>>>(b->d_scal + b->count, b->count, &b->d_ctl->all_done);
+  BCUDA(b, cudaGetLastError());
   return MFTO_OK;
 }
 
-mfto_status get_graph(mfto_batch* b, BatchGraph** out) {
+mfto_status get_graph(mfto_batch* b, double rtol, int maxit, BatchGraph** out) {
   BatchGraph* g = b->graph;
-  if (g && g->chunk == b->p.check_every && g->shape == b->shape) {
+  if (g && g->chunk == b->p.check_every && g->maxit == maxit && g->rtol == rtol) {
     *out = g;
     return MFTO_OK;
   }
@@ -628,13 +483,12 @@ mfto_status get_graph(mfto_batch* b, BatchGraph** out) {
   }
   g = new BatchGraph();
   g->chunk = b->p.check_every;
-  g->shape = b->shape;
+  g->maxit = maxit;
+  g->rtol = rtol;
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) { delete g; return bfail(b, MFTO_CUDA_ERROR, "batch graph capture failed"); }
-  const int64_t l0 = b->launches;
-  mfto_status s = enqueue_chunk(b, b->cap_stream, g->chunk);
-  b->launches = l0;   // counted per graph launch instead
+  mfto_status s = enqueue_chunk(b, b->cap_stream, g->chunk, rtol, maxit);
   e = cudaStreamEndCapture(b->cap_stream, &graph);
   if (s != MFTO_OK || e != cudaSuccess) {
     if (graph) cudaGraphDestroy(graph);
@@ -675,6 +529,102 @@ mfto_status upload_inst(mfto_batch* b) {
   return MFTO_OK;
 }
 
+// Rows and z-chunks of every instance for a chunk length of about `layers`
+// node layers; the tile count.
+int plan_tiles(const mfto_batch* b, int layers, std::vector<BatchTiles>& out) {
+  out.resize(b->count);
+  int tile = 0, up = 0;
+  for (int i = 0; i < b->count; ++i) {
+    const mfto_mesh& m = b->meshes[i];
+    const int nx = m.nelx + 1, ny = m.nely + 1, nz = m.nelz + 1;
+    BatchTiles& t = out[i];
+    t.ntx = nx <= kBatchRow ? 1 : (nx + kBatchRow - 3) / (kBatchRow - 2);
+    t.ow = (nx + t.ntx - 1) / t.ntx;
+    t.c0 = t.ntx > 1 ? 1 : 0;                      // a halo column on each side where x is cut
+    t.w = t.ntx > 1 ? t.ow + 2 : nx;
+    const int most = MFTO_BLOCK / t.w - 1;         // owned rows, at most
+    t.nty = (ny + most - 1) / most;
+    t.rows = (ny + t.nty - 1) / t.nty + 1;
+    const int ntz = (nz + layers - 1) / layers;
+    t.nzc = (nz + ntz - 1) / ntz;
+    t.tile0 = tile;
+    t.ntile = t.ntx * t.nty * ((nz + t.nzc - 1) / t.nzc);
+    tile += t.ntile;
+    t.up0 = up;
+    t.nup = (int)((3ll * nx * ny * nz + kBatchUpdate - 1) / kBatchUpdate);
+    up += t.nup;
+  }
+  return tile;
+}
+
+// Tiles of the inner CG: the chunk length with the least time of the busiest
+// SM, a CTA taking its layers, the recomputed one and about two of start and
+// end.  FP64 tiles: whole columns cut into at most four chunks.
+mfto_status make_tiles(mfto_batch* b) {
+  std::vector<BatchTiles> t;
+  int best = 0, longest = 1;
+  double cost = 0.0;
+  for (const mfto_mesh& m : b->meshes) longest = longest > m.nelz + 1 ? longest : m.nelz + 1;
+  for (int layers = 1; layers <= longest; ++layers) {
+    const int n = plan_tiles(b, layers, t);
+    double work = 0.0;
+    int most = 0;
+    for (const BatchTiles& x : t) {
+      work += (double)x.ntile * (x.nzc + 3);
+      most = most > x.nzc ? most : x.nzc;
+    }
+    const double slots = 3.0 * b->num_sms;
+    const double c = n <= slots ? most + 3.0 : work / slots + 0.5 * (most + 3.0);
+    if (best == 0 || c < cost) {
+      cost = c;
+      best = layers;
+    }
+  }
+  b->cg_tiles = plan_tiles(b, best, t);
+  b->cg_updates = t.back().up0 + t.back().nup;
+  std::vector<int> tile_inst, up_inst, tile64_inst;
+  std::vector<BatchTiles64> t64(b->count);
+  for (int i = 0; i < b->count; ++i) {
+    tile_inst.insert(tile_inst.end(), t[i].ntile, i);
+    up_inst.insert(up_inst.end(), t[i].nup, i);
+    BatchTiles64& f = t64[i];
+    f.g = make_grid(b->meshes[i]);
+    f.tl.tx = (f.g.nx + BatchShape64::OX - 1) / BatchShape64::OX;
+    f.tl.ty = (f.g.ny + BatchShape64::OY - 1) / BatchShape64::OY;
+    const int tz = f.g.nz >= 32 ? 4 : (f.g.nz + 7) / 8;
+    f.tl.nzc = (f.g.nz + tz - 1) / tz;
+    f.tl.tz = (f.g.nz + f.tl.nzc - 1) / f.tl.nzc;
+    f.tile0 = (int)tile64_inst.size();
+    tile64_inst.insert(tile64_inst.end(), f.tl.count(), i);
+  }
+  b->tiles64 = (int)tile64_inst.size();
+  auto put = [&](void** d, const void* h, size_t bytes) -> mfto_status {
+    if (cudaMalloc(d, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return MFTO_OOM;
+    }
+    BCUDA(b, cudaMemcpy(*d, h, bytes, cudaMemcpyHostToDevice));
+    return MFTO_OK;
+  };
+  mfto_status s = put((void**)&b->d_tiles, t.data(), sizeof(BatchTiles) * t.size());
+  if (s == MFTO_OK) s = put((void**)&b->d_tiles64, t64.data(), sizeof(BatchTiles64) * t64.size());
+  if (s == MFTO_OK) s = put((void**)&b->d_tile_inst, tile_inst.data(), 4 * tile_inst.size());
+  if (s == MFTO_OK) s = put((void**)&b->d_up_inst, up_inst.data(), 4 * up_inst.size());
+  if (s == MFTO_OK)
+    s = put((void**)&b->d_tile64_inst, tile64_inst.data(), 4 * tile64_inst.size());
+  if (s != MFTO_OK) return s;
+  if (cudaMalloc(&b->d_share_a, sizeof(float2) * b->cg_tiles) != cudaSuccess ||
+      cudaMalloc(&b->d_share_b, sizeof(float2) * 2 * b->cg_updates) != cudaSuccess) {
+    cudaGetLastError();
+    return MFTO_OOM;
+  }
+  BCUDA(b, cudaFuncSetAttribute(batch_cg_kv, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kBatchCgSmem));
+  BCUDA(b, cudaFuncSetAttribute(batch_kv_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kBatch64Smem));
+  return MFTO_OK;
+}
+
 void free_batch(mfto_batch* b) {
   if (!b) return;
   if (b->graph) {
@@ -682,8 +632,9 @@ void free_batch(mfto_batch* b) {
     delete b->graph;
   }
   void* ptrs[] = {b->d_fixed, b->r32, b->z32, b->p0, b->p1, b->q32, b->e32, b->dinv32, b->E32,
-                  b->q64, b->d_scal, b->d_ctl, b->d_part_a, b->d_part_b, b->d_res, b->d_mask,
-                  b->d_rzp,
+                  b->q64, b->d_scal, b->d_ctl, b->d_part_a, b->d_res, b->d_mask, b->d_rzp,
+                  b->d_share_a, b->d_share_b, b->d_tiles, b->d_tiles64, b->d_tile_inst,
+                  b->d_up_inst, b->d_tile64_inst,
                   b->d_inst[0], b->d_inst[1], b->d_inst[2], b->d_inst[3]};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -760,10 +711,9 @@ extern "C" mfto_status mfto_batch_create(int32_t count, const mfto_mesh* meshes,
   A((void**)&b->dinv32, nd32);
   A((void**)&b->E32, sizeof(float) * b->n_elem);
   A((void**)&b->q64, sizeof(double) * b->n_dof);
-  A((void**)&b->d_scal, sizeof(BatchScal) * count);
+  A((void**)&b->d_scal, sizeof(BatchScal) * 2 * count);
   A((void**)&b->d_ctl, sizeof(BatchCtl));
   A((void**)&b->d_part_a, sizeof(double) * 2 * max_blocks);
-  A((void**)&b->d_part_b, sizeof(double) * 2 * max_blocks);
   A((void**)&b->d_res, sizeof(double) * 2 * count);
   A((void**)&b->d_rzp, sizeof(double) * count);
   A((void**)&b->d_mask, sizeof(int) * count);
@@ -781,10 +731,11 @@ extern "C" mfto_status mfto_batch_create(int32_t count, const mfto_mesh* meshes,
   if (s == MFTO_OK) s = shape_attrs<1>(b);
   if (s == MFTO_OK) s = shape_attrs<2>(b);
   if (s == MFTO_OK) s = shape_attrs<3>(b);
+  if (s == MFTO_OK) s = make_tiles(b);
   if (s != MFTO_OK) { free_batch(b); return s; }
   if (cudaMemcpyAsync(b->d_fixed, h_fixed, b->n_node, cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
       cudaMemsetAsync(b->d_ctl, 0, sizeof(BatchCtl), b->stream) != cudaSuccess ||
-      cudaMemsetAsync(b->d_scal, 0, sizeof(BatchScal) * count, b->stream) != cudaSuccess ||
+      cudaMemsetAsync(b->d_scal, 0, sizeof(BatchScal) * 2 * count, b->stream) != cudaSuccess ||
       cudaStreamSynchronize(b->stream) != cudaSuccess) {
     free_batch(b);
     return MFTO_CUDA_ERROR;
@@ -794,6 +745,7 @@ extern "C" mfto_status mfto_batch_create(int32_t count, const mfto_mesh* meshes,
   mfto_unit_ke(1.0, params->nu, b->h, ke);
   b->ke_diag = ke[0];
   mode_coefficients(params->nu, b->h, &b->mc64, &b->mc32);
+  b->fix_ok = fixed_op(params->nu, b->h, &b->fix);
   *out = b;
   return MFTO_OK;
 }
@@ -821,7 +773,7 @@ extern "C" mfto_status mfto_batch_kv(mfto_batch* b, mfto_form form, const void* 
   if (!b) return MFTO_INVALID_ARG;
   if (!E || !V || !Y || V == Y) return bfail(b, MFTO_INVALID_ARG, "mfto_batch_kv: bad pointers");
   if (form == MFTO_FORM_F64)
-    return launch_kv<double>(b, b->shape, (const double*)E, (const double*)V, (double*)Y, b->stream, b->mc64);
+    return launch_kv64(b, (const double*)E, (const double*)V, (double*)Y);
   if (form == MFTO_FORM_F32)
     return launch_kv<float>(b, b->shape, (const float*)E, (const float*)V, (float*)Y, b->stream, b->mc32);
   return bfail(b, MFTO_UNSUPPORTED, "mfto_batch_kv: forms F64 and F32 only");
@@ -896,7 +848,7 @@ extern "C" mfto_status mfto_batch_solve(mfto_batch* b, double inner_tol, const d
   for (int outer = 0;; ++outer) {
     BCUDA(b, cudaMemcpyAsync(b->d_mask, mask.data(), sizeof(int) * count, cudaMemcpyHostToDevice,
                              b->stream));
-    mfto_status s = launch_kv<double>(b, b->shape, E, U, b->q64, b->stream, b->mc64);
+    mfto_status s = launch_kv64(b, E, U, b->q64);
     if (s != MFTO_OK) return s;
     b->launches++;
     batch_residual<<<ug, MFTO_BLOCK, 0, b->stream>>>(F, b->q64, b->r32, b->d_mask,
@@ -953,22 +905,21 @@ extern "C" mfto_status mfto_batch_solve(mfto_batch* b, double inner_tol, const d
     BCUDA(b, cudaMemcpyAsync(b->d_rzp, rzp.data(), sizeof(double) * count, cudaMemcpyHostToDevice,
                              b->stream));
     b->launches++;
-    batch_init<<<ug, MFTO_BLOCK, 0, b->stream>>>(b->r32, b->z32, b->dinv32, b->d_inst[b->shape],
-                                                 b->d_scal, b->d_ctl, b->d_part_a, b->up_total,
-                                                 stride, inner_tol, inner_maxit, count, b->d_rzp);
+    batch_cg_start<<<b->cg_updates, MFTO_BLOCK, 0, b->stream>>>(
+        b->r32, b->z32, b->dinv32, b->d_inst[0], b->d_tiles, b->d_up_inst, b->d_scal + count,
+        b->d_rzp, b->d_share_b, b->cg_updates);
     BCUDA(b, cudaGetLastError());
     BatchGraph* g = nullptr;
-    s = get_graph(b, &g);
+    s = get_graph(b, inner_tol, inner_maxit, &g);
     if (s != MFTO_OK) return s;
-    for (;;) {
+    do {
+      BCUDA(b, cudaGraphLaunch(g->exec, b->stream));
+      b->launches += 2 * (int64_t)g->chunk + 1;
       BCUDA(b, cudaMemcpyAsync(b->h_ctl, b->d_ctl, sizeof(BatchCtl), cudaMemcpyDeviceToHost,
                                b->stream));
       BCUDA(b, cudaStreamSynchronize(b->stream));
-      if (b->h_ctl->all_done) break;
-      BCUDA(b, cudaGraphLaunch(g->exec, b->stream));
-      b->launches += 2 * (int64_t)g->chunk;
-    }
-    BCUDA(b, cudaMemcpyAsync(b->h_scal, b->d_scal, sizeof(BatchScal) * count,
+    } while (!b->h_ctl->all_done);
+    BCUDA(b, cudaMemcpyAsync(b->h_scal, b->d_scal + count, sizeof(BatchScal) * count,
                              cudaMemcpyDeviceToHost, b->stream));
     BCUDA(b, cudaStreamSynchronize(b->stream));
     for (int i = 0; i < count; ++i) {
