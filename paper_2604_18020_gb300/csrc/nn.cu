@@ -15,6 +15,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <random>
 #include <string>
 #include <vector>
@@ -323,38 +324,63 @@ unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
 //
 // out[co][v] = b[co] + sum_ci sum_k w[co][ci][k] in[ci][v + d_k] as the GEMM
 // D[128 voxels x N] = sum_k sum_ci A_k[voxel][ci] B_k[ci][co], N = a slice of
-// NS output channels, accumulated in FP32 in tensor memory.  A CTA computes an
-// output tile of 8 (x) x 16 (y) voxels of one z-plane (M = 128) and stages its
-// input halo tile, 10 x 18 x 3 voxels, 16 input channels at a time, as BF16 in
-// the canonical no-swizzle K-major layout: one 16-byte row per (voxel, 8
-// channels).  For tap (dx, dy, dz) the A operand is that staged tile read in
-// place: the core-matrix rows of output voxels x = 0..7 of one y-row are the
-// staged voxels x + dx of y-row y + dy (consecutive, 16 bytes apart), the
-// 8-row groups step one staged y-row (SBO = 160 bytes) and the two 8-channel
-// halves of the K = 16 step sit one channel part apart (LBO).  The FP32
-// activations are split into BF16 hi + lo (two products against the same
-// BF16 weights), so the result carries the activations to about 2^-16 and
-// the weights as stored.  Per stage one thread issues 27 taps x 2 parts
-// MMAs (M = 128, N = NS, K = 16), commits them to an mbarrier (bounded wait),
-// and the CTA stages the next 16 channels after they completed; three CTAs
-// per SM overlap one another's staging and MMAs.  The epilogue reads each
-// voxel's row of D with tcgen05.ld and writes bias + ReLU in FP32 (bias may
-// be NULL; with gate given, outputs whose gate value is not positive are
-// zero: the ReLU adjoint of the data gradient, which runs through this
-// kernel with the adjoint weights of pack_w3).
+// NS output channels, accumulated in FP32 in tensor memory.  A CTA computes
+// output tiles of 8 (x) x 16 (y) voxels (M = 128) of up to kCtZ consecutive
+// z-planes, each with its own NS columns of tensor memory, and streams the
+// input planes past them: per 16 input channels it loads the weights once,
+// then stages one halo plane of 10 x 18 voxels after the other, and each feeds
+// the outputs of the plane below (dz = +1), its own and the one above.  A plane
+// is staged once per chunk instead of once for each of its three outputs, and
+// the weights once per chunk instead of once per output plane.
+//
+// Staged plane: BF16 in the canonical no-swizzle K-major layout, one 16-byte
+// row per (voxel, 8 channels).  For tap (dx, dy) the A operand is that plane
+// read in place: the core-matrix rows of output voxels x = 0..7 of one y-row
+// are the staged voxels x + dx of y-row y + dy (consecutive, 16 bytes apart),
+// the 8-row groups step one staged y-row (SBO = 160 bytes) and the two
+// 8-channel halves of the K = 16 step sit one channel part apart (LBO).  The
+// FP32 activations are split into BF16 hi + lo (two products against the same
+// BF16 weights), so the result carries the activations to about 2^-16 and the
+// weights as stored.
+//
+// Four warps stage planes into two buffers while a fifth warp's lane issues the
+// MMAs (M = 128, N = NS, K = 16; 9 taps x 2 parts for each of up to 3 outputs)
+// of the last: a plane's 128 stagers arrive on its "full" mbarrier, the MMAs'
+// commit on its "empty" one (all waits bounded).  Up to four CTAs share an SM
+// (shared memory and 128 tensor-memory columns each).  The epilogue (the four
+// staging warps) reads each voxel's row of D with tcgen05.ld and writes bias +
+// ReLU in FP32 (bias may be NULL; with gate given, outputs whose gate value is
+// not positive are zero: the ReLU adjoint of the data gradient, which runs
+// through this kernel with the adjoint weights of pack_w3).  An output's
+// products are added in the order of stage, dz, dy, dx, part.
+//
+// Bound by the MMAs' reads of A from shared memory: an MMA of 128 x 16 x NS
+// products takes 38 clocks of an SM (NS = 16 and 32 alike) for 4 KB of A.
+// Measured on a GB300 against one plane at a time, its three halo planes staged
+// anew and the CTA waiting for its MMAs: the network's forward pass on 136 x 72 x
+// 72 nodes 994 against 1,442 us, loss and gradient on 72 x 40 x 40 1,951 against
+// 2,170 us; the same bits.
 constexpr int kCtTX = 8, kCtTY = 16;                  // output tile (M = 128)
-constexpr int kCtHX = kCtTX + 2, kCtHY = kCtTY + 2;   // staged halo tile, 3 z-planes
-constexpr int kCtPos = kCtHX * kCtHY * 3;             // 540 staged voxels
-constexpr int kCtPart = kCtPos * 16;                  // one 8-channel part: 8,640 bytes
+constexpr int kCtHX = kCtTX + 2, kCtHY = kCtTY + 2;   // staged halo plane
+constexpr int kCtPart = kCtHX * kCtHY * 16;           // one 8-channel part: 2,880 bytes
 constexpr int kCtA = 4 * kCtPart;                     // hi 0-7, hi 8-15, lo 0-7, lo 8-15
 constexpr int kCtCin = 16;                            // input channels per stage
+constexpr int kCtCols = 128;                          // TMEM columns of a CTA
+constexpr int kCtPerSm = 4;                           // CTAs an SM holds
+constexpr int kCtThreads = 160;                       // four staging warps, one for the MMAs
 constexpr uint32_t kCtSpin = 1u << 20;                // bound of the mbarrier wait
 template <int NS>
 struct CtShape {
   static constexpr int B = 27 * 2 * (NS / 8) * 128;   // packed weights of one stage
-  static constexpr int COLS = NS < 32 ? 32 : NS;      // TMEM columns (allocation >= 32)
-  static constexpr int SMEM = kCtA + B + 128 + 128;   // + mbarrier / TMEM slot + alignment
+  static constexpr int Z = kCtCols / NS;              // output planes of a chunk, at most
+  // two planes, weights, mbarriers and the TMEM slot, alignment; at least
+  // what keeps a fifth CTA (and its TMEM columns) off the SM
+  static constexpr int USED = 2 * kCtA + B + 128 + 128;
+  static constexpr int SMEM = USED > 48 * 1024 ? USED : 48 * 1024;
 };
+static_assert(5 * CtShape<16>::SMEM > 228 * 1024 && 5 * CtShape<32>::SMEM > 228 * 1024 &&
+                  kCtPerSm * kCtCols <= 512,
+              "the resident CTAs' TMEM columns fit");
 
 // Packed weights of one 3x3x3 layer, slice by slice (NS output channels) and
 // stage by stage (16 input channels): [tap 27][kc 2][ng NS/8][r 8][c 8] BF16,
@@ -384,161 +410,216 @@ __global__ void pack_w3(const __nv_bfloat16* __restrict__ w, int Cin, int Cout, 
   out[i] = (co < Cout && ci < Cin) ? w[src] : __float2bfloat16_rn(0.f);
 }
 
+// polls an mbarrier's phase, bounded; backs off between polls: the other warps
+// of the SM need the issue slots
+__device__ __forceinline__ void ct_poll(uint64_t* bar, uint32_t parity, int32_t* err) {
+  uint32_t spins = 0;
+  bool ok;
+  while (!(ok = mbar_try_wait(bar, parity))) {
+    if (++spins > kCtSpin) break;
+    __nanosleep(32);
+  }
+  if (!ok) {
+    atomicExch(err, 1);
+    for (uint32_t s2 = 0; s2 < kCtSpin && !mbar_try_wait(bar, parity); ++s2) {
+    }
+  }
+}
+// one lane per warp polls; the warp barrier and the fence order the rest
+__device__ __forceinline__ void ct_wait(uint64_t* bar, uint32_t parity, int32_t* err) {
+  if ((threadIdx.x & 31) == 0) ct_poll(bar, parity, err);
+  __syncwarp();
+  tc_fence_after();
+}
+
+// the nine taps (dy, dx) of one output, activations hi and lo
 template <int NS>
-__global__ void __launch_bounds__(128)
+__device__ __forceinline__ void ct_taps(uint32_t dcol, uint64_t ad, uint64_t bd, bool first) {
+  constexpr uint32_t IDESC = make_idesc(1u, 128, NS);
+#pragma unroll
+  for (int tap = 0; tap < 9; ++tap)
+#pragma unroll
+    for (int part = 0; part < 2; ++part) {
+      // descriptors count 16 bytes
+      constexpr int kTapB = 2 * (NS / 8) * 128 / 16;
+      const int aoff = (tap / 3) * kCtHX + tap % 3 + part * (2 * kCtPart / 16);
+      mma_f16(dcol, ad + (uint64_t)aoff, bd + (uint64_t)(tap * kTapB), IDESC,
+              first && tap == 0 && part == 0 ? 0u : 1u);
+    }
+}
+
+template <int NS>
+__global__ void __launch_bounds__(kCtThreads, kCtPerSm)
 conv3_tc(const float* __restrict__ in, int Cin, const __nv_bfloat16* __restrict__ wp,
          const float* __restrict__ bias, float* __restrict__ out, int Cout, Dims d, int relu,
-         const float* __restrict__ gate, int tiles_x, int tiles_y, int32_t* err) {
+         const float* __restrict__ gate, int tiles_x, int tiles_y, int zc, int32_t* err) {
   using C = CtShape<NS>;
   extern __shared__ __align__(16) unsigned char ct_raw[];
   unsigned char* As = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(ct_raw) + 127) & ~(uintptr_t)127);
-  unsigned char* Bs = As + kCtA;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(Bs + C::B);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(Bs + C::B + 8);
+  unsigned char* Bs = As + 2 * kCtA;
+  uint64_t* full = reinterpret_cast<uint64_t*>(Bs + C::B);   // [2], one per plane buffer
+  uint64_t* empty = full + 2;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(Bs + C::B + 32);
   const int tid = threadIdx.x, warp = tid >> 5;
   const int slice = blockIdx.y;
   const int S = (Cin + kCtCin - 1) / kCtCin;
-  const int ntiles = tiles_x * tiles_y * d.D;
+  const int nchunk = (d.D + zc - 1) / zc;
+  const int ntiles = tiles_x * tiles_y * nchunk;
   const size_t V = (size_t)d.V();
   if (warp == 0) {
-    tmem_alloc(tslot, C::COLS);
+    tmem_alloc(tslot, kCtCols);
     tmem_relinquish();
   }
   if (tid == 0) {
-    mbar_init(bar, 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(full + b, 128);
+      mbar_init(empty + b, 1);
+    }
     mbar_init_fence();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
-  const uint32_t a_addr = smem_u32(As), b_addr = smem_u32(Bs);
-  constexpr uint32_t IDESC = make_idesc(1u, 128, NS);
-  uint32_t phase = 0;
-  // staging assignment, the same for every tile and stage: thread t < 120
-  // owns staged column xx = t % 10 of rows r = t / 10 + 12 k (row r = z-plane
-  // r / 18, y-row r % 18 of the halo tile), for both 8-channel groups
-  const bool stager = tid < 120;
-  const int xx = tid % kCtHX, r0 = tid / kCtHX;
-  auto stage_b = [&](int s) {
-    const uint4* src = reinterpret_cast<const uint4*>(wp) + ((size_t)slice * S + s) * (C::B / 16);
-    uint4* dst = reinterpret_cast<uint4*>(Bs);
-    for (int i = tid; i < C::B / 16; i += 128) dst[i] = src[i];
-  };
-  if (S == 1) stage_b(0);   // one stage: the weights stay for every tile
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int tx = t % tiles_x, ty = (t / tiles_x) % tiles_y, z = t / (tiles_x * tiles_y);
-    const int x0 = tx * kCtTX, y0 = ty * kCtTY;
-    const int gx = x0 - 1 + xx;
-    const bool xin = gx >= 0 && gx < d.W;
-    for (int s = 0; s < S; ++s) {
-      if (stager) {
-#pragma unroll 2
-        for (int r = r0; r < 3 * kCtHY; r += 12) {
-          const int zz = r / kCtHY, yy = r - zz * kCtHY;
-          const int gy = y0 - 1 + yy, gz = z - 1 + zz;
-          const bool inside = xin && gy >= 0 && gz >= 0 && gy < d.H && gz < d.D;
-          const size_t vox = inside ? ((size_t)gz * d.H + gy) * d.W + gx : 0;
-          const int pos = r * kCtHX + xx;
-#pragma unroll
-          for (int g = 0; g < 2; ++g) {
-            const int c0 = s * kCtCin + 8 * g;
-            const float* p = in + (size_t)c0 * V + vox;
-            float v[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) v[c] = (inside && c0 + c < Cin) ? p[(size_t)c * V] : 0.f;
-            uint32_t hi[4], lo[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
-              const float2 hf = __bfloat1622float2(h);
-              const __nv_bfloat162 l = __floats2bfloat162_rn(v[2 * q] - hf.x, v[2 * q + 1] - hf.y);
-              hi[q] = *reinterpret_cast<const uint32_t*>(&h);
-              lo[q] = *reinterpret_cast<const uint32_t*>(&l);
-            }
-            *reinterpret_cast<uint4*>(As + g * kCtPart + pos * 16) =
-                make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            *reinterpret_cast<uint4*>(As + (2 + g) * kCtPart + pos * 16) =
-                make_uint4(lo[0], lo[1], lo[2], lo[3]);
-          }
-        }
-      }
-      if (S > 1) stage_b(s);
-      fence_proxy_async_smem();
-      tc_fence_before();
-      __syncthreads();
-      if (tid == 0) {
-        tc_fence_after();
+  uint32_t n = 0;           // planes so far: buffer n & 1, its use n >> 1
+  if (warp == 4) {
+    // the MMAs of every plane, in the order in which it is staged
+    if ((tid & 31) == 0) {
+      const uint32_t a_addr = smem_u32(As), b_addr = smem_u32(Bs);
+      const uint64_t bd0 = smem_desc(b_addr, (NS / 8) * 128, 128);
+      for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const int ch = t / (tiles_x * tiles_y);
+        const int z0 = ch * zc, z1 = min(z0 + zc, d.D);
+        const int p0 = max(z0 - 1, 0), p1 = min(z1 + 1, d.D);
+        for (int s = 0; s < S; ++s)
+          for (int p = p0; p < p1; ++p, ++n) {
+            ct_poll(full + (n & 1), (n >> 1) & 1, err);
+            tc_fence_after();
+            const uint64_t ad = smem_desc(a_addr + (n & 1) * kCtA, kCtPart, kCtHX * 16);
+            // outputs z = p + 1, p, p - 1, to which this plane is dz = 0, 1, 2;
+            // an output's first plane overwrites (plane -1 does not exist)
 #pragma unroll 1
-        for (int tap = 0; tap < 27; ++tap) {
-          const int dx = tap % 3, dy = (tap / 3) % 3, dz = tap / 9;
-          const uint32_t aoff = (uint32_t)(((dz * kCtHY + dy) * kCtHX + dx) * 16);
-          const uint64_t bd = smem_desc(b_addr + tap * (2 * (NS / 8) * 128), (NS / 8) * 128, 128);
-#pragma unroll
-          for (int part = 0; part < 2; ++part) {   // activations hi, lo
-            const uint64_t ad = smem_desc(a_addr + part * 2 * kCtPart + aoff, kCtPart, kCtHX * 16);
-            mma_f16(tmem, ad, bd, IDESC, (s | tap | part) ? 1u : 0u);
+            for (int dz = 0; dz < 3; ++dz) {
+              const int z = p + 1 - dz;
+              if (z < z0 || z >= z1) continue;
+              ct_taps<NS>(tmem + (uint32_t)((z - z0) * NS), ad,
+                          bd0 + (uint64_t)(dz * 9 * (2 * (NS / 8) * 128 / 16)),
+                          s == 0 && (dz == 0 || (dz == 1 && z == 0)));
+            }
+            mma_commit(empty + (n & 1));
           }
-        }
-        mma_commit(bar);
-      }
-      // the next stage (or tile) rewrites A and B, the epilogue reads D: wait
-      // for these MMAs (one lane per warp polls; the warp barrier and the
-      // fence order the rest of the warp)
-      if ((tid & 31) == 0) {
-        uint32_t spins = 0;
-        bool ok;
-        // back off between polls: the other CTAs of the SM need the issue
-        // slots for their staging while these MMAs run
-        while (!(ok = mbar_try_wait(bar, phase))) {
-          if (++spins > kCtSpin) break;
-          __nanosleep(128);
-        }
-        if (!ok) {
-          atomicExch(err, 1);
-          for (uint32_t s2 = 0; s2 < kCtSpin && !mbar_try_wait(bar, phase); ++s2) {
-          }
-        }
-      }
-      __syncwarp();
-      phase ^= 1u;
-      tc_fence_after();
-    }
-    // epilogue: thread tid holds TMEM lane tid = output voxel (x0 + tid % 8, y0 + tid / 8)
-    float acc[NS];
-    const uint32_t lane_addr = tmem + ((uint32_t)(32 * warp) << 16);
-    if constexpr (NS == 16) {
-      tmem_ld16(lane_addr, acc);
-    } else {
-#pragma unroll
-      for (int h = 0; h < NS / 32; ++h) {
-        float part[32];
-        tmem_ld32(lane_addr + 32 * h, part);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc[32 * h + j] = part[j];
       }
     }
-    tc_fence_before();   // the next tile's first MMA overwrites D after the next barrier
-    const int ox = x0 + (tid & 7), oy = y0 + (tid >> 3);
-    if (ox < d.W && oy < d.H) {
-      const size_t vox = ((size_t)z * d.H + oy) * d.W + ox;
+    __syncwarp();
+  } else {
+    // staging assignment, the same for every plane: thread t < 120 owns staged
+    // column xx = t % 10 of y-rows t / 10 and t / 10 + 12, for both 8-channel
+    // groups
+    const bool stager = tid < 120;
+    const int xx = tid % kCtHX, r0 = tid / kCtHX;
+    auto stage_b = [&](int s) {
+      const uint4* src =
+          reinterpret_cast<const uint4*>(wp) + ((size_t)slice * S + s) * (C::B / 16);
+      uint4* dst = reinterpret_cast<uint4*>(Bs);
+      for (int i = tid; i < C::B / 16; i += 128) dst[i] = src[i];
+    };
+    if (S == 1) stage_b(0);   // one stage: the weights stay for every tile
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      const int tx = t % tiles_x, ty = (t / tiles_x) % tiles_y, ch = t / (tiles_x * tiles_y);
+      const int x0 = tx * kCtTX, y0 = ty * kCtTY;
+      const int z0 = ch * zc, z1 = min(z0 + zc, d.D);       // output planes [z0, z1)
+      const int p0 = max(z0 - 1, 0), p1 = min(z1 + 1, d.D);  // input planes [p0, p1)
+      const int gx = x0 - 1 + xx;
+      const bool xin = gx >= 0 && gx < d.W;
+      for (int s = 0; s < S; ++s) {
+        for (int p = p0; p < p1; ++p, ++n) {
+          // a plane's values are requested before the wait for its buffer
+          float v[2][2][8];
 #pragma unroll
-      for (int j = 0; j < NS; ++j) {
-        const int co = slice * NS + j;
-        if (co < Cout) {
-          float r = bias ? acc[j] + bias[co] : acc[j];
-          if (relu) r = fmaxf(r, 0.f);
-          if (gate && !(gate[(size_t)co * V + vox] > 0.f)) r = 0.f;
-          out[(size_t)co * V + vox] = r;
+          for (int h = 0; h < 2; ++h) {
+            const int yy = r0 + 12 * h, gy = y0 - 1 + yy;
+            const bool inside = stager && yy < kCtHY && xin && gy >= 0 && gy < d.H;
+            const size_t vox = inside ? ((size_t)p * d.H + gy) * d.W + gx : 0;
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+              const int c0 = s * kCtCin + 8 * g;
+              const float* q = in + (size_t)c0 * V + vox;
+#pragma unroll
+              for (int c = 0; c < 8; ++c)
+                v[h][g][c] = (inside && c0 + c < Cin) ? q[(size_t)c * V] : 0.f;
+            }
+          }
+          // the buffer is free when the MMAs of its last use are done; the
+          // weights when those of every plane so far are
+          if (S > 1 && p == p0) {
+            if (n >= 1) ct_wait(empty + ((n - 1) & 1), ((n - 1) >> 1) & 1, err);
+            stage_b(s);
+          } else if (n >= 2) {
+            ct_wait(empty + (n & 1), ((n >> 1) - 1) & 1, err);
+          }
+          unsigned char* Ap = As + (n & 1) * kCtA;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int yy = r0 + 12 * h;
+            if (stager && yy < kCtHY) {
+              const int pos = yy * kCtHX + xx;
+#pragma unroll
+              for (int g = 0; g < 2; ++g) {
+                uint32_t hi[4], lo[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  const float a = v[h][g][2 * k], b = v[h][g][2 * k + 1];
+                  const __nv_bfloat162 b2 = __floats2bfloat162_rn(a, b);
+                  const float2 hf = __bfloat1622float2(b2);
+                  const __nv_bfloat162 l2 = __floats2bfloat162_rn(a - hf.x, b - hf.y);
+                  hi[k] = *reinterpret_cast<const uint32_t*>(&b2);
+                  lo[k] = *reinterpret_cast<const uint32_t*>(&l2);
+                }
+                *reinterpret_cast<uint4*>(Ap + g * kCtPart + pos * 16) =
+                    make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                *reinterpret_cast<uint4*>(Ap + (2 + g) * kCtPart + pos * 16) =
+                    make_uint4(lo[0], lo[1], lo[2], lo[3]);
+              }
+            }
+          }
+          fence_proxy_async_smem();
+          tc_fence_before();   // the epilogue's reads of D come before the next MMAs
+          mbar_arrive(full + (n & 1));
         }
+      }
+      ct_wait(empty + ((n - 1) & 1), ((n - 1) >> 1) & 1, err);
+      // epilogue: thread tid holds TMEM lane tid = output voxel (x0 + tid % 8, y0 + tid / 8)
+      const int ox = x0 + (tid & 7), oy = y0 + (tid >> 3);
+      for (int z = z0; z < z1; ++z) {
+        float acc[NS];
+        const uint32_t lane_addr =
+            tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)((z - z0) * NS);
+        if constexpr (NS == 16)
+          tmem_ld16(lane_addr, acc);
+        else
+          tmem_ld32(lane_addr, acc);
+        if (ox < d.W && oy < d.H) {
+          const size_t vox = ((size_t)z * d.H + oy) * d.W + ox;
+#pragma unroll
+          for (int j = 0; j < NS; ++j) {
+            const int co = slice * NS + j;
+            if (co < Cout) {
+              float r = bias ? acc[j] + bias[co] : acc[j];
+              if (relu) r = fmaxf(r, 0.f);
+              if (gate && !(gate[(size_t)co * V + vox] > 0.f)) r = 0.f;
+              out[(size_t)co * V + vox] = r;
+            }
+          }
+        }
+        __syncwarp();
       }
     }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 0) tmem_dealloc(tmem, C::COLS);
+  if (warp == 0) tmem_dealloc(tmem, kCtCols);
 }
 
 // output-channel slice of a layer: 16 for at most 16 channels, else 32
@@ -620,18 +701,30 @@ mfto_status conv3_tc_launch(mfto_nn* n, const float* in, int cin, const __nv_bfl
                             const float* gate) {
   const int ns = ct_ns(cout);
   const int tiles_x = (d.W + kCtTX - 1) / kCtTX, tiles_y = (d.H + kCtTY - 1) / kCtTY;
-  // persistent CTAs: as many as fit on the GPU (shared memory: 4 per SM for
-  // 16-channel slices, 3 for 32), at most one per tile
-  const size_t tiles = (size_t)tiles_x * tiles_y * d.D;
-  const size_t fit = (size_t)n->num_sms * (ns == 16 ? 4 : 3);
-  const dim3 grid((unsigned)(tiles < fit ? tiles : fit), (unsigned)((cout + ns - 1) / ns));
+  // persistent CTAs, at most as many as fit; chunks of zc planes: the waves
+  // of CTAs times a chunk's MMAs (zc planes), its staging (zc + 2, about 0.6 of
+  // a plane's MMAs each) and its start and end
+  const int slices = (cout + ns - 1) / ns, most = ns == 16 ? CtShape<16>::Z : CtShape<32>::Z;
+  const int64_t fit = std::max<int64_t>(1, (int64_t)n->num_sms * kCtPerSm / slices);
+  int zc = 1;
+  double best = 0.0;
+  for (int z = 1; z <= most && z <= d.D; ++z) {
+    const int64_t items = (int64_t)tiles_x * tiles_y * ((d.D + z - 1) / z);
+    const double cost = (double)((items + fit - 1) / fit) * (z + 0.6 * (z + 2) + 1.0);
+    if (best == 0.0 || cost < best) {
+      best = cost;
+      zc = z;
+    }
+  }
+  const int64_t items = (int64_t)tiles_x * tiles_y * ((d.D + zc - 1) / zc);
+  const dim3 grid((unsigned)std::min(items, fit), (unsigned)slices);
   n->launches++;
   if (ns == 16)
-    conv3_tc<16><<<grid, 128, CtShape<16>::SMEM, n->stream>>>(in, cin, wp, bias, out, cout, d, relu,
-                                                              gate, tiles_x, tiles_y, n->d_err);
+    conv3_tc<16><<<grid, kCtThreads, CtShape<16>::SMEM, n->stream>>>(in, cin, wp, bias, out, cout, d, relu,
+                                                              gate, tiles_x, tiles_y, zc, n->d_err);
   else
-    conv3_tc<32><<<grid, 128, CtShape<32>::SMEM, n->stream>>>(in, cin, wp, bias, out, cout, d, relu,
-                                                              gate, tiles_x, tiles_y, n->d_err);
+    conv3_tc<32><<<grid, kCtThreads, CtShape<32>::SMEM, n->stream>>>(in, cin, wp, bias, out, cout, d, relu,
+                                                              gate, tiles_x, tiles_y, zc, n->d_err);
   NCUDA(n, cudaGetLastError());
   return MFTO_OK;
 }
