@@ -343,7 +343,8 @@ unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
 // BF16 weights), so the result carries the activations to about 2^-16 and the
 // weights as stored.
 //
-// Four warps stage planes into two buffers while a fifth warp's lane issues the
+// The next 16 channels' weights are copied asynchronously into a second buffer
+// meanwhile.  Four warps stage planes into two buffers while a fifth warp's lane issues the
 // MMAs (M = 128, N = NS, K = 16; 9 taps x 2 parts for each of up to 3 outputs)
 // of the last: a plane's 128 stagers arrive on its "full" mbarrier, the MMAs'
 // commit on its "empty" one (all waits bounded).  Up to four CTAs share an SM
@@ -358,8 +359,8 @@ unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
 // products takes 38 clocks of an SM (NS = 16 and 32 alike) for 4 KB of A.
 // Measured on a GB300 against one plane at a time, its three halo planes staged
 // anew and the CTA waiting for its MMAs: the network's forward pass on 136 x 72 x
-// 72 nodes 994 against 1,442 us, loss and gradient on 72 x 40 x 40 1,951 against
-// 2,170 us; the same bits.
+// 72 nodes 944 against 1,442 us (994 with one weight buffer), loss and gradient
+// on 72 x 40 x 40 1,723 against 2,170 us (1,951); the same bits.
 constexpr int kCtTX = 8, kCtTY = 16;                  // output tile (M = 128)
 constexpr int kCtHX = kCtTX + 2, kCtHY = kCtTY + 2;   // staged halo plane
 constexpr int kCtPart = kCtHX * kCtHY * 16;           // one 8-channel part: 2,880 bytes
@@ -373,12 +374,18 @@ template <int NS>
 struct CtShape {
   static constexpr int B = 27 * 2 * (NS / 8) * 128;   // packed weights of one stage
   static constexpr int Z = kCtCols / NS;              // output planes of a chunk, at most
-  // two planes, weights, mbarriers and the TMEM slot, alignment; at least
-  // what keeps a fifth CTA (and its TMEM columns) off the SM
-  static constexpr int USED = 2 * kCtA + B + 128 + 128;
-  static constexpr int SMEM = USED > 48 * 1024 ? USED : 48 * 1024;
+  // two planes, the weights of one stage or two, mbarriers and the TMEM slot,
+  // alignment; at least what keeps a fifth CTA (and its TMEM columns) off the SM
+  static constexpr int smem(int stages) {
+    const int used = 2 * kCtA + (stages > 1 ? 2 : 1) * B + 128 + 128;
+    return used > 48 * 1024 ? used : 48 * 1024;
+  }
+  static constexpr int per_sm(int stages) {
+    const int fit = 227 * 1024 / (smem(stages) + 1024);
+    return fit < kCtPerSm ? fit : kCtPerSm;
+  }
 };
-static_assert(5 * CtShape<16>::SMEM > 228 * 1024 && 5 * CtShape<32>::SMEM > 228 * 1024 &&
+static_assert(5 * CtShape<16>::smem(1) > 228 * 1024 && 5 * CtShape<32>::smem(1) > 228 * 1024 &&
                   kCtPerSm * kCtCols <= 512,
               "the resident CTAs' TMEM columns fit");
 
@@ -458,9 +465,10 @@ conv3_tc(const float* __restrict__ in, int Cin, const __nv_bfloat16* __restrict_
   unsigned char* As = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(ct_raw) + 127) & ~(uintptr_t)127);
   unsigned char* Bs = As + 2 * kCtA;
-  uint64_t* full = reinterpret_cast<uint64_t*>(Bs + C::B);   // [2], one per plane buffer
+  // [2], one per plane buffer, behind the weights (a second buffer with S > 1)
+  uint64_t* full = reinterpret_cast<uint64_t*>(Bs + (Cin > kCtCin ? 2 : 1) * C::B);
   uint64_t* empty = full + 2;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(Bs + C::B + 32);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(full + 4);
   const int tid = threadIdx.x, warp = tid >> 5;
   const int slice = blockIdx.y;
   const int S = (Cin + kCtCin - 1) / kCtCin;
@@ -483,6 +491,7 @@ conv3_tc(const float* __restrict__ in, int Cin, const __nv_bfloat16* __restrict_
   tc_fence_after();
   const uint32_t tmem = *tslot;
   uint32_t n = 0;           // planes so far: buffer n & 1, its use n >> 1
+  uint32_t w = 0;           // stages so far: weight buffer w & 1 (S > 1)
   if (warp == 4) {
     // the MMAs of every plane, in the order in which it is staged
     if ((tid & 31) == 0) {
@@ -492,7 +501,8 @@ conv3_tc(const float* __restrict__ in, int Cin, const __nv_bfloat16* __restrict_
         const int ch = t / (tiles_x * tiles_y);
         const int z0 = ch * zc, z1 = min(z0 + zc, d.D);
         const int p0 = max(z0 - 1, 0), p1 = min(z1 + 1, d.D);
-        for (int s = 0; s < S; ++s)
+        for (int s = 0; s < S; ++s, ++w) {
+          const uint64_t bd = bd0 + (uint64_t)((S > 1 ? w & 1 : 0) * (C::B / 16));
           for (int p = p0; p < p1; ++p, ++n) {
             ct_poll(full + (n & 1), (n >> 1) & 1, err);
             tc_fence_after();
@@ -504,11 +514,12 @@ conv3_tc(const float* __restrict__ in, int Cin, const __nv_bfloat16* __restrict_
               const int z = p + 1 - dz;
               if (z < z0 || z >= z1) continue;
               ct_taps<NS>(tmem + (uint32_t)((z - z0) * NS), ad,
-                          bd0 + (uint64_t)(dz * 9 * (2 * (NS / 8) * 128 / 16)),
+                          bd + (uint64_t)(dz * 9 * (2 * (NS / 8) * 128 / 16)),
                           s == 0 && (dz == 0 || (dz == 1 && z == 0)));
             }
             mma_commit(empty + (n & 1));
           }
+        }
       }
     }
     __syncwarp();
@@ -518,13 +529,21 @@ conv3_tc(const float* __restrict__ in, int Cin, const __nv_bfloat16* __restrict_
     // groups
     const bool stager = tid < 120;
     const int xx = tid % kCtHX, r0 = tid / kCtHX;
-    auto stage_b = [&](int s) {
-      const uint4* src =
-          reinterpret_cast<const uint4*>(wp) + ((size_t)slice * S + s) * (C::B / 16);
-      uint4* dst = reinterpret_cast<uint4*>(Bs);
-      for (int i = tid; i < C::B / 16; i += 128) dst[i] = src[i];
+    // requests stage s's weights into buffer b (asynchronous copies)
+    auto request_b = [&](int s, int b) {
+      const unsigned char* src = reinterpret_cast<const unsigned char*>(wp) +
+                                 ((size_t)slice * S + s) * C::B;
+      const uint32_t dst = smem_u32(Bs + b * C::B);
+      for (int i = tid; i < C::B / 16; i += 128)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 16 * i),
+                     "l"(src + 16 * i)
+                     : "memory");
     };
-    if (S == 1) stage_b(0);   // one stage: the weights stay for every tile
+    // the first stage's; one or two stages' weights stay for every tile
+    if ((int)blockIdx.x < ntiles) {
+      request_b(0, 0);
+      if (S == 2) request_b(1, 1);
+    }
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
       const int tx = t % tiles_x, ty = (t / tiles_x) % tiles_y, ch = t / (tiles_x * tiles_y);
       const int x0 = tx * kCtTX, y0 = ty * kCtTY;
@@ -532,7 +551,7 @@ conv3_tc(const float* __restrict__ in, int Cin, const __nv_bfloat16* __restrict_
       const int p0 = max(z0 - 1, 0), p1 = min(z1 + 1, d.D);  // input planes [p0, p1)
       const int gx = x0 - 1 + xx;
       const bool xin = gx >= 0 && gx < d.W;
-      for (int s = 0; s < S; ++s) {
+      for (int s = 0; s < S; ++s, ++w) {
         for (int p = p0; p < p1; ++p, ++n) {
           // a plane's values are requested before the wait for its buffer
           float v[2][2][8];
@@ -550,13 +569,14 @@ conv3_tc(const float* __restrict__ in, int Cin, const __nv_bfloat16* __restrict_
                 v[h][g][c] = (inside && c0 + c < Cin) ? q[(size_t)c * V] : 0.f;
             }
           }
-          // the buffer is free when the MMAs of its last use are done; the
-          // weights when those of every plane so far are
-          if (S > 1 && p == p0) {
-            if (n >= 1) ct_wait(empty + ((n - 1) & 1), ((n - 1) >> 1) & 1, err);
-            stage_b(s);
-          } else if (n >= 2) {
-            ct_wait(empty + (n & 1), ((n >> 1) - 1) & 1, err);
+          // the buffer is free when the MMAs of its last use are done
+          if (n >= 2) ct_wait(empty + (n & 1), ((n >> 1) - 1) & 1, err);
+          // the next stage's weights, from the first plane on after which all of
+          // the last stage's MMAs (which read that buffer) are done: the second,
+          // which waited for the plane two before it
+          if (S > 2 && p == (p1 - p0 > 1 ? p0 + 1 : p0)) {
+            if (p1 - p0 == 1 && n >= 1) ct_wait(empty + ((n - 1) & 1), ((n - 1) >> 1) & 1, err);
+            request_b(s + 1 < S ? s + 1 : 0, (w + 1) & 1);
           }
           unsigned char* Ap = As + (n & 1) * kCtA;
 #pragma unroll
@@ -583,6 +603,8 @@ conv3_tc(const float* __restrict__ in, int Cin, const __nv_bfloat16* __restrict_
               }
             }
           }
+          // this stage's weights have landed before its first plane is handed over
+          if (p == p0) asm volatile("cp.async.wait_all;\n" ::: "memory");
           fence_proxy_async_smem();
           tc_fence_before();   // the epilogue's reads of D come before the next MMAs
           mbar_arrive(full + (n & 1));
@@ -616,6 +638,7 @@ conv3_tc(const float* __restrict__ in, int Cin, const __nv_bfloat16* __restrict_
       }
     }
   }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");   // weights requested for a next tile
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -705,7 +728,9 @@ mfto_status conv3_tc_launch(mfto_nn* n, const float* in, int cin, const __nv_bfl
   // of CTAs times a chunk's MMAs (zc planes), its staging (zc + 2, about 0.6 of
   // a plane's MMAs each) and its start and end
   const int slices = (cout + ns - 1) / ns, most = ns == 16 ? CtShape<16>::Z : CtShape<32>::Z;
-  const int64_t fit = std::max<int64_t>(1, (int64_t)n->num_sms * kCtPerSm / slices);
+  const int S = (cin + kCtCin - 1) / kCtCin;
+  const int per_sm = ns == 16 ? CtShape<16>::per_sm(S) : CtShape<32>::per_sm(S);
+  const int64_t fit = std::max<int64_t>(1, (int64_t)n->num_sms * per_sm / slices);
   int zc = 1;
   double best = 0.0;
   for (int z = 1; z <= most && z <= d.D; ++z) {
@@ -720,10 +745,10 @@ mfto_status conv3_tc_launch(mfto_nn* n, const float* in, int cin, const __nv_bfl
   const dim3 grid((unsigned)std::min(items, fit), (unsigned)slices);
   n->launches++;
   if (ns == 16)
-    conv3_tc<16><<<grid, kCtThreads, CtShape<16>::SMEM, n->stream>>>(in, cin, wp, bias, out, cout, d, relu,
+    conv3_tc<16><<<grid, kCtThreads, CtShape<16>::smem(S), n->stream>>>(in, cin, wp, bias, out, cout, d, relu,
                                                               gate, tiles_x, tiles_y, zc, n->d_err);
   else
-    conv3_tc<32><<<grid, kCtThreads, CtShape<32>::SMEM, n->stream>>>(in, cin, wp, bias, out, cout, d, relu,
+    conv3_tc<32><<<grid, kCtThreads, CtShape<32>::smem(S), n->stream>>>(in, cin, wp, bias, out, cout, d, relu,
                                                               gate, tiles_x, tiles_y, zc, n->d_err);
   NCUDA(n, cudaGetLastError());
   return MFTO_OK;
@@ -1124,9 +1149,9 @@ extern "C" mfto_status mfto_nn_create(int32_t base, int32_t levels, int64_t max_
   to_bf16<<<cdiv(off, 256), 256, 0, n->stream>>>(n->w32, n->w16, off);
   if (cudaMemsetAsync(n->d_err, 0, sizeof(int32_t), n->stream) != cudaSuccess ||
       cudaFuncSetAttribute(conv3_tc<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           CtShape<16>::SMEM) != cudaSuccess ||
+                           CtShape<16>::smem(2)) != cudaSuccess ||
       cudaFuncSetAttribute(conv3_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           CtShape<32>::SMEM) != cudaSuccess ||
+                           CtShape<32>::smem(2)) != cudaSuccess ||
       cudaFuncSetAttribute(wgrad3<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem) !=
           cudaSuccess ||
       cudaFuncSetAttribute(wgrad3<14>, cudaFuncAttributeMaxDynamicSharedMemorySize,
