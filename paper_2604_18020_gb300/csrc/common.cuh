@@ -190,6 +190,35 @@ mfto_status mfto_fail(mfto_handle* h, mfto_status code, const char* fmt, ...);
     if (!(cond)) return mfto_fail((h), MFTO_INVALID_ARG, "%s", msg);        \
   } while (0)
 
+// ------------------------------------------- programmatic dependent launch
+// A kernel launched by launch_pdl may have its CTAs placed on the SMs while the
+// kernel before it on the stream still runs, which hides the launch (about 1
+// us between two dependent kernels).  Such a kernel calls pdl_enter() before
+// its first access to memory: it lets the next launch begin to place its CTAs,
+// then waits until the kernel before it has completed and its writes are
+// visible.  As every kernel waits before it completes, all earlier ones have
+// completed as well.  Both are no-ops for a kernel launched otherwise.
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+static inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                     cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // --------------------------------------------------------- index helpers
 struct Grid {
   int nelx, nely, nelz;   // elements

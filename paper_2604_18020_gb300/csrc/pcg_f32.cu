@@ -20,6 +20,11 @@
 // holds no FP64 division).  This removes
 // the fence, ticket atomic and last-block pass that end each kernel of the
 // graph engine.
+//
+// Both kernels are launched as programmatic dependents (launch_pdl), so that a
+// launch's CTAs are placed while the kernel before it ends.  Measured on a
+// GB300, per iteration: 16.9 against 18.2 us at 120 x 60 x 30, 172 against 183
+// us at 256 x 128 x 150, 13.0 against 16.0 us at 24 x 12 x 12.
 #include <math.h>
 
 #include "cg_update.cuh"
@@ -231,6 +236,7 @@ cg2_kv_kernel(const float* __restrict__ E, const float* __restrict__ z,
               const uint8_t* __restrict__ fixed, ModeCoef<float> K, Grid g, ColTiling tl,
               PcgScalars* s, const double* part_b, int nb_b, double* part_a, int par) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_enter();
   DotAcc<float> acc;
   bool skipped = false;   // uniform over the grid
   acc.s = kv_column_body(E, fixed, K, g, tl, ColLoadDirection{z, p_old, 0.f}, ColPcg{p_new, q},
@@ -271,6 +277,7 @@ cg2_update_kernel(float* __restrict__ u, const float* __restrict__ p, const floa
                   float* __restrict__ r, float* __restrict__ z, const float* __restrict__ dinv,
                   int n, PcgScalars* s, const double* part_a, int nb_a, double* part_b,
                   int par) {
+  pdl_enter();
   const int n4 = n >> 2;
   const int first = blockIdx.x * blockDim.x + threadIdx.x;
   const int stride = gridDim.x * blockDim.x;
@@ -463,20 +470,12 @@ mfto_status cg2_enqueue(mfto_handle* h, cudaStream_t st, const PcgVecs<float>& v
     return MFTO_OK;
   }
   const ColTiling tl = col_launch_tiling(h, h->occ_col[kind], &grid);
-  const size_t sm = kColSmem;
-  if (kind == 1)
-    cg2_kv_kernel<3><<<grid, MFTO_BLOCK, sm, st>>>(v.E, v.z, p_old, p_new, v.q, h->d_fixed,
-                                                   h->mc32, g, tl, v.s, v.part_b, nb_b, v.part_a,
-                                                   par);
-  else
-    cg2_kv_kernel<2><<<grid, MFTO_BLOCK, sm, st>>>(v.E, v.z, p_old, p_new, v.q, h->d_fixed,
-                                                   h->mc32, g, tl, v.s, v.part_b, nb_b, v.part_a,
-                                                   par);
+  MFTO_CUDA(h, launch_pdl(kind == 1 ? cg2_kv_kernel<3> : cg2_kv_kernel<2>, grid, MFTO_BLOCK,
+                          kColSmem, st, v.E, v.z, p_old, p_new, v.q, h->d_fixed, h->mc32, g, tl,
+                          v.s, v.part_b, nb_b, v.part_a, par));
   if (ev1) MFTO_CUDA(h, cudaEventRecordWithFlags(ev1, st, cudaEventRecordExternal));
-  cg2_update_kernel<<<nb_b, MFTO_BLOCK, 0, st>>>(v.u, p_new, v.q, v.r, v.z, v.dinv,
-                                                 (int)h->n_dof, v.s, v.part_a, grid, v.part_b,
-                                                 par);
-  MFTO_LAUNCH_CHECK(h);
+  MFTO_CUDA(h, launch_pdl(cg2_update_kernel, nb_b, MFTO_BLOCK, 0, st, v.u, p_new, v.q, v.r, v.z,
+                          v.dinv, (int)h->n_dof, v.s, v.part_a, grid, v.part_b, par));
   return MFTO_OK;
 }
 
