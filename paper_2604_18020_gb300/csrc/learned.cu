@@ -34,7 +34,8 @@ long long nn_max_voxels(const mfto_nn* n);
 const char* nn_message(const mfto_nn* n);
 mfto_status nn_train_forward(mfto_nn* n, cudaStream_t st, int D, int H, int W, const float* x,
                              float** out);
-mfto_status nn_train_backward(mfto_nn* n, cudaStream_t st, int D, int H, int W, float lr);
+mfto_status nn_train_backward(mfto_nn* n, cudaStream_t st, int D, int H, int W, const float* x,
+                              float lr);
 
 // decision of one correction (device)
 struct FpcgCtl {
@@ -726,7 +727,7 @@ extern "C" mfto_status mfto_nn_train_energy(mfto_handle* h, mfto_nn* nn, const d
   energy_grad<<<nblk((int64_t)w->D * w->H * w->W), MFTO_BLOCK, 0, h->stream>>>(
       f, h->d_q, h->d_fixed, h->d_misc, compliance, out, g, vox(w));
   MFTO_LAUNCH_CHECK(h);
-  s = nn_train_backward(nn, h->stream, w->D, w->H, w->W, lr);
+  s = nn_train_backward(nn, h->stream, w->D, w->H, w->W, w->x, lr);
   if (s != MFTO_OK) return mfto_fail(h, s, "network: %s", nn_message(nn));
   if (loss) {
     MFTO_CUDA(h, cudaMemcpyAsync(h->h_misc, h->d_misc, sizeof(MiscScalars), cudaMemcpyDeviceToHost,
