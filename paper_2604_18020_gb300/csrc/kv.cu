@@ -61,13 +61,13 @@ diag_node(const T* __restrict__ E, T* __restrict__ d, const uint8_t* __restrict_
 
 template <typename T>
 __global__ void __launch_bounds__(MFTO_BLOCK)
-modulus_kernel(const double* __restrict__ rho, T* __restrict__ E, double E0, double Emin,
+modulus_kernel(const double* __restrict__ rho, T* __restrict__ E, double dE, double Emin,
                double penal, PowPlan plan, int n) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n) return;
   double rp, unused;
   simp_powers<false>(rho[e], penal, plan, rp, unused);
-  E[e] = (T)(Emin + (E0 - Emin) * rp);
+  E[e] = (T)(Emin + dE * rp);
 }
 
 }  // namespace
@@ -130,10 +130,10 @@ mfto_status modulus_launch(mfto_handle* h, mfto_form form, const double* rho, vo
   h->launches++;
   if (form == MFTO_FORM_F64) {
     modulus_kernel<double><<<blocks_for(n), MFTO_BLOCK, 0, h->stream>>>(
-        rho, (double*)E, h->p.E0, h->p.Emin, h->p.penal, pow_plan(h->p.penal), n);
+        rho, (double*)E, h->p.E0 - h->p.Emin, h->p.Emin, h->p.penal, pow_plan(h->p.penal), n);
   } else if (form == MFTO_FORM_F32) {
     modulus_kernel<float><<<blocks_for(n), MFTO_BLOCK, 0, h->stream>>>(
-        rho, (float*)E, h->p.E0, h->p.Emin, h->p.penal, pow_plan(h->p.penal), n);
+        rho, (float*)E, h->p.E0 - h->p.Emin, h->p.Emin, h->p.penal, pow_plan(h->p.penal), n);
   } else {
     return mfto_fail(h, MFTO_UNSUPPORTED, "mfto_simp_modulus: unsupported form %d", (int)form);
   }

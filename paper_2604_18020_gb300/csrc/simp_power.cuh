@@ -5,9 +5,9 @@
 // of 1/2, and for those the powers are products: r is multiplied up as an
 // unevaluated sum hi + lo (the exact product error of each step by FMA), so the
 // one rounding is that of the final sum, as good as pow's.  Outside
-// [1e-30, 1e30] (where a product error could underflow; r = 0 apart) and for
-// other p, pow itself.  Measured at p = 3: modulus of 4,915,200 elements 100
-// against 833 us.
+// [2^-99, 2^99) (where a product error could underflow; r = 0 apart) and for
+// other p, pow itself.  Measured at p = 3, 7 FP64 operations: modulus of
+// 4,915,200 elements 66 against 833 us.
 #pragma once
 
 struct PowPlan {
@@ -28,7 +28,8 @@ static inline PowPlan pow_plan(double p) {
 template <bool WITH_P1>
 __device__ __forceinline__ void simp_powers(double r, double p, PowPlan q, double& rp,
                                             double& rp1) {
-  if (q.k > 0 && r >= 1e-30 && r <= 1e30) {
+  // r in [2^-99, 2^99), by its exponent (a comparison takes the FP64 pipe)
+  if (q.k > 0 && (unsigned)__double2hiint(r) - ((1023u - 99u) << 20) < (198u << 20)) {
     double h = 1.0, l = 0.0;
     if (q.half) {                        // sqrt(r) = s + (r - s^2) / (2 s)
       const double y = rsqrt(r);
@@ -37,8 +38,15 @@ __device__ __forceinline__ void simp_powers(double r, double p, PowPlan q, doubl
     } else if (q.k > 1) {
       h = r;
     }
-    // h + l = r^(1/2), r (k > 1) or 1; multiplied up to r^(p-1)
-    for (int i = q.half ? 1 : 2; i < q.k; ++i) {
+    int i = q.half ? 1 : 2;
+    if (!q.half && q.k > 2) {            // the first product has no l
+      const double t = r * r;
+      l = fma(r, r, -t);
+      h = t;
+      i = 3;
+    }
+    // h + l = r^(1/2), r (k > 1), r^2 or 1; multiplied up to r^(p-1)
+    for (; i < q.k; ++i) {
       const double t = h * r;
       l = fma(l, r, fma(h, r, -t));
       h = t;
