@@ -231,10 +231,10 @@ constexpr size_t energy_smem() {
 // One cooperative grid; a grid barrier counts arrivals (release-add of one per
 // CTA, acquire-polls; bounded), and every CTA adds the per-CTA partials in the
 // same order, so that all take the same branches.  Bound by the FP64 pipe in
-// the first pass (a_e: about 30 operations) and by about ten grid barriers of
-// 2 to 3 us.  Measured on a GB300: 41 against 265 us at
-// 216,000 elements (a bisection of about 37 full evaluations), 325 against
-// 1,917 us at 4,915,200.
+// the first pass (a_e: 8 operations) and by about ten grid barriers of
+// 2 to 3 us.  Measured on a GB300: 37 against 265 us at
+// 216,000 elements (a bisection of about 37 full evaluations), 250 against
+// 1,917 us at 4,915,200 (325 with the library's square root and FP64 comparisons).
 constexpr int kOcThreads = 512;
 constexpr int kOcSeg = 64;        // undecided elements a CTA may list
 constexpr int kOcMine = 4;        // ... and a thread
@@ -250,6 +250,51 @@ struct OcUp {                     // the bisection whose every midpoint exceeds 
   double l1, l2, last;
   int step;
 };
+
+// The FP64 pipe bounds the passes over the elements, and comparisons, minima
+// and conversions take it too: these go by the bits where the operands allow.
+
+// a = r sqrt(max(0, -dc) n), neg_n = -n.  The square root by Goldschmidt's
+// iteration with a final residual (P. Markstein, "Software division and square
+// root using Goldschmidt's algorithms", 2004) from the hardware's
+// approximation: 6 FP64 operations, the result within an ulp; sqrt where the
+// argument lies near the ends of the exponent range.
+__device__ __forceinline__ double oc_scale(double r, double dc, double neg_n) {
+  const double x = dc * neg_n;
+  const unsigned hi = (unsigned)__double2hiint(x);
+  if (hi - 0x20000000u >= 0x40000000u) {
+    // not positive (or NaN, as fmax(0, NaN) = 0)
+    if (__double_as_longlong(x) <= 0 || hi >= 0x7ff80000u) return r * 0.0;
+    return r * sqrt(x);
+  }
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double g = x * y;
+  double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));   // y / 2
+  const double e = fma(-g, h, 0.5);
+  g = fma(g, e, g);
+  h = fma(h, e, h);
+  g = fma(fma(-g, g, x), h, g);
+  return r * g;
+}
+
+// (float)x for x >= 0 in FP32's normal range (ties away from zero); the
+// conversion elsewhere
+__device__ __forceinline__ float oc_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  if (hi - (897u << 20) >= (253u << 20)) return (hi | lo) == 0u ? 0.f : (float)x;
+  return __uint_as_float(((hi - (896u << 20)) << 3 | lo >> 29) + (lo >> 28 & 1u));
+}
+
+// max(0, r - move) and min(1, r + move) (r no NaN)
+__device__ __forceinline__ double oc_low(double r, double move) {
+  const double v = r - move;
+  return __double2hiint(v) < 0 ? 0.0 : v;
+}
+__device__ __forceinline__ double oc_high(double r, double move) {
+  const double v = r + move;
+  return __double_as_longlong(v) > 0x3ff0000000000000ll ? 1.0 : v;
+}
 
 template <int G>
 __global__ void __launch_bounds__(kOcThreads, G > 0 ? 1 : 2)
@@ -267,6 +312,7 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
   const int stride = gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float movef = (float)move;
+  const double neg_n = -(double)n;
   // per element a (FP64) and (a, rho) in FP32: in registers (G > 0: up to G
   // elements per thread) or in scratch arrays (G == 0, larger meshes)
   double ra[G > 0 ? G : 1];
@@ -341,11 +387,11 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
   float sum_lo = 0.f, sum_hi = 0.f, sum_a = 0.f;
   auto init = [&](int e, double& a, float2& f) {
     const double r = rho[e];
-    a = r * sqrt(fmax(0.0, -dc[e]) * (double)n);
-    f = make_float2((float)a, (float)r);
+    a = oc_scale(r, dc[e], neg_n);
+    f = make_float2(oc_f32(a), oc_f32(r));
     const float lo = fmaxf(0.f, f.y - movef);
     sum_lo += lo;
-    sum_hi += a > 0.0 ? fminf(1.f, f.y + movef) : lo;
+    sum_hi += f.x > 0.f ? fminf(1.f, f.y + movef) : lo;
     sum_a += f.x;
   };
   if constexpr (G > 0) {
@@ -449,10 +495,10 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
     each([&](int e, double a, float2 f) {
       const float t = f.x * sf;
       const float lo = fmaxf(0.f, f.y - movef), hi = fminf(1.f, f.y + movef);
-      if (t * (1.f + kOcMargin) < lo || a == 0.0) {
-        cacc += fmax(0.0, rho[e] - move);
+      if (t * (1.f + kOcMargin) < lo || __double_as_longlong(a) == 0) {
+        cacc += oc_low(rho[e], move);
       } else if (t * (1.f - kOcMargin) > hi) {
-        cacc += fmin(1.0, rho[e] + move);
+        cacc += oc_high(rho[e], move);
       } else if (t * (1.f - kOcMargin) > lo && t * (1.f + kOcMargin) < hi && t > 1e-30f) {
         aacc += a;
       } else {
@@ -662,10 +708,23 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
   double mx = 0.0;
   each([&](int e, double a, float2) {
     const double r = rho[e];
-    const double rn =
-        last > 0.0 ? fmax(fmax(0.0, r - move), fmin(fmin(1.0, r + move), a * sc)) : r;
+    double rn = r;
+    if (last > 0.0) {
+      if (__double2hiint(r) < 0x7ff00000) {
+        // the candidate between its bounds; neither it nor the lower one is
+        // negative, so the bits order as the values do
+        const long long t = __double_as_longlong(a * sc);
+        const long long lo = __double_as_longlong(oc_low(r, move));
+        const long long hi = __double_as_longlong(oc_high(r, move));
+        const long long m = t < hi ? t : hi;
+        rn = __longlong_as_double(lo > m ? lo : m);
+      } else {
+        rn = fmax(fmax(0.0, r - move), fmin(fmin(1.0, r + move), a * sc));
+      }
+    }
     rho_new[e] = rn;
-    mx = fmax(mx, fabs(rn - r));
+    const long long d = __double_as_longlong(rn - r) & 0x7fffffffffffffffll;
+    mx = __double_as_longlong(mx) < d && d <= 0x7ff0000000000000ll ? __longlong_as_double(d) : mx;
   });
   double* buf = partials + 6 * MFTO_RED_SLOTS;
   const double bm = block_max(mx, sh);
