@@ -73,9 +73,9 @@ divide_kernel(const double* __restrict__ x, const double* __restrict__ W, double
 // and neither changes a bit of it.
 //
 // Measured on a GB300, forward and transpose, against the general kernel (every
-// product formed anew, a division per element): 19 terms at 256 x 128 x 150 326
-// and 353 against 433 and 438 us, at 120 x 60 x 30 25 and 27 against 27 and 31;
-// 27 terms 408 and 445 against 584 and 588 us.  At 7 terms (rmin <= sqrt 2) the
+// product formed anew, a division per element): 19 terms at 256 x 128 x 150 289
+// and 306 against 433 and 438 us, at 120 x 60 x 30 25 and 25 against 27 and 31;
+// 27 terms 382 and 398 against 584 and 588 us.  At 7 terms (rmin <= sqrt 2) the
 // products are few and the staging costs more: 33 against 27 us at 55 x 55 x
 // 165, so these stay with the general kernel.
 constexpr int kFilterThreads = 256;   // threads of a CTA
@@ -85,29 +85,42 @@ struct FilterWeights {
   double w[4];
 };
 
-// a / w in the IEEE rounding, r = RN(1 / w): Markstein's correction (P.
-// Markstein, "Computation of elementary functions on the IBM RISC System/6000
-// processor", 1990) of a quotient good to an ulp; the first correction makes it
-// so.  w is a row sum (between 1 and 54); where a lies near the ends of the
-// exponent range, or is no number, the division itself.
-__device__ __forceinline__ double filter_divide(double a, double w, double r) {
-  const unsigned hi = (unsigned)__double2hiint(a) & 0x7fffffffu;
-  if (hi - 0x10000000u >= 0x60000000u && (hi | (unsigned)__double2loint(a)) != 0u)
-    return __ddiv_rn(a, w);
-  double q = __dmul_rn(a, r);
-  q = __fma_rn(__fma_rn(-q, w, a), r, q);
-  return __fma_rn(__fma_rn(-q, w, a), r, q);
-}
-
-// a row sum and its reciprocal, renewed when the sum changes along z
+// A row sum w (between 1 and 54), its reciprocal r = RN(1 / w) and whether that
+// is so close that a r is within an ulp of a / w (half an ulp of rounding and
+// half of the reciprocal's error); renewed when the sum changes along z.
 struct FilterRow {
   double w = 1.0, r = 1.0;
+  bool close = true;
   __device__ __forceinline__ void set(double v) {
     if (__double_as_longlong(v) == __double_as_longlong(w)) return;
     w = v;
     r = __drcp_rn(v);
+    close = fabs(__fma_rn(-v, r, 1.0)) <= 0.99 * 0x1p-54;
   }
 };
+
+// a / w in the IEEE rounding: Markstein's correction (P. Markstein, "Computation
+// of elementary functions on the IBM RISC System/6000 processor", 1990) of a
+// quotient good to an ulp; an r that is not close takes a first correction to
+// get there.  Where a lies near the ends of the exponent range, or is no number,
+// the division itself.
+__device__ __forceinline__ double filter_divide(double a, const FilterRow& row) {
+  const unsigned hi = (unsigned)__double2hiint(a) & 0x7fffffffu;
+  if (hi - 0x10000000u >= 0x60000000u && (hi | (unsigned)__double2loint(a)) != 0u)
+    return __ddiv_rn(a, row.w);
+  double q = __dmul_rn(a, row.r);
+  if (!row.close) q = __fma_rn(__fma_rn(-q, row.w, a), row.r, q);
+  return __fma_rn(__fma_rn(-q, row.w, a), row.r, q);
+}
+
+// w x; x / 2 (half: w = 1/2, the neighbours' weight at rmin = 1.5) by the exponent
+__device__ __forceinline__ double filter_product(double w, bool half, double x) {
+  const int hi = __double2hiint(x);
+  const unsigned e = (unsigned)hi & 0x7ff00000u;
+  if (half && e - 0x00200000u < 0x7fd00000u)
+    return __hiloint2double(hi - 0x00100000, __double2loint(x));
+  return __dmul_rn(w, x);
+}
 
 // the first term of a sum that starts from +0
 __device__ __forceinline__ double filter_first(double t) {
@@ -150,6 +163,7 @@ filter_near_kernel(const double* __restrict__ x, double* __restrict__ y,
   const bool hin = halo && hi >= 0 && hj >= 0 && hi < g.nelx && hj < g.nely;
   const int hcol = hin ? hi + g.nelx * hj : 0;
   const bool warp_halo = __any_sync(0xffffffffu, hin);
+  const bool half = fw.w[1] == 0.5;
   // planes start as zeros: columns outside the mesh stay so
   for (int t = tid; t < 2 * C * P; t += kFilterThreads) (&planes[0][0][0])[t] = 0.0;
   __syncthreads();
@@ -176,10 +190,10 @@ filter_near_kernel(const double* __restrict__ x, double* __restrict__ y,
         double v = xo;
         if constexpr (T) {
           ro.set(wo);
-          v = filter_divide(v, ro.w, ro.r);
+          v = filter_divide(v, ro);
         }
         p[0] = __dmul_rn(fw.w[0], v);
-        p[1] = __dmul_rn(fw.w[1], v);
+        p[1] = filter_product(fw.w[1], half, v);
         pl[0][q] = p[1];
 #pragma unroll
         for (int c = 2; c <= C; ++c) pl[c - 1][q] = __dmul_rn(fw.w[c], v);
@@ -188,11 +202,12 @@ filter_near_kernel(const double* __restrict__ x, double* __restrict__ y,
         double v = xh;
         if constexpr (T) {
           rh.set(wh);
-          v = filter_divide(v, rh.w, rh.r);
+          v = filter_divide(v, rh);
         }
         if (halo) {
 #pragma unroll
-          for (int c = 1; c <= C; ++c) pl[c - 1][hq] = __dmul_rn(fw.w[c], v);
+          for (int c = 1; c <= C; ++c)
+            pl[c - 1][hq] = c == 1 ? filter_product(fw.w[1], half, v) : __dmul_rn(fw.w[c], v);
         }
       }
     }
@@ -226,7 +241,7 @@ filter_near_kernel(const double* __restrict__ x, double* __restrict__ y,
       double out = lo;
       if constexpr (!T) {
         ry.set(wy);
-        out = filter_divide(out, ry.w, ry.r);
+        out = filter_divide(out, ry);
       }
       y[col + nxy * (L - 1)] = out;
     }
