@@ -573,7 +573,7 @@ mfto_status make_tiles(mfto_batch* b) {
       work += (double)x.ntile * (x.nzc + 3);
       most = most > x.nzc ? most : x.nzc;
     }
-    const double slots = 3.0 * b->num_sms;
+    const double slots = (double)kBatchPerSm * b->num_sms;
     const double c = n <= slots ? most + 3.0 : work / slots + 0.5 * (most + 3.0);
     if (best == 0 || c < cost) {
       cost = c;

@@ -32,6 +32,7 @@ constexpr int kBatchNodes = MFTO_BLOCK + kBatchRow + 2; // staged nodes of a lay
 constexpr int kBatchSums = MFTO_BLOCK + 1;              // column sums, one (zero) in front
 constexpr int kBatchUpdate = 1024;                      // DOFs of an update CTA
 constexpr int kBatchLayer = 3 * kBatchNodes;            // floats of a staged layer
+constexpr int kBatchPerSm = 2;                          // CTAs of A (three: registers spill)
 
 // The tiles of an instance (bx + ntx (by + nty bz), from tile0): rows of
 // pitch w, `rows` of them (the first a halo), ow owned nodes along x from
@@ -141,7 +142,7 @@ constexpr size_t kBatchCgSmem =
 static_assert(kBatchLayer % 2 == 0 && kBatchNodes % 2 == 0 && kBatchRingFloats % 2 == 0,
               "pairs are 8-byte aligned");
 
-__global__ void __launch_bounds__(MFTO_BLOCK, 3)
+__global__ void __launch_bounds__(MFTO_BLOCK, kBatchPerSm)
 batch_cg_kv(BatchCgArgs a, ModeCoef<float> K) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ float s_beta;
