@@ -1,6 +1,8 @@
 // Launchers of the mode-space K.v kernels (FP32: kv_column.cuh and the block
 // variant of kv_tile.cuh; FP64: kv_column64.cuh): plain y = K v and the CG form
 // that also forms p_new = z + beta p_old, q = K p_new and alpha.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kv_column.cuh"
 #include "kv_column64.cuh"
@@ -698,7 +700,7 @@ extern "C" mfto_status mfto_kv_autotune(mfto_handle* h, int32_t* nzc_out, int32_
   cudaEvent_t a, b;
   MFTO_CUDA(h, cudaEventCreate(&a));
   MFTO_CUDA(h, cudaEventCreate(&b));
-  const int saved_nzc = h->col_nzc, saved_kind = h->col_kind;
+  const int saved_nzc = h->col_nzc, saved_kind = h->col_kind, chunk = h->p.check_every;
   int best = 0, best_kind = 0;
   float best_ms = 0.f;
   // the graph CG engines time one inner CG iteration (the K.v launch with
@@ -711,7 +713,11 @@ extern "C" mfto_status mfto_kv_autotune(mfto_handle* h, int32_t* nzc_out, int32_
       if (cg) {
         pcg_graph_release(h);
         float us = 0.f;
-        mfto_status st = pcg_time_iterations(h, 2, &us);
+        // graphs of 8 iterations, replayed 4 times: instantiating one of the
+        // usual length takes longer than timing it
+        h->p.check_every = std::min(8, chunk);
+        mfto_status st = pcg_time_iterations(h, 4, &us);
+        h->p.check_every = chunk;
         if (st != MFTO_OK) {
           h->col_nzc = saved_nzc;
           h->col_kind = saved_kind;
