@@ -55,18 +55,18 @@ SMI_FIELDS = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.act
               "clocks_event_reasons.sw_thermal_slowdown,clocks_event_reasons.sw_power_cap")
 IR_MODES = {"restart": 0, "continue": 1}
 # DRAM bytes (read + write) per launch of the dominant kernels from one ncu
-# capture (profiles/kv_f32_cg2_cantilever_120x60x30_full.md,
+# capture (profiles/perf_cases_kernels.md; with all counters profiles/kv_f32_cg2_cantilever_120x60x30_full.md,
 # profiles/kv_f32_cg2_cantilever_256x128x150_full.md), cold caches, each with a
 # digest of the kernel's source files at capture time: when the sources change the figure is reported as stale (null) until it is re-taken.
 KERNEL_SOURCES = {
     "cg2_kv_kernel": ["kv_column.cuh", "pcg_f32.cu", "modes.cuh"],
-    "pcg_kv_col64_kernel": ["kv_column64.cuh", "kv_tile.cu", "modes.cuh"],
+    "pcg_kv_fixed_kernel": ["kv_fixed.cuh", "kv_column_fixed.cuh", "kv_tile.cu"],
 }
 NCU_DRAM_BYTES = {
-    ("cg2_kv_kernel<2>", WORKLOAD): (6.646272e6, "0c045bd0c8e8"),
-    ("cg2_kv_kernel<3>", WORKLOAD): (6.649088e6, "0c045bd0c8e8"),
-    ("cg2_kv_kernel<2>", "cantilever_256x128x150"): (143.325184e6 + 74.990592e6, "0c045bd0c8e8"),
-    ("cg2_kv_kernel<3>", "cantilever_256x128x150"): (144.233472e6 + 74.192384e6, "0c045bd0c8e8"),
+    ("cg2_kv_kernel<2>", WORKLOAD): (6.646528e6, "ee6ff0790f2f"),
+    ("cg2_kv_kernel<3>", WORKLOAD): (6.650112e6, "ee6ff0790f2f"),
+    ("cg2_kv_kernel<2>", "cantilever_256x128x150"): (143.270656e6 + 75.499776e6, "ee6ff0790f2f"),
+    ("cg2_kv_kernel<3>", "cantilever_256x128x150"): (144.322048e6 + 74.235648e6, "ee6ff0790f2f"),
 }
 
 
@@ -654,14 +654,14 @@ def gpu_bench(args, rank, local_rank, world):
                          "launches": cgt[0], "iterations_per_launch": cgt[1] / cgt[0],
                          "launch_us": cgt[2] * 1e3 / cgt[0]})
     else:
-        fp64_peak_tflops = n_sm * 2 * 2 * sm_mhz * 1e6 / 1e12   # 2 DFMA/clk/SM, measured clock
-        roof = {"bound": "alu", "achieved": FLOP_PER_ELEM * m.n_elem / kv_avg_s / 1e12,
-                "peak": fp64_peak_tflops, "unit": "TFLOP/s",
-                "kernel": "pcg_kv_col64_kernel",
-                "traffic": ncu_traffic("pcg_kv_col64_kernel", WORKLOAD)[0],
-                "peak_source": f"FP64 FMA pipe, {n_sm} SMs x 2 DFMA/clk x 2 flop x "
-                               f"{sm_mhz:.0f} MHz median SM clock under load",
-                "flop_per_elem": FLOP_PER_ELEM}
+        # the fixed-point operator runs on the integer pipes; against HBM: reads
+        # z, p_old, E and the mask, writes p_new and q
+        nbytes = 8 * (4 * m.n_dof + m.n_elem) + m.n_node
+        roof = {"bound": "hbm", "achieved": nbytes / kv_avg_s / 1e9, "peak": measured_hbm_gbs(),
+                "unit": "GB/s", "kernel": "pcg_kv_fixed_kernel",
+                "traffic": ncu_traffic("pcg_kv_fixed_kernel", WORKLOAD)[0],
+                "bytes_per_launch": nbytes, "flop_per_elem": FLOP_PER_ELEM,
+                "tflops_dense": FLOP_PER_ELEM * m.n_elem / kv_avg_s / 1e12}
     roof["frac"] = roof["achieved"] / roof["peak"]
     large = None
     if args.form == "mixed" and args.inner_form == "f32" and not args.no_large and rank == 0:
