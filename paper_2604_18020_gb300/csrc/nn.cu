@@ -813,19 +813,18 @@ int wgrad_co(int cout) {
 
 mfto_status wgrad_launch(mfto_nn* n, const NnLayer& L, const float* in, const float* dout, Dims d) {
   const int co = wgrad_co(L.cout);
-  // one wave: three CTAs per SM (shared memory)
-  const WgradPlan pl = wgrad_plan(L.cin, L.cout, d, co, 3 * n->num_sms, n->wpart_elems);
+  const WgradPlan pl = wgrad_plan(L.cin, L.cout, d, co, n->num_sms, n->wpart_elems);
   const size_t row = (size_t)L.cout * pl.pairs * 3;
   if ((size_t)pl.tasks * row > n->wpart_elems)
     return nfail(n, MFTO_INVALID_ARG, "weight partials too small");
   const dim3 grid(pl.pblocks * pl.cblocks, pl.tasks);
   n->launches += 2;
   if (co == 14)
-    wgrad3<14><<<grid, 128, kWgSmem, n->stream>>>(in, L.cin, dout, L.cout, d, pl, n->wpart);
+    wgrad3<14><<<grid, 128, wg_smem_bytes(pl.xt), n->stream>>>(in, L.cin, dout, L.cout, d, pl, n->wpart);
   else if (co == 16)
-    wgrad3<16><<<grid, 128, kWgSmem, n->stream>>>(in, L.cin, dout, L.cout, d, pl, n->wpart);
+    wgrad3<16><<<grid, 128, wg_smem_bytes(pl.xt), n->stream>>>(in, L.cin, dout, L.cout, d, pl, n->wpart);
   else
-    wgrad3<8><<<grid, 128, kWgSmem, n->stream>>>(in, L.cin, dout, L.cout, d, pl, n->wpart);
+    wgrad3<8><<<grid, 128, wg_smem_bytes(pl.xt), n->stream>>>(in, L.cin, dout, L.cout, d, pl, n->wpart);
   NCUDA(n, cudaGetLastError());
   wgrad_sum<<<cdiv(row, 32), 256, 0, n->stream>>>(n->wpart, L.cin, L.cout, pl, n->grad + L.w_off,
                                                   n->grad + L.b_off);
@@ -1118,7 +1117,7 @@ extern "C" mfto_status mfto_nn_create(int32_t base, int32_t levels, int64_t max_
         // the weight gradient's partials: one wave of CTAs, each 128 pairs x 3
         // x its output channels; never more than one task per voxel
         const size_t row = (size_t)ly.cout * (9 * ly.cin + 1) * 3;
-        const size_t wave = (size_t)(3 * n->num_sms) * 128 * 3 * 16;
+        const size_t wave = (size_t)(4 * n->num_sms) * 128 * 3 * 16;
         const size_t most = row * (size_t)(TV >> (3 * l));
         const size_t take = most < wave ? most : wave;
         wp = wp > take + row ? wp : take + row;
@@ -1174,12 +1173,12 @@ extern "C" mfto_status mfto_nn_create(int32_t base, int32_t levels, int64_t max_
                            CtShape<16>::smem(2)) != cudaSuccess ||
       cudaFuncSetAttribute(conv3_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            CtShape<32>::smem(2)) != cudaSuccess ||
-      cudaFuncSetAttribute(wgrad3<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem) !=
+      cudaFuncSetAttribute(wgrad3<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wg_smem_bytes(kWgX)) !=
           cudaSuccess ||
       cudaFuncSetAttribute(wgrad3<14>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kWgSmem) != cudaSuccess ||
+                           (int)wg_smem_bytes(kWgX)) != cudaSuccess ||
       cudaFuncSetAttribute(wgrad3<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kWgSmem) != cudaSuccess ||
+                           (int)wg_smem_bytes(kWgX)) != cudaSuccess ||
       cudaStreamSynchronize(n->stream) != cudaSuccess) {
     cudaGetLastError();
     free_nn(n);

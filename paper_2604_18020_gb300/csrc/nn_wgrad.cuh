@@ -17,11 +17,11 @@
 // a fixed order: along a row into one set of accumulators, rows into a second
 // set, tasks by wgrad_sum -- short chains, so that the rounding stays below
 // that of the products' inputs.  Measured on a GB300, 72 x 40 x 40 voxels, 14 to 14
-// channels: 48 against 389 us; all 14 layers of a gradient 0.6 against 3.9 ms.
+// channels: 48 against 389 us; all 14 layers of a gradient 0.58 against 3.9 ms (0.60 with
+// three CTAs per SM).
 #pragma once
 
 constexpr int kWgX = 62;           // voxels of a row segment (with its halo: two warp passes)
-constexpr int kWgPitch = 67;       // odd: lanes read different rows
 constexpr int kWgCi = 16;          // input channels that 128 pairs can touch
 constexpr int kWgRows = 8;         // y rows of a unit
 constexpr int kWgG = 16;           // staged gradient values per voxel
@@ -30,9 +30,19 @@ struct WgradPlan {
   int pairs, pblocks, cblocks;     // 9 Cin + 1 pairs; blocks of 128 pairs and CO channels
   int xtiles, xt, yblocks, units;  // row segments and their length; row blocks per z; units
   int per_task, tasks;             // units per task; tasks
+  int pitch;                       // floats of a staged x row: odd, lanes read different rows
 };
 
-constexpr size_t kWgSmem = sizeof(float) * (kWgCi * 3 * 4 * kWgPitch + 2 * kWgX * kWgG);
+// shared memory of segments of xt voxels, and the CTAs an SM holds with it (four
+// by the registers; segments of 39 voxels and more: three)
+__host__ __device__ constexpr int wg_pitch(int xt) { return (xt + 2) | 1; }
+constexpr size_t wg_smem_bytes(int xt) {
+  return sizeof(float) * (size_t)(kWgCi * 3 * 4 * wg_pitch(xt) + 2 * xt * kWgG);
+}
+constexpr int wg_per_sm(int xt) {
+  const int fit = (int)(227 * 1024 / (wg_smem_bytes(xt) + 1024));
+  return fit < 4 ? fit : 4;
+}
 
 __device__ __forceinline__ void wg_cp4(float* dst, const float* src, bool valid) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -42,13 +52,14 @@ __device__ __forceinline__ void wg_cp4(float* dst, const float* src, bool valid)
 }
 
 template <int CO>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 4)
 wgrad3(const float* __restrict__ in, int Cin, const float* __restrict__ dout, int Cout, Dims d,
        WgradPlan pl, float* __restrict__ partial) {
   static_assert(CO % 2 == 0 && CO <= kWgG, "pairs of output channels");
   extern __shared__ __align__(16) float wg_smem[];
-  float* gs = wg_smem;                              // [2][kWgX][kWgG]
-  float* xs = wg_smem + 2 * kWgX * kWgG;            // [kWgCi][3][4 slots][kWgPitch]
+  const int pitch = pl.pitch, gstep = pl.xt * kWgG;
+  float* gs = wg_smem;                              // [2][xt][kWgG]
+  float* xs = wg_smem + 2 * gstep;                  // [kWgCi][3][4 slots][pitch]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int pb = blockIdx.x % pl.pblocks, cb = blockIdx.x / pl.pblocks;
   const int co0 = cb * CO, c0 = pb * 128 / 9;
@@ -59,7 +70,7 @@ wgrad3(const float* __restrict__ in, int Cin, const float* __restrict__ dout, in
   const bool is_bias = p == 9 * Cin, live = p < 9 * Cin;
   const int ci = live ? p / 9 - c0 : 0, k9 = live ? p % 9 : 0;
   const int dz = k9 / 3, dy = k9 % 3;
-  const float* xrow = xs + (ci * 3 + dz) * 4 * kWgPitch;
+  const float* xrow = xs + (ci * 3 + dz) * 4 * pitch;
 
   // copies of x row y (planes z - 1 .. z + 1, this block's channels) into slot
   // y & 3, and of gradient row yg into buffer yg & 1 (zero outside the grid)
@@ -70,7 +81,7 @@ wgrad3(const float* __restrict__ in, int Cin, const float* __restrict__ dout, in
       const bool row_in = c0 + c < Cin && zz >= 0 && zz < d.D && y >= 0 && y < d.H;
       const float* src = in + (size_t)(row_in ? c0 + c : 0) * V +
                          (row_in ? ((size_t)zz * d.H + y) * d.W : 0);
-      float* dst = xs + (r * 4 + (y & 3)) * kWgPitch;
+      float* dst = xs + (r * 4 + (y & 3)) * pitch;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int i = lane + 32 * h, x = x0 - 1 + i;
@@ -82,7 +93,7 @@ wgrad3(const float* __restrict__ in, int Cin, const float* __restrict__ dout, in
     }
   };
   auto load_g = [&](int z, int y) {
-    float* dst = gs + (y & 1) * kWgX * kWgG;
+    float* dst = gs + (y & 1) * gstep;
     for (int j = warp; j < CO; j += 4) {
       const bool row_in = co0 + j < Cout && y < d.H;
       const float* src = dout + (size_t)(row_in ? co0 + j : 0) * V +
@@ -125,8 +136,8 @@ wgrad3(const float* __restrict__ in, int Cin, const float* __restrict__ dout, in
       commit();
       asm volatile("cp.async.wait_group 1;\n" ::: "memory");
       __syncthreads();
-      const float* xr = xrow + ((y - 1 + dy) & 3) * kWgPitch;
-      const float* gr = gs + (y & 1) * kWgX * kWgG;
+      const float* xr = xrow + ((y - 1 + dy) & 3) * pitch;
+      const float* gr = gs + (y & 1) * gstep;
       float2 acc[CO / 2][3];
 #pragma unroll
       for (int j = 0; j < CO / 2; ++j)
@@ -193,9 +204,9 @@ wgrad_sum(const float* __restrict__ partial, int Cin, int Cout, WgradPlan pl,
   else if (q == 27 * Cin + 1) gb[co] = a + b;   // the x = 1 pair, dx = 0
 }
 
-// Tasks of a layer: units grouped so that about `ctas` blocks run, as far
-// as the partials (max_partial floats) allow.
-static inline WgradPlan wgrad_plan(int Cin, int Cout, const Dims& d, int co, int ctas,
+// Tasks of a layer: units grouped into one wave of blocks, as far as the
+// partials (max_partial floats) allow.
+static inline WgradPlan wgrad_plan(int Cin, int Cout, const Dims& d, int co, int num_sms,
                                    size_t max_partial) {
   WgradPlan p;
   p.pairs = 9 * Cin + 1;
@@ -203,10 +214,11 @@ static inline WgradPlan wgrad_plan(int Cin, int Cout, const Dims& d, int co, int
   p.cblocks = (Cout + co - 1) / co;
   p.xtiles = (d.W + kWgX - 1) / kWgX;
   p.xt = (d.W + p.xtiles - 1) / p.xtiles;
+  p.pitch = wg_pitch(p.xt);
   p.yblocks = (d.H + kWgRows - 1) / kWgRows;
   p.units = d.D * p.yblocks * p.xtiles;
   const size_t one = (size_t)Cout * p.pairs * 3;   // partials of one task
-  long long tasks = ctas / ((long long)p.pblocks * p.cblocks);
+  long long tasks = (long long)wg_per_sm(p.xt) * num_sms / ((long long)p.pblocks * p.cblocks);
   if (tasks > (long long)(max_partial / one)) tasks = (long long)(max_partial / one);
   if (tasks < 1) tasks = 1;
   if (tasks > p.units) tasks = p.units;
