@@ -703,7 +703,7 @@ mfto_status cg2_enqueue(mfto_handle* h, cudaStream_t st, const PcgVecs<float>& v
                         cudaEvent_t ev1);
 mfto_status pcg_persist_iterate(mfto_handle* h, const PcgVecs<float>& v, PcgScalars* host_s);
 mfto_status kv_tile_init(mfto_handle* h);
-void kv_tile_retile(mfto_handle* h);
+mfto_status kv_tile_retile(mfto_handle* h);
 mfto_status simp_init(mfto_handle* h);
 template <typename T>
 mfto_status kv_tile_launch(mfto_handle* h, const T* E, const T* v, T* y, cudaStream_t st);

@@ -216,7 +216,10 @@ static mfto_status upload_params(mfto_handle* h) {
   }
   mode_coefficients(h->p.nu, h->mesh.h, &h->mc64, &h->mc32);
   h->fix_ok = fixed_op(h->p.nu, h->mesh.h, &h->fix);
-  kv_tile_retile(h);
+  {
+    const mfto_status s = kv_tile_retile(h);
+    if (s != MFTO_OK) return s;
+  }
   MFTO_CUDA(h, cudaMemcpyAsync(h->d_ke64, ke, sizeof(ke), cudaMemcpyHostToDevice, h->stream));
   MFTO_CUDA(h, cudaMemcpyAsync(h->d_ke32, ke32, sizeof(ke32), cudaMemcpyHostToDevice, h->stream));
   return filter_setup(h);

@@ -150,22 +150,23 @@ void col64_tile(const mfto_handle* h, const Grid& g, int* shape, int* nzc, int c
     col64_choose(1, g.nx, g.ny, g.nz, 1.5, h->num_sms, shape, nzc, copies);
 }
 
+// shared memory of the FP64 column kernels in use
 mfto_status col64_attrs(mfto_handle* h) {
   for (int i = 0; i < kCol64Shapes; ++i) {
     const mfto_status s = col64_dispatch(i, [&](auto shape) -> mfto_status {
       using S = decltype(shape);
-      MFTO_CUDA(h, cudaFuncSetAttribute(kv_col64_kernel<S::CX, S::CY>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)S::template smem_bytes<1>()));
-      MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_col64_kernel<S::CX, S::CY>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)S::template smem_bytes<2>()));
-      MFTO_CUDA(h, cudaFuncSetAttribute(kv_fixed_kernel<S::CX, S::CY>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)fixed_smem<S::CX, S::CY>()));
-      MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_fixed_kernel<S::CX, S::CY>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)pcg_fixed_smem<S::CX, S::CY>()));
+      const bool fix = h->fix_ok;
+      const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+      const void* plain = fix ? (const void*)kv_fixed_kernel<S::CX, S::CY>
+                              : (const void*)kv_col64_kernel<S::CX, S::CY>;
+      const void* cg = fix ? (const void*)pcg_kv_fixed_kernel<S::CX, S::CY>
+                           : (const void*)pcg_kv_col64_kernel<S::CX, S::CY>;
+      MFTO_CUDA(h, cudaFuncSetAttribute(plain, attr,
+                                        (int)(fix ? fixed_smem<S::CX, S::CY>()
+                                                  : S::template smem_bytes<1>())));
+      MFTO_CUDA(h, cudaFuncSetAttribute(cg, attr,
+                                        (int)(fix ? pcg_fixed_smem<S::CX, S::CY>()
+                                                  : S::template smem_bytes<2>())));
       return MFTO_OK;
     });
     if (s != MFTO_OK) return s;
@@ -405,14 +406,14 @@ ColTiling col_launch_tiling(const mfto_handle* h, int per_sm, int* grid) {
   return tl;
 }
 
-// The FP64 column kernel's tiles, for the operator of the current parameters.
-void kv_tile_retile(mfto_handle* h) {
+// The FP64 column kernel's tiles and attributes, for the operator of the current
+// parameters.
+mfto_status kv_tile_retile(mfto_handle* h) {
   col64_tile(h, make_grid(h->mesh), &h->col64_shape, &h->col64_nzc, 1);
+  return col64_attrs(h);
 }
 
 mfto_status kv_tile_init(mfto_handle* h) {
-  const mfto_status s = col64_attrs(h);
-  if (s != MFTO_OK) return s;
   MFTO_CUDA(h, cudaFuncSetAttribute(kv_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)kBlockSmem));
   MFTO_CUDA(h, cudaFuncSetAttribute(pcg_kv_block_kernel,

@@ -792,9 +792,7 @@ mfto_status simp_init(mfto_handle* h) {
       MFTO_CUDA(h, cudaFuncSetAttribute(compliance_kernel<S::CX, S::CY>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)S::template stream_bytes<1>()));
-      MFTO_CUDA(h, cudaFuncSetAttribute(compliance_fixed_kernel<S::CX, S::CY>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)energy_smem<S>()));
+      static_assert(energy_smem<S>() <= 48 * 1024, "no attribute needed");
       return MFTO_OK;
     });
     if (s != MFTO_OK) return s;
