@@ -460,12 +460,13 @@ mfto_status enqueue_chunk(mfto_batch* b, cudaStream_t st, int chunk, double rtol
     const BatchCgArgs a{b->E32,     b->z32,         p_old, p_new, b->q32,       b->d_fixed,
                         b->d_inst[0], b->d_tiles,   b->d_tile_inst, prev, cur, b->d_share_b,
                         b->d_share_a, b->cg_updates, maxit, rtol * rtol};
-    batch_cg_kv<<<b->cg_tiles, MFTO_BLOCK, kBatchCgSmem, st>>>(a, b->mc32);
-    batch_cg_update<<<b->cg_updates, MFTO_BLOCK, 0, st>>>(
-        b->e32, p_new, b->q32, b->r32, b->z32, b->dinv32, b->d_inst[0], b->d_tiles, b->d_up_inst,
-        cur, b->d_share_a, b->d_share_b, b->cg_updates);
+    BCUDA(b, launch_pdl(batch_cg_kv, b->cg_tiles, MFTO_BLOCK, kBatchCgSmem, st, a, b->mc32));
+    BCUDA(b, launch_pdl(batch_cg_update, b->cg_updates, MFTO_BLOCK, 0, st, b->e32, p_new, b->q32,
+                        b->r32, b->z32, b->dinv32, b->d_inst[0], b->d_tiles, b->d_up_inst, cur,
+                        b->d_share_a, b->d_share_b, b->cg_updates));
   }
-  batch_cg_done<<<1, MFTO_BLOCK, 0, st>>>(b->d_scal + b->count, b->count, &b->d_ctl->all_done);
+  BCUDA(b, launch_pdl(batch_cg_done, 1, MFTO_BLOCK, 0, st, b->d_scal + b->count, b->count,
+                      &b->d_ctl->all_done));
   BCUDA(b, cudaGetLastError());
   return MFTO_OK;
 }

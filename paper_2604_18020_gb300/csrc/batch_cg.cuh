@@ -151,6 +151,7 @@ batch_cg_kv(BatchCgArgs a, ModeCoef<float> K) {
   float* ring = nodes + 3 * kBatchLayer;                // [3][6][kBatchNodes], slot (k + 3) % 3
   float* sums = ring + kBatchRingFloats;                // slot k & 1: 4 pairs, then 4 z
   const int tid = threadIdx.x;
+  pdl_wait();
   const int i = a.tile_inst[blockIdx.x];
   const BatchTiles t = a.tiles[i];
   const BatchInst in = a.inst[i];
@@ -377,6 +378,7 @@ batch_cg_update(float* __restrict__ u, const float* __restrict__ p, const float*
   constexpr int N = kBatchUpdate / MFTO_BLOCK;
   __shared__ float s_alpha;
   __shared__ int s_skip;
+  pdl_wait();
   const int i = up_inst[blockIdx.x];
   const int up0 = tiles[i].up0;
   const int n = 3 * inst[i].nx * inst[i].ny * inst[i].nz;
@@ -466,6 +468,7 @@ batch_cg_start(const float* __restrict__ r, float* __restrict__ z, const float* 
 // whether every instance is done, after a chunk of iterations
 __global__ void __launch_bounds__(MFTO_BLOCK)
 batch_cg_done(const BatchScal* sc, int count, int* all_done) {
+  pdl_wait();
   int live = 0;
   for (int i = threadIdx.x; i < count; i += blockDim.x) live |= !sc[i].done;
   live = __syncthreads_or(live);

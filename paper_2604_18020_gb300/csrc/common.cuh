@@ -191,15 +191,15 @@ mfto_status mfto_fail(mfto_handle* h, mfto_status code, const char* fmt, ...);
   } while (0)
 
 // ------------------------------------------- programmatic dependent launch
-// A kernel launched by launch_pdl may have its CTAs placed on the SMs while the
-// kernel before it on the stream still runs, which hides the launch (about 1
-// us between two dependent kernels).  Such a kernel calls pdl_enter() before
-// its first access to memory: it lets the next launch begin to place its CTAs,
-// then waits until the kernel before it has completed and its writes are
-// visible.  As every kernel waits before it completes, all earlier ones have
-// completed as well.  Both are no-ops for a kernel launched otherwise.
-__device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+// A kernel launched by launch_pdl is made ready while the kernel before it on the
+// stream still runs and starts as that one ends, which hides the launch (about 1
+// us between two dependent kernels).  Such a kernel calls pdl_wait() before its
+// first access to memory: it waits until the kernel before it has completed and
+// its writes are visible.  As every kernel waits before it completes, all
+// earlier ones have completed as well.  A no-op for a kernel launched otherwise.
+// (Placing CTAs earlier still, by launch_dependents, took longer: they hold
+// slots that the running kernel's own CTAs could use.)
+__device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 

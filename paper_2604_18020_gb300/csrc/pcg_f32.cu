@@ -21,10 +21,10 @@
 // the fence, ticket atomic and last-block pass that end each kernel of the
 // graph engine.
 //
-// Both kernels are launched as programmatic dependents (launch_pdl), so that a
-// launch's CTAs are placed while the kernel before it ends.  Measured on a
-// GB300, per iteration: 16.9 against 18.2 us at 120 x 60 x 30, 172 against 183
-// us at 256 x 128 x 150, 13.0 against 16.0 us at 24 x 12 x 12.
+// Both kernels are launched as programmatic dependents (launch_pdl).  Measured
+// on a GB300, per iteration: 16.2 against 18.2 us at 120 x 60 x 30, 20.3 against
+// 23.1 at 64 x 64 x 60, 173 against 183 at 256 x 128 x 150, 13.3 against 16.0 at 24
+// x 12 x 12.
 #include <math.h>
 
 #include "cg_update.cuh"
@@ -236,7 +236,7 @@ cg2_kv_kernel(const float* __restrict__ E, const float* __restrict__ z,
               const uint8_t* __restrict__ fixed, ModeCoef<float> K, Grid g, ColTiling tl,
               PcgScalars* s, const double* part_b, int nb_b, double* part_a, int par) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_enter();
+  pdl_wait();
   DotAcc<float> acc;
   bool skipped = false;   // uniform over the grid
   acc.s = kv_column_body(E, fixed, K, g, tl, ColLoadDirection{z, p_old, 0.f}, ColPcg{p_new, q},
@@ -277,7 +277,7 @@ cg2_update_kernel(float* __restrict__ u, const float* __restrict__ p, const floa
                   float* __restrict__ r, float* __restrict__ z, const float* __restrict__ dinv,
                   int n, PcgScalars* s, const double* part_a, int nb_a, double* part_b,
                   int par) {
-  pdl_enter();
+  pdl_wait();
   const int n4 = n >> 2;
   const int first = blockIdx.x * blockDim.x + threadIdx.x;
   const int stride = gridDim.x * blockDim.x;
