@@ -63,10 +63,10 @@ KERNEL_SOURCES = {
     "pcg_kv_fixed_kernel": ["kv_fixed.cuh", "kv_column_fixed.cuh", "kv_tile.cu"],
 }
 NCU_DRAM_BYTES = {
-    ("cg2_kv_kernel<2>", WORKLOAD): (6.646528e6, "ee6ff0790f2f"),
-    ("cg2_kv_kernel<3>", WORKLOAD): (6.650112e6, "ee6ff0790f2f"),
-    ("cg2_kv_kernel<2>", "cantilever_256x128x150"): (143.270656e6 + 75.499776e6, "ee6ff0790f2f"),
-    ("cg2_kv_kernel<3>", "cantilever_256x128x150"): (144.322048e6 + 74.235648e6, "ee6ff0790f2f"),
+    ("cg2_kv_kernel<2>", WORKLOAD): (6.647552e6, "b59f0e9ab240"),
+    ("cg2_kv_kernel<3>", WORKLOAD): (6.649856e6, "b59f0e9ab240"),
+    ("cg2_kv_kernel<2>", "cantilever_256x128x150"): (143.266816e6 + 75.114240e6, "b59f0e9ab240"),
+    ("cg2_kv_kernel<3>", "cantilever_256x128x150"): (144.243200e6 + 73.851648e6, "b59f0e9ab240"),
 }
 
 
