@@ -217,14 +217,26 @@ mfto_status mfto_kv(mfto_handle* h, mfto_form form, const void* d_E,
 
 /* Choose the K.v kernel used by mfto_kv, mfto_pcg and mfto_simp_step:
  * 0 (default) = element operator in the per-axis (sum, difference) mode
- * basis, about 220 arithmetic operations per element; FP64 runs node-owned
- * tiles streaming along z through a shared-memory ring, FP32 runs one
- * z-column of elements per thread with the face transforms carried from
- * layer to layer (about 170 operations per element); 1 = one thread per node
+ * basis, one z-column of elements per thread with the face transforms carried
+ * from layer to layer; FP32 about 170 operations per element, FP64 in 64-bit
+ * block fixed point for Poisson's ratios in [0, 0.454), on the FP64 pipe
+ * otherwise; 1 = one thread per node
  * gathering its 8 elements with the dense 24x24 KE from shared memory (576
- * multiply-adds per node, the operation count of Alg. 1); 2 = as 0 for FP64,
- * and for FP32 one element per thread over 8 x 8 x 4 element blocks that own
- * their 7 x 7 x 3 interior nodes.  All are atomic-free and bit-reproducible. */
+ * multiply-adds per node, the operation count of Alg. 1); 2 = as 0 with FP64
+ * always on the FP64 pipe (the energies of mfto_compliance_sens and
+ * mfto_simp_step as well), and for FP32 one element per thread over 8 x 8 x 4
+ * element blocks that own their 7 x 7 x 3 interior nodes.  All are atomic-free
+ * and bit-reproducible.
+ *
+ * Precision of the FP64 operator in fixed point: an element's share of a force
+ * is off by at most E times one FP64 rounding of each component's largest
+ * displacement in the element and a few 2^-56 of the largest difference of
+ * displacements there.  That is below the roundings of FP64 sums, except where
+ * such sums are exact: with a simple shear or a rotation of one component,
+ * given by few bits, beside strains of another component 2^4 times smaller and
+ * more, variants 1 and 2 return the smaller force to more bits.  Not finite
+ * inputs give outputs that are not finite at every node of the element (NaN,
+ * where the FP64 pipe may give an infinity). */
 mfto_status mfto_set_kv_variant(mfto_handle* h, int32_t variant);
 
 /* Choose how the FP32 inner Jacobi-PCG of the mixed solve (mfto_ir_solve and

@@ -101,7 +101,7 @@ struct mfto_handle {
   FixOp fix;                // ... in fixed point (kv_fixed.cuh), where it fits
   bool fix_ok;
   ModeCoef<float> mc32;
-  int kv_variant;           // 0: tiled mode-space kernel, 1: node-centric dense KE
+  int kv_variant;           // mfto_set_kv_variant
   int cg_engine;            // FP32 inner CG: 0 two kernels per iteration, 1 persistent,
                             // 2 two ticket-free kernels per iteration
   int persist_grid;         // CTAs of the persistent CG launch (0: unavailable)
@@ -173,6 +173,10 @@ struct mfto_handle {
 };
 
 // --------------------------------------------------------------- errors
+// Whether FP64 K.v and energies run in fixed point (kv_fixed.cuh): where the
+// operator fits, unless the caller chose the FP64 pipe's kernels.
+static inline bool fixed_route(const mfto_handle* h) { return h->fix_ok && h->kv_variant != 2; }
+
 mfto_status mfto_fail(mfto_handle* h, mfto_status code, const char* fmt, ...);
 
 #define MFTO_CUDA(h, call)                                                   \

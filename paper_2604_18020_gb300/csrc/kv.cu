@@ -152,9 +152,10 @@ extern "C" mfto_status mfto_kv(mfto_handle* h, mfto_form form, const void* E, co
 extern "C" mfto_status mfto_set_kv_variant(mfto_handle* h, int32_t variant) {
   if (!h) return MFTO_INVALID_ARG;
   MFTO_REQUIRE(h, variant >= 0 && variant <= 2, "mfto_set_kv_variant: variant must be 0, 1 or 2");
-  if (h->kv_variant != variant) pcg_graph_release(h);
+  if (h->kv_variant == variant) return MFTO_OK;
+  pcg_graph_release(h);
   h->kv_variant = variant;
-  return MFTO_OK;
+  return kv_tile_retile(h);   // the FP64 kernel may be another
 }
 
 extern "C" mfto_status mfto_jacobi_diag(mfto_handle* h, mfto_form form, const void* E,

@@ -4,7 +4,7 @@
 //
 // Per node layer the tile's nodes are copied asynchronously into a ring two
 // layers ahead; the thread that copied a node converts it (masked, combined)
-// to fixed point with the node's exponent in shared memory.  A barrier later
+// to fixed point with its components' exponents in shared memory.  A barrier later
 // every column forms its face modes from four nodes, its element from two
 // faces, and leaves three of its four node shares in shared memory, where the
 // nodes' owners add them a layer later.  One barrier per layer.
@@ -22,14 +22,14 @@ struct FixStream {
   static constexpr int kRing = 2 * 3 * KS * NV;              // doubles, slot of layer k: k & 1
   static constexpr int kNodes = 2 * 3 * NV;                  // int64, slot k & 1
   static constexpr int kOwn = OWN ? 4 * 3 * NV : 0;          // doubles, slot k & 3
-  static constexpr int kExp = 4 * NV;                        // int, slot k & 3
+  static constexpr int kExp = 4 * NV;                        // uint2, slot k & 3
   static constexpr int kWords = kRing + kNodes + kOwn;       // 8-byte words
   static_assert(NV > NT && NV <= 2 * NT, "two nodes at most per thread and layer");
 
   double* ring;
   int64_t* nodes;
   double* ownv;
-  int* nexp;                // exponent | mask << 16
+  uint2* nexp;              // exponents (x | y << 16, z) and the mask (<< 16)
   const Load& ld;
   const uint8_t* fixed;
   int last, nxy, q, left;
@@ -38,7 +38,7 @@ struct FixStream {
 
   // words, exps: shared memory; (i0, j0): node of the tile's corner; last
   // layer: the topmost to copy; k: the operator's FixOp::k
-  __device__ __forceinline__ FixStream(double* words, int* exps, const Load& load,
+  __device__ __forceinline__ FixStream(double* words, uint2* exps, const Load& load,
                                        const uint8_t* fix, const Grid& g, int i0, int j0,
                                        int last_layer, int k)
       : ring(words), nodes(reinterpret_cast<int64_t*>(words + kRing)),
@@ -86,23 +86,21 @@ struct FixStream {
       const uint32_t fm = (masks >> (8 * p)) & 0xffu;
       const double* R = ring + (L & 1) * 3 * KS * NV + t;
       double v[3];
-      int e = 0;
+      uint32_t e[3];
+      int64_t* N = nodes + (L & 1) * 3 * NV + t;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         double r[KS];
 #pragma unroll
         for (int s = 0; s < KS; ++s) r[s] = R[(3 * s + c) * NV];
         v[c] = ((fm >> c) & 1) ? 0.0 : ld.combine(r);
-        e = max(e, __double2hiint(v[c]) & 0x7fffffff);
+        const int hi = __double2hiint(v[c]) & 0x7fffffff;
+        const bool finite = hi < 0x7ff00000, zero = (hi | __double2loint(v[c])) == 0;
+        e[c] = zero ? 0u : finite ? (uint32_t)max(hi >> 20, kFixMinE) : (uint32_t)kFixNan;
+        N[c * NV] = finite ? fix_value((uint64_t)__double_as_longlong(v[c]), left) : 0ll;
       }
-      e = max(e >> 20, kFixMinE);
-      const bool finite = e < 0x7ff;
-      int64_t* N = nodes + (L & 1) * 3 * NV + t;
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        N[c * NV] = finite ? fix_value((uint64_t)__double_as_longlong(v[c]), e, left) : 0ll;
       const int slot = L & 3;
-      nexp[slot * NV + t] = (finite ? e : kFixNan) | (int)(fm << 16);
+      nexp[slot * NV + t] = make_uint2(e[0] | e[1] << 16, e[2] | fm << 16);
       if constexpr (OWN) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) ownv[(slot * 3 + c) * NV + t] = v[c];
@@ -113,18 +111,21 @@ struct FixStream {
   // face modes of node layer L, a barrier after its stage()
   __device__ __forceinline__ void face(int L, FixFace& F) const {
     const int64_t* N = nodes + (L & 1) * 3 * NV + q;
-    const int* X = nexp + (L & 3) * NV + q;
+    const uint2* X = nexp + (L & 3) * NV + q;
     constexpr int at[4] = {0, 1, NX, NX + 1};
-    int e[4];
+    uint2 e[4];
 #pragma unroll
-    for (int n = 0; n < 4; ++n) e[n] = X[at[n]] & 0xffff;
-    F.e = max(max(e[0], e[1]), max(e[2], e[3]));
+    for (int n = 0; n < 4; ++n) e[n] = X[at[n]];
+    // 16-bit lanes: none borrows below, as none exceeds its maximum
+    F.e.xy = fix_max_lanes(fix_max_lanes(e[0].x, e[1].x), fix_max_lanes(e[2].x, e[3].x));
+    F.e.z = fix_max_lanes(fix_max_lanes(e[0].y, e[1].y), fix_max_lanes(e[2].y, e[3].y));
     int64_t v[4][3];
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
-      const int d = min(F.e - e[n], 63);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) v[n][c] = N[c * NV + at[n]] >> d;
+      const uint32_t dx = F.e.xy - e[n].x, dy = F.e.z - e[n].y;
+      v[n][0] = fix_sar(N[at[n]], (int)(dx & 0xffffu));
+      v[n][1] = fix_sar(N[NV + at[n]], (int)(dx >> 16));
+      v[n][2] = fix_sar(N[2 * NV + at[n]], (int)(dy & 0xffffu));
     }
     fix_face(v, F);
   }
@@ -143,7 +144,7 @@ struct FixShape {
   static constexpr int kUp = 12 * St::NT;   // int64, upper outputs of the element below
   static constexpr int kBack = 2 * 9 * St::NT, kBackExp = 2 * St::NT;
   static constexpr size_t kBytes =
-      8 * (size_t)(St::kWords + kBack + kUp) + 4 * (size_t)(St::kExp + kBackExp);
+      8 * (size_t)(St::kWords + kBack + kUp + St::kExp) + 4 * (size_t)kBackExp;
 };
 
 // d 2^t times the operator's unit.
@@ -173,8 +174,8 @@ __device__ __forceinline__ double kv_column_fixed_body(const double* __restrict_
   constexpr int NT = St::NT;
   int64_t* back = reinterpret_cast<int64_t*>(smem + St::kWords);
   int64_t* ups = back + L::kBack + threadIdx.x;
-  int* nexp = reinterpret_cast<int*>(back + L::kBack + L::kUp);
-  int* bexp = nexp + St::kExp;
+  uint2* nexp = reinterpret_cast<uint2*>(back + L::kBack + L::kUp);
+  int* bexp = reinterpret_cast<int*>(nexp + St::kExp);
 
   const int tid = threadIdx.x;
   const int bx = tile % tl.tx, by = (tile / tl.tx) % tl.ty, bz = tile / (tl.tx * tl.ty);
@@ -210,7 +211,7 @@ __device__ __forceinline__ double kv_column_fixed_body(const double* __restrict_
                                : fix_scaled(__ll2double_rn(s), em - 2098 + K.k, K);
     }
     const int slot = k & 3;
-    const uint32_t fm = (uint32_t)nexp[slot * St::NV + st.q] >> 16;
+    const uint32_t fm = nexp[slot * St::NV + st.q].y >> 16;
     if constexpr (Epi::kOwn) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) pn[c] = st.ownv[(slot * 3 + c) * St::NV + st.q];
@@ -238,7 +239,8 @@ __device__ __forceinline__ double kv_column_fixed_body(const double* __restrict_
   };
   uint64_t Ebits = load_modulus(kb - 1);
   __syncthreads();
-  FixFace F0, F1, U;
+  FixFace F0, F1;
+  FixOut U;
   if (warp_elem) st.face(kb - 1, F0);
   auto clear = [&]() {
     U.e = kFixEmpty;
@@ -263,12 +265,15 @@ __device__ __forceinline__ double kv_column_fixed_body(const double* __restrict_
     if (ez - 1 >= kb) finish(ez - 1);
     if (warp_elem) {
       st.face(ez + 1, Fup);
-      FixFace Ms;
+      FixOut Ms;
       if (ez >= 0 && ez < g.nelz) {
-        const int em = max(Flo.e, Fup.e);
-        const int dl = min(em - Flo.e, 63), du = min(em - Fup.e, 63);
         int64_t X[3][8], Z[3][8];
-        fix_modes(Flo, Fup, dl, du, X);
+        const FixExp e{fix_max_lanes(Flo.e.xy, Fup.e.xy), fix_max_lanes(Flo.e.z, Fup.e.z)};
+        const bool nan = fix_nan(e);
+        const int t = fix_modes(Flo, Fup, e, __any_sync(0xffffffffu, fix_apart(e, K.k)), K.k, X);
+        // (by a vote: the answer is then formed here, before the operator needs the
+        // modes' registers; 68 bytes spilled instead of 144)
+        const unsigned strained = __ballot_sync(0xffffffffu, fix_strained(X));
         const FixModulus Em = fix_modulus(Ebits);
         fix_operator(X, K, Em, Z);
         if (__any_sync(0xffffffffu, Em.negative)) {
@@ -277,9 +282,11 @@ __device__ __forceinline__ double kv_column_fixed_body(const double* __restrict_
 #pragma unroll
             for (int m = 1; m < 8; ++m) Z[c][m] = Em.negative ? -Z[c][m] : Z[c][m];
         }
-        const int eo = em >= kFixNan || Em.e == 0x7ff ? (elem_in ? kFixNanOut : kFixEmpty)
-                       : Em.e == 0                    ? kFixEmpty
-                                                      : em + Em.e;
+        // a block that holds nothing shifts no neighbour's bits away
+        const bool any = (strained >> (tid & 31)) & 1u;
+        const int eo = nan || Em.e == 0x7ff ? (elem_in ? kFixNanOut : kFixEmpty)
+                       : Em.e == 0 || !any           ? kFixEmpty
+                                                     : t + Em.e;
 #pragma unroll
         for (int i = 0; i < 12; ++i) U.m[i / 4][i % 4] = ups[i * NT];
         fix_join(Z, eo, U, Ms);

@@ -5,27 +5,37 @@
 // 153 FP64 operations per element of kv_column64.cuh are additions and products
 // by a few constants, so they are done on integers.  What floating point does
 // by the operation is done once per node, face and element here: a block of
-// values shares one exponent (that of its largest), and a block meets another
-// at the larger of the two exponents.
-//   node      3 components: |S| < 2^(57-k), one conversion by the FP64 pipe each
-//   face      4 nodes of a column at the exponent of the largest
-//   element   2 faces; mode operator, modulus (its mantissa as a 62-bit
-//             fraction, its exponent added to the block's)
+// values shares one exponent, and a block meets another at the larger of the two.
+//   node      3 components, each with its own exponent: |S| < 2^(57-k), exact
+//   face      4 nodes of a column; a component at the exponent of its largest
+//   element   2 faces; all components at one exponent, directly where theirs lie
+//             close, else as fix_modes says; mode operator, modulus (its
+//             mantissa as a 62-bit fraction, its exponent added to the block's)
 //   sum       with the element below, then over the 4 columns of a node;
 //             converted back to FP64 by its owner
-// Everything between is exact but for the products by constants and by the
-// modulus, which lose a few units of the last place, so the error of a block is
-// about 2^-57 of its largest input times the operator's norm: less than the
-// roundings of FP64 sums (2^-53 of every partial sum).  Against extended
-// precision (relative 2-norm; FP64 column kernel, then this): K u of a bending
-// field over graded moduli 3.3e-15, 5.6e-16, of a solved cantilever's u 5.8e-14,
-// 6.5e-15; the sensitivities 1.4e-15, 1.8e-16 and 2.3e-15, 4.3e-16.
+// Sums and differences are exact; alignments, products by constants and the
+// modulus lose a few units of the last place.  So a share of an element carries
+// an error of at most one FP64 rounding (2^-53) of each component's own largest value
+// in the element, and a few 2^-56 of the largest mode difference of any component,
+// times E.  A block without strain shifts nothing of its neighbours away, however
+// stiff it is.
 //
-// Measured on a GB300, y = K v, against the FP64 column kernel: 392 against
-// 1,973 us at 256 x 128 x 150, 54 against 232 at 55 x 55 x 165, 31 against 117 at
-// 120 x 60 x 30, 11 against 21 at 24 x 12 x 12 (cold L2).  About 1,100 instructions
-// per element and layer, issued on 55 % of the cycles; the rest waits for the
-// layer's barrier and for dependent results.
+// FP64 sums in the mode basis carry 2^-53 E times the components' largest
+// values, but where their sums happen to be exact: against extended precision
+// (relative 2-norm; FP64 column kernel, then this) K u of a bending field over
+// graded moduli 3.3e-15, 1.1e-16, of a solved cantilever's u 5.8e-14, 5.4e-15; the
+// sensitivities 1.4e-15, 1.3e-16 and 2.3e-15, 1.5e-16.  What FP64 keeps and this does not:
+// where one component's exact strain (a simple shear, a rigid rotation) exceeds another
+// component's by more than 2^4, the smaller force keeps 57 bits of the larger, not
+// of itself.  kv_column64.cuh serves callers for whom that matters
+// (mfto_set_kv_variant).
+//
+// Measured on a GB300, y = K v, against the FP64 column kernel: 52 (components of one
+// size) to 63 us (components far apart) against 229 at 55 x 55 x 165, 31 to 35
+// against 117 at 120 x 60 x 30, 8 to 10 against 18 at 24 x 12 x 12.  About 1,150
+// instructions per element and layer, 1,350 with components far apart, issued on
+// about half of the cycles; the rest waits for the layer's barrier and for
+// dependent results.
 #pragma once
 #include <math.h>
 #include <stdint.h>
@@ -44,11 +54,13 @@ FIX_HD FixConst fix_const(int64_t c62) {
   return {(int32_t)((c62 + 0x80000000ll) >> 32), (int32_t)(uint32_t)(uint64_t)c62};
 }
 
-// x c / 4 for |x| < 2^63: to within two units
+// x c / 4 for |x| < 2^63, to the nearest within a unit (errors of products do not
+// lean one way)
 FIX_HD int64_t fix_mul(int64_t x, FixConst c) {
   const uint32_t xl = (uint32_t)(uint64_t)x;
   const int32_t xh = (int32_t)(x >> 32);
-  const int64_t low = (int64_t)((uint64_t)xl * (uint32_t)c.hi) + (int64_t)xh * c.lo;
+  const int64_t low =
+      (int64_t)((uint64_t)xl * (uint32_t)c.hi + 0x80000000ull) + (int64_t)xh * c.lo;
   return (int64_t)xh * c.hi + (low >> 32);
 }
 FIX_HD int64_t fix_shl(int64_t x, int s) { return (int64_t)((uint64_t)x << s); }
@@ -75,30 +87,60 @@ bool fixed_op(double nu, double h, FixOp* op);   // host.cu
 FIX_HD int fix_min(int a, int b) { return a < b ? a : b; }
 FIX_HD int fix_max(int a, int b) { return a > b ? a : b; }
 
-// Exponents.  A node value is S 2^(e - 1079 + k), e the biased exponent of its
-// largest component, at least 64: what lies 64 or more below the exponent,
-// zeros and subnormals among it, becomes 0.  A value after the modulus is
+// Exponents.  A component of a node value is S 2^(e - 1079 + k), e its own biased
+// exponent.  A block's modes are X 2^(t - 1079 + k); a value after the modulus is
 // Z 2^(e - 2099 + k).
 constexpr int kFixMinE = 64;
-constexpr int kFixNan = 1 << 14;          // a block with an infinity or a NaN
+constexpr int kFixNan = 1 << 14;          // a component that is an infinity or a NaN
 constexpr int kFixEmpty = -(1 << 20);     // no contribution
 constexpr int kFixNanOut = 1 << 20;
 
-// four face modes (a + 2b) of three components and their exponent
+// x >> s for any s >= 0
+FIX_HD int64_t fix_sar(int64_t x, int s) {
+#ifdef __CUDA_ARCH__
+  int64_t r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));   // amounts above 63 count as 64
+  return r;
+#else
+  return x >> (s < 63 ? s : 63);
+#endif
+}
+
+// Exponents of three components in 16-bit lanes (0: the component is zero): the
+// first two in xy, the third in the low lane of z.
+struct FixExp {
+  uint32_t xy, z;
+  FIX_HD int at(int c) const { return (int)(c == 0 ? xy & 0xffffu : c == 1 ? xy >> 16 : z & 0xffffu); }
+};
+FIX_HD uint32_t fix_max_lanes(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+  return __vmaxu2(a, b);
+#else
+  const uint32_t l = 0xffffu;
+  return ((a & l) > (b & l) ? a & l : b & l) | ((a >> 16) > (b >> 16) ? a & ~l : b & ~l);
+#endif
+}
+
+// four face modes (a + 2b) of three components and the components' exponents
 struct FixFace {
+  int64_t m[3][4];
+  FixExp e;
+};
+
+// ... of a block of outputs, with one exponent
+struct FixOut {
   int64_t m[3][4];
   int e;
 };
 
-// the value with these bits at exponent e, to the nearest: its mantissa shifted left
-// by `left` (4 - k), right by what its own exponent lacks, negated by the sign.
+// the value with these bits at its own exponent: its mantissa shifted left by
+// `left` (4 - k), negated by the sign; values below 2^(kFixMinE - 1023) become 0.
 // On the integer pipes: the conversion of the FP64 pipe, in front of the
 // layer's barrier, made the warps wait.
-FIX_HD int64_t fix_value(uint64_t bits, int e, int left) {
-  const int sh = fix_min(e - (int)((bits >> 52) & 0x7ff), 63);
-  const int64_t m =
-      (((int64_t)(((bits & 0xfffffffffffffull) | 0x10000000000000ull) << (left + 1)) >> sh) + 1) >>
-      1;
+FIX_HD int64_t fix_value(uint64_t bits, int left) {
+  const int sh = fix_max(kFixMinE - (int)((bits >> 52) & 0x7ff), 0);
+  const int64_t m = fix_sar(
+      (int64_t)(((bits & 0xfffffffffffffull) | 0x10000000000000ull) << left), sh);
   const int64_t sign = (int64_t)bits >> 63;
   return (m ^ sign) - sign;
 }
@@ -116,17 +158,75 @@ FIX_HD void fix_face(const int64_t (&v)[4][3], FixFace& F) {
   }
 }
 
-// z stage: modes f + 4 (z difference) of the element between two faces shifted
-// right by dl and du; mode 0, a translation, is left out
-FIX_HD void fix_modes(const FixFace& lo, const FixFace& up, int dl, int du, int64_t (&X)[3][8]) {
+FIX_HD int fix_clz(uint32_t x) {
+#ifdef __CUDA_ARCH__
+  return __clz((int)x);
+#else
+  return x ? __builtin_clz(x) : 32;
+#endif
+}
+
+FIX_HD bool fix_nan(const FixExp& e) {
+  return fix_max(e.at(0), fix_max(e.at(1), e.at(2))) >= kFixNan;
+}
+
+// Whether the components' exponents lie so far apart that a common one would
+// cost a component bits that FP64 holds (4 - k are spare).
+FIX_HD bool fix_apart(const FixExp& e, int k) {
+  const int a = e.at(0), b = e.at(1), c = e.at(2), m = fix_max(a, fix_max(b, c)) - 4 + k;
+  return (a != 0 && a < m) || (b != 0 && b < m) || (c != 0 && c < m);
+}
+
+// z stage: modes f + 4 (z difference) of the element between two faces (e: their
+// larger exponents); mode 0, a translation, is left out.  Returns the modes'
+// common exponent (kFixEmpty: all zero).  each: form the modes of a component at
+// its own exponent, where a common translation leaves exact zeros and what
+// another component holds costs nothing, and then shift it to the exponent of
+// the largest mode there is: what is lost lies 2^-57 or 2^-56 below that, not
+// below the largest displacement.  |X| < 2^58 then (2^57 with k = 2): the modes' worst
+// sum over a node of two elements, 9.3, 15.1 and 27.1 |X| for k = 0, 1 and 2
+// after the quarter of fix_operator, stays below 2^62.
+FIX_HD int fix_modes(const FixFace& lo, const FixFace& up, const FixExp& e, bool each, int k,
+                     int64_t (&X)[3][8]) {
+  const int common = fix_max(e.at(0), fix_max(e.at(1), e.at(2)));
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
+  for (int c = 0; c < 3; ++c) {
+    const int at = each ? e.at(c) : common, dl = at - lo.e.at(c), du = at - up.e.at(c);
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      const int64_t a = lo.m[c][f] >> dl, b = up.m[c][f] >> du;
+      const int64_t a = fix_sar(lo.m[c][f], dl), b = fix_sar(up.m[c][f], du);
       X[c][f] = f == 0 ? 0 : a + b;
       X[c][f | 4] = b - a;
     }
+  }
+  if (!each) return common;
+  const int head = k > 1 ? 7 : 6;         // leading sign bits left
+  int t = kFixEmpty;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    uint32_t big = 0;
+#pragma unroll
+    for (int m = 1; m < 8; ++m) {
+      const int32_t hi = (int32_t)(X[c][m] >> 32);
+      big |= (uint32_t)(hi ^ (hi >> 31));
+    }
+    int z = fix_clz(big);
+    if (big == 0) {                       // below 2^32, or no modes at all
+      uint32_t low = 0;
+#pragma unroll
+      for (int m = 1; m < 8; ++m) low |= (uint32_t)(X[c][m] ^ (X[c][m] >> 63));
+      z = low != 0 ? 32 + fix_clz(low) : 1 << 16;
+    }
+    t = fix_max(t, e.at(c) + head - z);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    // (zero modes may be shifted by any amount)
+    const int net = e.at(c) - t, l = fix_min(fix_max(net, 0), 63), r = fix_max(-net, 0);
+#pragma unroll
+    for (int m = 1; m < 8; ++m) X[c][m] = fix_sar(fix_shl(X[c][m], l), r);
+  }
+  return t;
 }
 
 // The modulus: fraction in [1/2, 1) and exponent e (0: zero or below FP64's
@@ -144,6 +244,18 @@ FIX_HD FixModulus fix_modulus(uint64_t bits) {
   E.f62 = E.e == 0 ? 0 : (int64_t)(((bits & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
   E.f = fix_const(E.f62);
   return E;
+}
+
+// Whether there is any strain: the modes but for the rotations in them.  (Asked of
+// the modes: kept for the operator's results it would hold all of them at once.)
+FIX_HD bool fix_strained(const int64_t (&X)[3][8]) {
+  int64_t any = (X[0][2] + X[1][1]) | (X[0][4] + X[2][1]) | (X[1][4] + X[2][2]);
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int m = 1; m < 8; ++m)
+      if (m == 1 << c || (m & (m - 1)) != 0) any |= X[c][m];
+  return any != 0;
 }
 
 // Z = E Kt X / 4 in the units above
@@ -180,14 +292,14 @@ FIX_HD void fix_operator(const int64_t (&X)[3][8], const FixOp& K, const FixModu
 
 // Undone z stage and the sum with the element below: Ms = upper outputs of the
 // element below (U) + this one's lower ones; U becomes this one's upper ones.
-FIX_HD void fix_join(const int64_t (&Z)[3][8], int e, FixFace& U, FixFace& Ms) {
-  const int em = fix_max(U.e, e), du = fix_min(em - U.e, 63), dz = fix_min(em - e, 63);
+FIX_HD void fix_join(const int64_t (&Z)[3][8], int e, FixOut& U, FixOut& Ms) {
+  const int em = fix_max(U.e, e), du = em - U.e, dz = em - e;
 #pragma unroll
   for (int c = 0; c < 3; ++c)
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const int64_t s = f == 0 ? 0 : Z[c][f], d = Z[c][f | 4];
-      Ms.m[c][f] = (U.m[c][f] >> du) + ((s - d) >> dz);
+      Ms.m[c][f] = fix_sar(U.m[c][f], du) + fix_sar(s - d, dz);
       U.m[c][f] = s + d;
     }
   Ms.e = em;
@@ -195,7 +307,7 @@ FIX_HD void fix_join(const int64_t (&Z)[3][8], int e, FixFace& U, FixFace& Ms) {
 }
 
 // Shares of a column's four edges' nodes (a + 2b) from face modes.
-FIX_HD void fix_corners(const FixFace& M, int64_t (&w)[4][3]) {
+FIX_HD void fix_corners(const FixOut& M, int64_t (&w)[4][3]) {
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const int64_t s0 = M.m[c][0] - M.m[c][2], d0 = M.m[c][1] - M.m[c][3];
@@ -218,23 +330,6 @@ struct FixSquares {
   }
   FIX_HD int64_t sum() const { return h + ((l + (1ll << 30)) >> 31); }
 };
-
-FIX_HD int fix_clz(uint32_t x) {
-#ifdef __CUDA_ARCH__
-  return __clz((int)x);
-#else
-  return x ? __builtin_clz(x) : 32;
-#endif
-}
-
-// x c / 4 to the nearest, for sums whose errors must not lean one way
-FIX_HD int64_t fix_mul_near(int64_t x, FixConst c) {
-  const uint32_t xl = (uint32_t)(uint64_t)x;
-  const int32_t xh = (int32_t)(x >> 32);
-  const int64_t low =
-      (int64_t)((uint64_t)xl * (uint32_t)c.hi + 0x80000000ull) + (int64_t)xh * c.lo;
-  return (int64_t)xh * c.hi + (low >> 32);
-}
 
 // X . Kt X in units of 2^(64 - 2 shift) (h mu / 2) of the modes' unit squared.
 // With the sums of fix_operator the 45 terms are 23 squares in five classes.
@@ -284,8 +379,8 @@ FIX_HD int64_t fix_energy(const int64_t (&X)[3][8], const FixOp& K, int& shift) 
 #pragma unroll
   for (int n = 3; n < 12; ++n) one.add(v[n]);
   // the classes at most 24, 9, 12, 12 and 3 times 2^56 (a quarter with k > 0)
-  return one.sum() + 2 * own.sum() + fix_shl(fix_mul_near(div.sum(), K.r), K.sr) +
-         fix_shl(fix_mul_near(lin.sum(), K.r3), K.s3) +
-         fix_shl(fix_mul_near(third.sum(), K.third), 2) +
-         fix_shl(fix_mul_near(bil.sum(), K.q), K.s3);
+  return one.sum() + 2 * own.sum() + fix_shl(fix_mul(div.sum(), K.r), K.sr) +
+         fix_shl(fix_mul(lin.sum(), K.r3), K.s3) +
+         fix_shl(fix_mul(third.sum(), K.third), 2) +
+         fix_shl(fix_mul(bil.sum(), K.q), K.s3);
 }

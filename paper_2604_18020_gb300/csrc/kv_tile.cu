@@ -91,7 +91,8 @@ pcg_kv_col64_kernel(const double* __restrict__ E, const double* __restrict__ z,
     pcg_alpha(s, tot[0]);
 }
 
-// FP64 in fixed point (kv_column_fixed.cuh), the operator of nu in [0, 0.454).
+// FP64 in fixed point (kv_column_fixed.cuh), the operator of nu in [0, 0.454) with
+// variants 0 and 1.
 template <int CX, int CY>
 __global__ void __launch_bounds__(CX * CY, kFixThreads / (CX * CY))
 kv_fixed_kernel(const double* __restrict__ E, const double* __restrict__ v,
@@ -144,7 +145,7 @@ Col64Tiling col64_tiling(const mfto_handle* h, int nzc) {
 
 // tile shape and z-chunk of the FP64 column kernel in use
 void col64_tile(const mfto_handle* h, const Grid& g, int* shape, int* nzc, int copies) {
-  if (h->fix_ok)
+  if (fixed_route(h))
     fixed_choose(g.nx, g.ny, g.nz, h->num_sms, shape, nzc, copies);
   else
     col64_choose(1, g.nx, g.ny, g.nz, 1.5, h->num_sms, shape, nzc, copies);
@@ -155,7 +156,7 @@ mfto_status col64_attrs(mfto_handle* h) {
   for (int i = 0; i < kCol64Shapes; ++i) {
     const mfto_status s = col64_dispatch(i, [&](auto shape) -> mfto_status {
       using S = decltype(shape);
-      const bool fix = h->fix_ok;
+      const bool fix = fixed_route(h);
       const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
       const void* plain = fix ? (const void*)kv_fixed_kernel<S::CX, S::CY>
                               : (const void*)kv_col64_kernel<S::CX, S::CY>;
@@ -407,7 +408,7 @@ ColTiling col_launch_tiling(const mfto_handle* h, int per_sm, int* grid) {
 }
 
 // The FP64 column kernel's tiles and attributes, for the operator of the current
-// parameters.
+// parameters and the route in use.
 mfto_status kv_tile_retile(mfto_handle* h) {
   col64_tile(h, make_grid(h->mesh), &h->col64_shape, &h->col64_nzc, 1);
   return col64_attrs(h);
@@ -536,7 +537,7 @@ static mfto_status col64_launch(mfto_handle* h, const double* E, const double* v
   const mfto_status s = col64_dispatch(shape, [&](auto sh) -> mfto_status {
     using S = decltype(sh);
     const Col64Tiling tl = col64_tiling<S>(h, nzc);
-    if (h->fix_ok) {
+    if (fixed_route(h)) {
       kv_fixed_kernel<S::CX, S::CY>
           <<<dim3(tl.count(), nrhs), S::NT, fixed_smem<S::CX, S::CY>(), st>>>(
               E, v, y, h->d_fixed, h->fix, make_grid(h->mesh), tl, (int)h->n_dof);
@@ -642,7 +643,7 @@ mfto_status pcg_kv_tile_launch<double>(mfto_handle* h, const double* E, const do
     const Col64Tiling tl = col64_tiling<S>(h, h->col64_nzc);
     if (tl.count() > MFTO_RED_SLOTS)
       return mfto_fail(h, MFTO_TOO_LARGE, "mesh too large for the K.v tiling");
-    if (h->fix_ok) {
+    if (fixed_route(h)) {
       pcg_kv_fixed_kernel<S::CX, S::CY>
           <<<tl.count(), S::NT, pcg_fixed_smem<S::CX, S::CY>(), st>>>(
               E, z, p_old, p_new, q, h->d_fixed, h->fix, make_grid(h->mesh), tl, s, partials);

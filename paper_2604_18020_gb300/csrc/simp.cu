@@ -152,7 +152,7 @@ compliance_fixed_kernel(const double* __restrict__ rho, const double* __restrict
   const int kb = bz * tl.nzc, ke = min(kb + tl.nzc, g.nelz);   // element layers [kb, ke)
   const Col64LoadPlain ld{u};
   double* words = reinterpret_cast<double*>(smem_raw);
-  St st(words, reinterpret_cast<int*>(words + St::kWords), ld, nullptr, g, bx * CX, by * CY, ke,
+  St st(words, reinterpret_cast<uint2*>(words + St::kWords), ld, nullptr, g, bx * CX, by * CY, ke,
         K.k);
   const int gi = bx * CX + threadIdx.x % CX, gj = by * CY + threadIdx.x / CX;
   const bool in = gi < g.nelx && gj < g.nely;
@@ -178,13 +178,13 @@ compliance_fixed_kernel(const double* __restrict__ rho, const double* __restrict
     __syncthreads();
     if (!warp_in) return;
     st.face(ez + 1, up);
-    const int em = max(lo.e, up.e);
     int64_t X[3][8];
-    fix_modes(lo, up, min(em - lo.e, 63), min(em - up.e, 63), X);
+    const FixExp both{fix_max_lanes(lo.e.xy, up.e.xy), fix_max_lanes(lo.e.z, up.e.z)};
+    const int t = fix_modes(lo, up, both, __any_sync(0xffffffffu, fix_apart(both, K.k)), K.k, X);
     int shift;
     const double e = __ll2double_rn(fix_energy(X, K, shift));
-    const double ce = em >= kFixNan ? __longlong_as_double(0x7ff8000000000000ll)
-                                    : fix_scaled(e, 2 * (em - 1079 + K.k - shift) + 64, K);
+    const double ce = fix_nan(both) ? __longlong_as_double(0x7ff8000000000000ll)
+                                   : fix_scaled(e, 2 * (t - 1079 + K.k - shift) + 64, K);
     if (in) element(r, ce, ez);
   };
   for (int ez = kb; ez < ke; ez += 2) {
@@ -202,7 +202,7 @@ compliance_fixed_kernel(const double* __restrict__ rho, const double* __restrict
 template <typename S>
 constexpr size_t energy_smem() {
   using St = FixStream<S::CX, S::CY, Col64LoadPlain, false>;
-  return 8 * (size_t)St::kWords + 4 * (size_t)St::kExp;
+  return 8 * (size_t)(St::kWords + St::kExp);
 }
 
 // OC with bisection on lambda.  The candidate of a midpoint lambda is, per
@@ -761,7 +761,7 @@ mfto_status compliance_launch(mfto_handle* h, const double* rho, const double* u
     tl.tz = (g.nelz + tl.nzc - 1) / tl.nzc;
     if (tl.count() > MFTO_RED_SLOTS)
       return mfto_fail(h, MFTO_TOO_LARGE, "mesh too large for the compliance tiling");
-    if (h->fix_ok) {
+    if (fixed_route(h)) {
       compliance_fixed_kernel<S::CX, S::CY><<<tl.count(), S::NT, energy_smem<S>(), h->stream>>>(
           rho, u, dc, h->fix, g, tl, h->p.E0, h->p.Emin, h->p.penal, pow_plan(h->p.penal),
           h->d_misc, h->d_partials);
