@@ -96,7 +96,7 @@ struct FixStream {
         v[c] = ((fm >> c) & 1) ? 0.0 : ld.combine(r);
         const int hi = __double2hiint(v[c]) & 0x7fffffff;
         const bool finite = hi < 0x7ff00000, zero = (hi | __double2loint(v[c])) == 0;
-        e[c] = zero ? 0u : finite ? (uint32_t)max(hi >> 20, kFixMinE) : (uint32_t)kFixNan;
+        e[c] = zero ? 0u : finite ? (uint32_t)max(hi >> 20, 1) : (uint32_t)kFixNan;
         N[c * NV] = finite ? fix_value((uint64_t)__double_as_longlong(v[c]), left) : 0ll;
       }
       const int slot = L & 3;
@@ -272,7 +272,7 @@ __device__ __forceinline__ double kv_column_fixed_body(const double* __restrict_
         const bool nan = fix_nan(e);
         const int t = fix_modes(Flo, Fup, e, __any_sync(0xffffffffu, fix_apart(e, K.k)), K.k, X);
         // (by a vote: the answer is then formed here, before the operator needs the
-        // modes' registers; 68 bytes spilled instead of 144)
+        // modes' registers)
         const unsigned strained = __ballot_sync(0xffffffffu, fix_strained(X));
         const FixModulus Em = fix_modulus(Ebits);
         fix_operator(X, K, Em, Z);
@@ -285,7 +285,7 @@ __device__ __forceinline__ double kv_column_fixed_body(const double* __restrict_
         // a block that holds nothing shifts no neighbour's bits away
         const bool any = (strained >> (tid & 31)) & 1u;
         const int eo = nan || Em.e == 0x7ff ? (elem_in ? kFixNanOut : kFixEmpty)
-                       : Em.e == 0 || !any           ? kFixEmpty
+                       : Em.f62 == 0 || !any         ? kFixEmpty
                                                      : t + Em.e;
 #pragma unroll
         for (int i = 0; i < 12; ++i) U.m[i / 4][i % 4] = ups[i * NT];

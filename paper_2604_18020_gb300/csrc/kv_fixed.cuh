@@ -88,9 +88,8 @@ FIX_HD int fix_min(int a, int b) { return a < b ? a : b; }
 FIX_HD int fix_max(int a, int b) { return a > b ? a : b; }
 
 // Exponents.  A component of a node value is S 2^(e - 1079 + k), e its own biased
-// exponent.  A block's modes are X 2^(t - 1079 + k); a value after the modulus is
+// exponent (1 for subnormals).  A block's modes are X 2^(t - 1079 + k); a value after the modulus is
 // Z 2^(e - 2099 + k).
-constexpr int kFixMinE = 64;
 constexpr int kFixNan = 1 << 14;          // a component that is an infinity or a NaN
 constexpr int kFixEmpty = -(1 << 20);     // no contribution
 constexpr int kFixNanOut = 1 << 20;
@@ -134,13 +133,11 @@ struct FixOut {
 };
 
 // the value with these bits at its own exponent: its mantissa shifted left by
-// `left` (4 - k), negated by the sign; values below 2^(kFixMinE - 1023) become 0.
-// On the integer pipes: the conversion of the FP64 pipe, in front of the
-// layer's barrier, made the warps wait.
+// `left` (4 - k), negated by the sign.  On the integer pipes: the conversion of
+// the FP64 pipe, in front of the layer's barrier, made the warps wait.
 FIX_HD int64_t fix_value(uint64_t bits, int left) {
-  const int sh = fix_max(kFixMinE - (int)((bits >> 52) & 0x7ff), 0);
-  const int64_t m = fix_sar(
-      (int64_t)(((bits & 0xfffffffffffffull) | 0x10000000000000ull) << left), sh);
+  const uint64_t one = (bits << 1) >> 53 ? 0x10000000000000ull : 0ull;   // subnormals have none
+  const int64_t m = (int64_t)(((bits & 0xfffffffffffffull) | one) << left);
   const int64_t sign = (int64_t)bits >> 63;
   return (m ^ sign) - sign;
 }
@@ -171,10 +168,11 @@ FIX_HD bool fix_nan(const FixExp& e) {
 }
 
 // Whether the components' exponents lie so far apart that a common one would
-// cost a component bits that FP64 holds (4 - k are spare).
+// cost a component bits that FP64 holds (4 - k are spare), or so low that the
+// values may be subnormals, which fill fewer bits.
 FIX_HD bool fix_apart(const FixExp& e, int k) {
-  const int a = e.at(0), b = e.at(1), c = e.at(2), m = fix_max(a, fix_max(b, c)) - 4 + k;
-  return (a != 0 && a < m) || (b != 0 && b < m) || (c != 0 && c < m);
+  const int a = e.at(0), b = e.at(1), c = e.at(2), top = fix_max(a, fix_max(b, c)), m = top - 4 + k;
+  return (a != 0 && a < m) || (b != 0 && b < m) || (c != 0 && c < m) || (uint32_t)(top - 1) < 63u;
 }
 
 // z stage: modes f + 4 (z difference) of the element between two faces (e: their
@@ -229,8 +227,7 @@ FIX_HD int fix_modes(const FixFace& lo, const FixFace& up, const FixExp& e, bool
   return t;
 }
 
-// The modulus: fraction in [1/2, 1) and exponent e (0: zero or below FP64's
-// normal range, taken as zero).
+// The modulus: fraction in [1/2, 1) (0: zero) and exponent e (0x7ff: no number).
 struct FixModulus {
   FixConst f;
   int64_t f62;
@@ -241,7 +238,16 @@ FIX_HD FixModulus fix_modulus(uint64_t bits) {
   FixModulus E;
   E.negative = (bits >> 63) != 0;
   E.e = (int)((bits >> 52) & 0x7ff);
-  E.f62 = E.e == 0 ? 0 : (int64_t)(((bits & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
+  uint64_t m = (bits & 0xfffffffffffffull) << 9;
+  if (E.e != 0) {
+    m |= 1ull << 61;
+  } else if (m != 0) {                    // subnormal: its leading bit to where the others have it
+    const uint32_t hi = (uint32_t)(m >> 32);
+    const int up = (hi != 0 ? fix_clz(hi) : 32 + fix_clz((uint32_t)m)) - 2;
+    m <<= up;
+    E.e = 1 - up;
+  }
+  E.f62 = (int64_t)m;
   E.f = fix_const(E.f62);
   return E;
 }

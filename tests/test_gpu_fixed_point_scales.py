@@ -104,3 +104,32 @@ def test_variant_2_runs_on_the_fp64_pipe(cuda, nu):
         h.set_kv_variant(0)
         h.kv(tE, tv, y)
         assert torch.equal(y, first)
+
+
+# powers of two: inputs are whole numbers times 2^low, the reference is formed at 2^0
+@pytest.mark.parametrize("low", [-1074, -1060, -1040, -1000, -960, -900])
+def test_kv_lower_end_values(cuda, low):
+    m = W.Mesh(*SHAPE)
+    E = np.random.default_rng(27).uniform(0.1, 1.0, m.n_elem)
+    whole = np.random.default_rng(28).integers(-2 ** 30, 2 ** 30, m.n_dof).astype(np.float64)
+    whole[::7] %= 5.0            # small ones among them
+    none = np.zeros(m.n_node, np.uint8)
+    fd = fem.dof_mask(none)
+    got = _kv(cuda, SHAPE, none, 0.3, E, np.ldexp(whole, low))
+    ref = fem.kv(fem.ke_exact(), E, fem.edof_table_fast(*SHAPE), whole, fd)
+    err = np.abs(np.ldexp(np.ldexp(got, 500), -low - 500) - ref)
+    # half a unit of the last subnormal place where the result is subnormal
+    assert np.all(err <= 2.0 ** -48 * _bound(SHAPE, 0.3, E, whole, fd) + np.ldexp(0.51, -1074 - low))
+
+
+@pytest.mark.parametrize("low", [-1074, -1060, -1030, -1000])
+def test_kv_lower_end_moduli(cuda, low):
+    m = W.Mesh(*SHAPE)
+    whole = np.random.default_rng(29).integers(1, 2 ** 40, m.n_elem).astype(np.float64)
+    whole[::5] %= 7.0            # zeros and single bits among them
+    v = np.random.default_rng(30).uniform(-1.0, 1.0, m.n_dof)
+    none = np.zeros(m.n_node, np.uint8)
+    fd = fem.dof_mask(none)
+    got = np.ldexp(_kv(cuda, SHAPE, none, 0.3, np.ldexp(whole, low), np.ldexp(v, 900)), -900 - low)
+    ref = fem.kv(fem.ke_exact(), whole, fem.edof_table_fast(*SHAPE), v, fd)
+    assert np.all(np.abs(got - ref) <= 2.0 ** -48 * _bound(SHAPE, 0.3, whole, v, fd))
