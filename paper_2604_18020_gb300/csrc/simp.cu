@@ -86,45 +86,47 @@ compliance_kernel(const double* __restrict__ rho, const double* __restrict__ u,
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double sh[64];
   using S = Col64Shape<CX, CY>;
-  const int tile = blockIdx.x;
-  const int bx = tile % tl.tx, by = (tile / tl.tx) % tl.ty, bz = tile / (tl.tx * tl.ty);
-  const int kb = bz * tl.nzc, ke = min(kb + tl.nzc, g.nelz);   // element layers [kb, ke)
   const Col64LoadPlain ld{u};
-  Col64Stream<CX, CY, Col64LoadPlain> st(reinterpret_cast<double*>(smem_raw), ld, nullptr, g,
-                                         bx * CX, by * CY, ke);
-  const bool in = st.gi < g.nelx && st.gj < g.nely;
-  const bool warp_in = __any_sync(0xffffffffu, in);
-  const int e0 = st.gi + g.nelx * st.gj, nexy = g.nelx * g.nely;
   double acc[2] = {0.0, 0.0};
-  double own[3];
-  st.issue(kb);
-  st.issue(kb + 1);
-  col64_wait<1>();
-  st.stage(kb, 0u, own);
-  st.issue(kb + 2);
-  __syncthreads();
-  Col64Face F0, F1;
-  st.face(kb, F0);
-  const ElementEnergy element{E0, Emin, penal, plan, dc, e0, nexy, acc};
-  auto layer = [&](int ez, const Col64Face& lo, Col64Face& up) {
-    double r = 0.0;
-    if (in) r = rho[e0 + nexy * ez];
+  for (int tile = blockIdx.x; tile < tl.count(); tile += gridDim.x) {
+    const int bx = tile % tl.tx, by = (tile / tl.tx) % tl.ty, bz = tile / (tl.tx * tl.ty);
+    const int kb = bz * tl.nzc, ke = min(kb + tl.nzc, g.nelz);   // element layers [kb, ke)
+    Col64Stream<CX, CY, Col64LoadPlain> st(reinterpret_cast<double*>(smem_raw), ld, nullptr, g,
+                                           bx * CX, by * CY, ke);
+    const bool in = st.gi < g.nelx && st.gj < g.nely;
+    const bool warp_in = __any_sync(0xffffffffu, in);
+    const int e0 = st.gi + g.nelx * st.gj, nexy = g.nelx * g.nely;
+    double own[3];
+    st.issue(kb);
+    st.issue(kb + 1);
     col64_wait<1>();
-    st.stage(ez + 1, 0u, own);
-    st.issue(ez + 3);
+    st.stage(kb, 0u, own);
+    st.issue(kb + 2);
     __syncthreads();
-    if (!warp_in) return;
-    st.face(ez + 1, up);
-    double X[3][8];
-    col64_modes(lo, up, X);
-    const double ce = mode_energy(X, K);
-    if (in) element(r, ce, ez);
-  };
-  for (int ez = kb; ez < ke; ez += 2) {
-    layer(ez, F0, F1);
-    if (ez + 1 < ke) layer(ez + 1, F1, F0);
+    Col64Face F0, F1;
+    st.face(kb, F0);
+    const ElementEnergy element{E0, Emin, penal, plan, dc, e0, nexy, acc};
+    auto layer = [&](int ez, const Col64Face& lo, Col64Face& up) {
+      double r = 0.0;
+      if (in) r = rho[e0 + nexy * ez];
+      col64_wait<1>();
+      st.stage(ez + 1, 0u, own);
+      st.issue(ez + 3);
+      __syncthreads();
+      if (!warp_in) return;
+      st.face(ez + 1, up);
+      double X[3][8];
+      col64_modes(lo, up, X);
+      const double ce = mode_energy(X, K);
+      if (in) element(r, ce, ez);
+    };
+    for (int ez = kb; ez < ke; ez += 2) {
+      layer(ez, F0, F1);
+      if (ez + 1 < ke) layer(ez + 1, F1, F0);
+    }
+    col64_wait<0>();
+    __syncthreads();   // the next tile's stages write what this one's faces read
   }
-  col64_wait<0>();
   double tot[2];
   if (last_block_reduce<2>(acc, partials, &s->ticket, tot, sh) && threadIdx.x == 0) {
     s->sum[0] = tot[0];
@@ -147,51 +149,53 @@ compliance_fixed_kernel(const double* __restrict__ rho, const double* __restrict
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double sh[64];
   using St = FixStream<CX, CY, Col64LoadPlain, false>;
-  const int tile = blockIdx.x;
-  const int bx = tile % tl.tx, by = (tile / tl.tx) % tl.ty, bz = tile / (tl.tx * tl.ty);
-  const int kb = bz * tl.nzc, ke = min(kb + tl.nzc, g.nelz);   // element layers [kb, ke)
   const Col64LoadPlain ld{u};
   double* words = reinterpret_cast<double*>(smem_raw);
-  St st(words, reinterpret_cast<uint2*>(words + St::kWords), ld, nullptr, g, bx * CX, by * CY, ke,
-        K.k);
-  const int gi = bx * CX + threadIdx.x % CX, gj = by * CY + threadIdx.x / CX;
-  const bool in = gi < g.nelx && gj < g.nely;
-  const bool warp_in = __any_sync(0xffffffffu, in);
-  const int e0 = gi + g.nelx * gj, nexy = g.nelx * g.nely;
   double acc[2] = {0.0, 0.0};
-  const ElementEnergy element{E0, Emin, penal, plan, dc, e0, nexy, acc};
-  st.issue(kb);
-  st.issue(kb + 1);
-  col64_wait<1>();
-  st.stage(kb, 0u);
-  st.issue(kb + 2);
-  double r_next = in ? rho[e0 + nexy * kb] : 0.0;
-  __syncthreads();
-  FixFace F0, F1;
-  st.face(kb, F0);
-  auto layer = [&](int ez, const FixFace& lo, FixFace& up) {
-    const double r = r_next;
-    if (in && ez + 1 < ke) r_next = rho[e0 + nexy * (ez + 1)];
+  for (int tile = blockIdx.x; tile < tl.count(); tile += gridDim.x) {
+    const int bx = tile % tl.tx, by = (tile / tl.tx) % tl.ty, bz = tile / (tl.tx * tl.ty);
+    const int kb = bz * tl.nzc, ke = min(kb + tl.nzc, g.nelz);   // element layers [kb, ke)
+    St st(words, reinterpret_cast<uint2*>(words + St::kWords), ld, nullptr, g, bx * CX, by * CY, ke,
+          K.k);
+    const int gi = bx * CX + threadIdx.x % CX, gj = by * CY + threadIdx.x / CX;
+    const bool in = gi < g.nelx && gj < g.nely;
+    const bool warp_in = __any_sync(0xffffffffu, in);
+    const int e0 = gi + g.nelx * gj, nexy = g.nelx * g.nely;
+    const ElementEnergy element{E0, Emin, penal, plan, dc, e0, nexy, acc};
+    st.issue(kb);
+    st.issue(kb + 1);
     col64_wait<1>();
-    st.stage(ez + 1, 0u);
-    st.issue(ez + 3);
+    st.stage(kb, 0u);
+    st.issue(kb + 2);
+    double r_next = in ? rho[e0 + nexy * kb] : 0.0;
     __syncthreads();
-    if (!warp_in) return;
-    st.face(ez + 1, up);
-    int64_t X[3][8];
-    const FixExp both{fix_max_lanes(lo.e.xy, up.e.xy), fix_max_lanes(lo.e.z, up.e.z)};
-    const int t = fix_modes(lo, up, both, __any_sync(0xffffffffu, fix_apart(both, K.k)), K.k, X);
-    int shift;
-    const double e = __ll2double_rn(fix_energy(X, K, shift));
-    const double ce = fix_nan(both) ? __longlong_as_double(0x7ff8000000000000ll)
-                                   : fix_scaled(e, 2 * (t - 1079 + K.k - shift) + 64, K);
-    if (in) element(r, ce, ez);
-  };
-  for (int ez = kb; ez < ke; ez += 2) {
-    layer(ez, F0, F1);
-    if (ez + 1 < ke) layer(ez + 1, F1, F0);
+    FixFace F0, F1;
+    st.face(kb, F0);
+    auto layer = [&](int ez, const FixFace& lo, FixFace& up) {
+      const double r = r_next;
+      if (in && ez + 1 < ke) r_next = rho[e0 + nexy * (ez + 1)];
+      col64_wait<1>();
+      st.stage(ez + 1, 0u);
+      st.issue(ez + 3);
+      __syncthreads();
+      if (!warp_in) return;
+      st.face(ez + 1, up);
+      int64_t X[3][8];
+      const FixExp both{fix_max_lanes(lo.e.xy, up.e.xy), fix_max_lanes(lo.e.z, up.e.z)};
+      const int t = fix_modes(lo, up, both, __any_sync(0xffffffffu, fix_apart(both, K.k)), K.k, X);
+      int shift;
+      const double e = __ll2double_rn(fix_energy(X, K, shift));
+      const double ce = fix_nan(both) ? __longlong_as_double(0x7ff8000000000000ll)
+                                     : fix_scaled(e, 2 * (t - 1079 + K.k - shift) + 64, K);
+      if (in) element(r, ce, ez);
+    };
+    for (int ez = kb; ez < ke; ez += 2) {
+      layer(ez, F0, F1);
+      if (ez + 1 < ke) layer(ez + 1, F1, F0);
+    }
+    col64_wait<0>();
+    __syncthreads();
   }
-  col64_wait<0>();
   double tot[2];
   if (last_block_reduce<2>(acc, partials, &s->ticket, tot, sh) && threadIdx.x == 0) {
     s->sum[0] = tot[0];
@@ -759,16 +763,16 @@ mfto_status compliance_launch(mfto_handle* h, const double* rho, const double* u
     tl.ty = (g.nely + S::CY - 1) / S::CY;
     tl.nzc = h->energy_nzc;
     tl.tz = (g.nelz + tl.nzc - 1) / tl.nzc;
-    if (tl.count() > MFTO_RED_SLOTS)
-      return mfto_fail(h, MFTO_TOO_LARGE, "mesh too large for the compliance tiling");
+    // one partial per CTA: on wider meshes a CTA takes several tiles
+    const int grid = tl.count() < MFTO_RED_SLOTS ? tl.count() : MFTO_RED_SLOTS;
     if (fixed_route(h)) {
-      compliance_fixed_kernel<S::CX, S::CY><<<tl.count(), S::NT, energy_smem<S>(), h->stream>>>(
+      compliance_fixed_kernel<S::CX, S::CY><<<grid, S::NT, energy_smem<S>(), h->stream>>>(
           rho, u, dc, h->fix, g, tl, h->p.E0, h->p.Emin, h->p.penal, pow_plan(h->p.penal),
           h->d_misc, h->d_partials);
       return MFTO_OK;
     }
     compliance_kernel<S::CX, S::CY>
-        <<<tl.count(), S::NT, S::template stream_bytes<1>(), h->stream>>>(
+        <<<grid, S::NT, S::template stream_bytes<1>(), h->stream>>>(
             rho, u, dc, h->mc64, g, tl, h->p.E0, h->p.Emin, h->p.penal, pow_plan(h->p.penal),
             h->d_misc, h->d_partials);
     return MFTO_OK;
