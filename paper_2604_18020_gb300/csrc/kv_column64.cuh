@@ -452,6 +452,7 @@ mfto_status col64_dispatch(int i, const F& f) {
 static inline void col64_choose(int halo, int nx, int ny, int nz, double extra, int num_sms,
                                 int* shape_out, int* nzc_out, int copies = 1) {
   double best = 0.0;
+  bool best_fits = false;
   for (int i = 0; i < kCol64Shapes; ++i)
     col64_dispatch(i, [&](auto shape) -> mfto_status {
       using S = decltype(shape);
@@ -460,15 +461,17 @@ static inline void col64_choose(int halo, int nx, int ny, int nz, double extra, 
       for (int tz = 1; tz <= nz; ++tz) {
         const int nzc = (nz + tz - 1) / tz;
         if ((nz + nzc - 1) / nzc != tz) continue;          // not a balanced count
-        if (txy * tz > MFTO_RED_SLOTS && tz > 1) break;     // one partial per CTA
+        const bool fits = txy * tz <= MFTO_RED_SLOTS;       // one partial per CTA
+        if (!fits && tz > 1) break;
         constexpr int resident = kCol64Threads / S::NT;
         const double mean = (double)(txy * tz * copies) / num_sms;
         const int64_t ctas = (txy * tz * copies + num_sms - 1) / num_sms;
         const double busy = ctas > resident ? mean + 0.5 : (double)ctas;
         const double warps = (double)(ctas > resident ? resident : ctas) * S::NT / 32;
         const double cost = busy * S::NT * (nzc + extra) * (1.03 + 2.0 / warps);
-        if (best == 0.0 || cost < best) {
+        if (best == 0.0 || (fits == best_fits ? cost < best : fits)) {
           best = cost;
+          best_fits = fits;
           *shape_out = i;
           *nzc_out = nzc;
         }

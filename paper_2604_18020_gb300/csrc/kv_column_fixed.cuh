@@ -333,6 +333,7 @@ __device__ __forceinline__ double kv_column_fixed_body(const double* __restrict_
 static inline void fixed_choose(int nx, int ny, int nz, int num_sms, int* shape_out, int* nzc_out,
                                 int copies = 1) {
   double best = 0.0;
+  bool best_fits = false;
   for (int i = 0; i < kCol64Shapes; ++i)
     col64_dispatch(i, [&](auto shape) -> mfto_status {
       using S = decltype(shape);
@@ -340,7 +341,8 @@ static inline void fixed_choose(int nx, int ny, int nz, int num_sms, int* shape_
       for (int tz = 1; tz <= nz; ++tz) {
         const int nzc = (nz + tz - 1) / tz;
         if ((nz + nzc - 1) / nzc != tz) continue;          // not a balanced count
-        if (txy * tz > MFTO_RED_SLOTS && tz > 1) break;     // one partial per CTA
+        const bool fits = txy * tz <= MFTO_RED_SLOTS;       // one partial per CTA, first choice
+        if (!fits && tz > 1) break;
         constexpr int resident = kFixThreads / S::NT;
         const int64_t ctas = (txy * tz * copies + num_sms - 1) / num_sms;
         const int64_t sets = ctas / resident, rest = ctas % resident;
@@ -348,8 +350,9 @@ static inline void fixed_choose(int nx, int ny, int nz, int num_sms, int* shape_
         // larger CTAs wait longer at their barriers
         const double cost = ((double)sets * layer(resident) + layer(rest)) * (nzc + 1.3) *
                             (S::NT > 128 ? 1.05 : 1.0);
-        if (best == 0.0 || cost < best) {
+        if (best == 0.0 || (fits == best_fits ? cost < best : fits)) {
           best = cost;
+          best_fits = fits;
           *shape_out = i;
           *nzc_out = nzc;
         }

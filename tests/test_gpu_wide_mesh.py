@@ -3,7 +3,7 @@ partial sums (16,384), for the operator in fixed point and on the FP64 pipe."""
 import numpy as np
 import pytest
 
-from oracle import fem
+from oracle import fem, solve
 
 pytestmark = pytest.mark.gpu
 
@@ -31,3 +31,27 @@ def test_compliance_on_wide_meshes(cuda, shape, nu):
         assert (dc - ref).abs().max().item() <= 1e-13 * abs(ref)
         E = 1e-9 + (1.0 - 1e-9) * 0.125
         assert abs(total - h.n_elem * E * ce) <= 1e-11 * h.n_elem * E * ce
+
+
+@pytest.mark.parametrize("nu", [0.3, 0.47, -0.2])
+def test_pcg_on_wide_meshes(cuda, nu):
+    """Two FP64 CG iterations against the oracle's recurrence: the CG operator takes
+    a tile shape that leaves at most 16,384 partial sums."""
+    import torch
+    from paper_2604_18020_gb300 import mfto
+    shape = (1400, 1400, 1)
+    nx, ny, nz = (s + 1 for s in shape)
+    fixed = np.zeros(nx * ny * nz, np.uint8)
+    fixed[::nx] = 7
+    fd = fem.dof_mask(fixed)
+    rng = np.random.default_rng(31)
+    E = rng.uniform(0.5, 1.0, shape[0] * shape[1] * shape[2])
+    f = np.where(fd, 0.0, rng.uniform(-1.0, 1.0, 3 * fixed.size))
+    KE, edof = fem.ke_exact(1.0, nu), fem.edof_table_fast(*shape)
+    d = fem.jacobi_diag(KE, E, edof, fd)
+    u, _ = solve.pcg(lambda v: fem.kv(KE, E, edof, v, fd), d, f, np.zeros_like(f), 1e-8, 2)
+    with mfto.Handle(*shape, fixed, mfto.default_params(nu=nu, maxit=2, check_every=2)) as h:
+        got = torch.zeros(h.n_dof, dtype=torch.float64, device=cuda)
+        st = h.pcg(torch.tensor(E, device=cuda), torch.tensor(f, device=cuda), got)
+        assert st.status == mfto.NOT_CONVERGED and st.iterations == 2
+    assert np.abs(got.cpu().numpy() - u).max() <= 1e-12 * np.abs(u).max()
