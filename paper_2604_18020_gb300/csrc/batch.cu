@@ -92,7 +92,7 @@ struct mfto_batch {
   BatchCtl* d_ctl;
   BatchCtl* h_ctl;
   double* d_part_a;                // [2][max blocks]
-  float2 *d_share_a, *d_share_b;   // inner CG: [cg_tiles], [2][cg_updates]
+  double *d_share_a, *d_share_b;   // inner CG: [cg_tiles], [2][cg_updates]
   double* d_res;                   // [2 * count] outer residual sums
   int* d_mask;                     // [count] 1 = instance converged/stopped
   double* d_rzp;                   // [count] r.z of a continued direction (0: p = z)
@@ -614,8 +614,8 @@ mfto_status make_tiles(mfto_batch* b) {
   if (s == MFTO_OK)
     s = put((void**)&b->d_tile64_inst, tile64_inst.data(), 4 * tile64_inst.size());
   if (s != MFTO_OK) return s;
-  if (cudaMalloc(&b->d_share_a, sizeof(float2) * b->cg_tiles) != cudaSuccess ||
-      cudaMalloc(&b->d_share_b, sizeof(float2) * 2 * b->cg_updates) != cudaSuccess) {
+  if (cudaMalloc(&b->d_share_a, sizeof(double) * b->cg_tiles) != cudaSuccess ||
+      cudaMalloc(&b->d_share_b, sizeof(double) * 2 * b->cg_updates) != cudaSuccess) {
     cudaGetLastError();
     return MFTO_OOM;
   }

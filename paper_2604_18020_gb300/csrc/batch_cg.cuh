@@ -48,53 +48,45 @@ struct BatchScal {
   int32_t it, done, status, pad;
 };
 
-// Sums of an instance's n shares (rows `stride` apart), fixed order; the
-// calling warp's lane 0 gets them.
+// The dot products: a warp's sums as FP32 pairs (DotAcc<float>), from there on in
+// FP64, where the chains of dependent operations are what they cost (an FP64
+// instruction takes a warp 64 clocks): a lane per row and warp, short trees.
+//
+// Sums of an instance's n shares in K (1 or 2) rows `stride` apart, fixed order,
+// by 32 / K lanes of the calling warp each; all its lanes get them.
 template <int K>
-__device__ __forceinline__ void batch_sum(const float2* part, int stride, int n,
+__device__ __forceinline__ void batch_sum(const double* part, int stride, int n,
                                           double (&out)[K]) {
+  constexpr int W = 32 / K;
   const int lane = threadIdx.x & 31;
-  DFloat t[K];
+  const double* row = part + lane / W * stride;
+  double t = 0.0;
+  for (int b = lane % W; b < n; b += W) t += row[b];
 #pragma unroll
-  for (int c = 0; c < K; ++c) t[c] = DFloat{0.f, 0.f};
-  for (int b = lane; b < n; b += 32) {
+  for (int o = W / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
 #pragma unroll
-    for (int c = 0; c < K; ++c) {
-      const float2 x = part[c * stride + b];
-      t[c] = df_add(t[c], DFloat{x.x, x.y});
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < K; ++c) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      DFloat v;
-      v.hi = __shfl_down_sync(0xffffffffu, t[c].hi, o);
-      v.lo = __shfl_down_sync(0xffffffffu, t[c].lo, o);
-      t[c] = df_add(t[c], v);
-    }
-    out[c] = (double)t[c].hi + (double)t[c].lo;
-  }
+  for (int c = 0; c < K; ++c) out[c] = __shfl_sync(0xffffffffu, t, c * W);
 }
 
-// The block's sums of K double-float values held by lane 0 of each warp, as
-// share `at` of its rows.
+// The block's sums of K double-float values held by lane 0 of each warp, in FP64,
+// as share `at` of its rows.
 template <int K>
-__device__ __forceinline__ void batch_publish(const DFloat (&v)[K], float2* part, int stride,
+__device__ __forceinline__ void batch_publish(const DFloat (&v)[K], double* part, int stride,
                                               int at) {
-  __shared__ float2 sh[K][MFTO_BLOCK / 32];
+  constexpr int W = MFTO_BLOCK / 32;
+  __shared__ float2 sh[K * W];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) {
 #pragma unroll
-    for (int c = 0; c < K; ++c) sh[c][warp] = make_float2(v[c].hi, v[c].lo);
+    for (int c = 0; c < K; ++c) sh[c * W + warp] = make_float2(v[c].hi, v[c].lo);
   }
   __syncthreads();
-  if (threadIdx.x < K) {
-    const int c = threadIdx.x;
-    DFloat t{sh[c][0].x, sh[c][0].y};
+  if (warp == 0) {
+    const float2 x = sh[lane % (K * W)];
+    double t = (double)x.x + (double)x.y;
 #pragma unroll
-    for (int i = 1; i < MFTO_BLOCK / 32; ++i) t = df_add(t, DFloat{sh[c][i].x, sh[c][i].y});
-    part[c * stride + at] = make_float2(t.hi, t.lo);
+    for (int o = W / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane < K * W && lane % W == 0) part[lane / W * stride + at] = t;
   }
 }
 
@@ -128,8 +120,8 @@ struct BatchCgArgs {
   const int* tile_inst;       // instance of a tile
   const BatchScal* prev;      // scalars of iteration k - 1
   BatchScal* cur;             // ... and k
-  const float2* part_b;       // r.z and r.r of the update CTAs, rows n_update apart
-  float2* part_a;             // p.q of the tiles
+  const double* part_b;       // r.z and r.r of the update CTAs, rows n_update apart
+  double* part_a;             // p.q of the tiles
   int n_update, maxit;
   double rtol2;
 };
@@ -373,8 +365,8 @@ __global__ void __launch_bounds__(MFTO_BLOCK)
 batch_cg_update(float* __restrict__ u, const float* __restrict__ p, const float* __restrict__ q,
                 float* __restrict__ r, float* __restrict__ z, const float* __restrict__ dinv,
                 const BatchInst* __restrict__ inst, const BatchTiles* __restrict__ tiles,
-                const int* __restrict__ up_inst, BatchScal* sc, const float2* part_a,
-                float2* part_b, int n_update) {
+                const int* __restrict__ up_inst, BatchScal* sc, const double* part_a,
+                double* part_b, int n_update) {
   constexpr int N = kBatchUpdate / MFTO_BLOCK;
   __shared__ float s_alpha;
   __shared__ int s_skip;
@@ -441,7 +433,7 @@ __global__ void __launch_bounds__(MFTO_BLOCK)
 batch_cg_start(const float* __restrict__ r, float* __restrict__ z, const float* __restrict__ dinv,
                const BatchInst* __restrict__ inst, const BatchTiles* __restrict__ tiles,
                const int* __restrict__ up_inst, BatchScal* sc, const double* __restrict__ rz_prev,
-               float2* part_b, int n_update) {
+               double* part_b, int n_update) {
   const int i = up_inst[blockIdx.x];
   const int up0 = tiles[i].up0;
   const int n = 3 * inst[i].nx * inst[i].ny * inst[i].nz;
