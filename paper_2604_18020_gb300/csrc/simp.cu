@@ -395,7 +395,9 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
     f = make_float2(oc_f32(a), oc_f32(r));
     const float lo = fmaxf(0.f, f.y - movef);
     sum_lo += lo;
-    sum_hi += f.x > 0.f ? fminf(1.f, f.y + movef) : lo;
+    // (a by its bits: its copy may be 0; a candidate that is no number counts as
+    // the upper bound)
+    sum_hi += __double_as_longlong(a) > 0 || f.x != f.x ? fminf(1.f, f.y + movef) : lo;
     sum_a += f.x;
   };
   if constexpr (G > 0) {

@@ -1,0 +1,34 @@
+"""The OC update where FP32 copies of its values could mislead it, against the
+oracle's bisection (design 1e-9, multiplier 4e-10, as in test_gpu_design_edges.py):
+sensitivities whose candidates underflow FP32."""
+import numpy as np
+import pytest
+
+from oracle import simp as osimp
+from paper_2604_18020_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+SMALL, LARGE = (24, 13, 11), (100, 100, 63)
+
+
+def _check(cuda, shape, rho, dc, volfrac, move, lam_tol=4e-10):
+    import torch
+    from paper_2604_18020_gb300 import mfto
+    ref, info = osimp.oc_update(rho, dc, volfrac, move)
+    m = W.Mesh(*shape)
+    with mfto.Handle(*shape, np.zeros(m.n_node, np.uint8),
+                     mfto.default_params(volfrac=volfrac, move=move)) as h:
+        out = torch.empty(m.n_elem, dtype=torch.float64, device=cuda)
+        st = h.oc_update(torch.tensor(rho, device=cuda), torch.tensor(dc, device=cuda), out)
+    got = out.cpu().numpy()
+    assert np.abs(got - ref).max() <= 1e-9
+    assert abs(st.change - info["change"]) <= 1e-9
+    assert abs(st.lambda_ - info["lambda"]) <= lam_tol * info["lambda"]
+
+
+@pytest.mark.parametrize("size", [1e-60, 1e-80, 1e-95, 1e-200, 1e-290])
+def test_small_sensitivities(cuda, size):
+    rng = np.random.default_rng(41)
+    n = W.Mesh(*SMALL).n_elem
+    _check(cuda, SMALL, rng.uniform(0.05, 0.6, n), -size * rng.uniform(1e-4, 1.0, n), 0.35, 0.2)
