@@ -244,6 +244,7 @@ constexpr int kOcSeg = 64;        // undecided elements a CTA may list
 constexpr int kOcMine = 4;        // ... and a thread
 constexpr int kOcList = 1024;     // ... and the grid
 constexpr float kOcMargin = 3e-5f;
+constexpr float kOcNear = 4e-7f;     // what FP32 may be off by in a bound near 1
 constexpr double kOcWindow = 1.5e-5;
 
 struct OcElem {                   // an undecided element
@@ -397,7 +398,7 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
     sum_lo += lo;
     // (a by its bits: its copy may be 0; a candidate that is no number counts as
     // the upper bound)
-    sum_hi += __double_as_longlong(a) > 0 || f.x != f.x ? fminf(1.f, f.y + movef) : lo;
+    sum_hi += __double_as_longlong(a) > 0 || f.x != f.x ? fmaxf(lo, fminf(1.f, f.y + movef)) : lo;
     sum_a += f.x;
   };
   if constexpr (G > 0) {
@@ -501,9 +502,12 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
     each([&](int e, double a, float2 f) {
       const float t = f.x * sf;
       const float lo = fmaxf(0.f, f.y - movef), hi = fminf(1.f, f.y + movef);
-      if (t * (1.f + kOcMargin) < lo || __double_as_longlong(a) == 0) {
+      // (a lower bound above 1 holds whatever the upper one is; near 1 it is left
+      // to the undecided)
+      const bool crossed = lo > 1.f - kOcNear;
+      if (t * (1.f + kOcMargin) < lo || __double_as_longlong(a) == 0 || lo > 1.f + kOcNear) {
         cacc += oc_low(rho[e], move);
-      } else if (t * (1.f - kOcMargin) > hi) {
+      } else if (t * (1.f - kOcMargin) > hi && !crossed) {
         cacc += oc_high(rho[e], move);
       } else if (t * (1.f - kOcMargin) > lo && t * (1.f + kOcMargin) < hi && t > 1e-30f) {
         aacc += a;

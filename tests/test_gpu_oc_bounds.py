@@ -1,6 +1,6 @@
 """The OC update where FP32 copies of its values could mislead it, against the
 oracle's bisection (design 1e-9, multiplier 4e-10, as in test_gpu_design_edges.py):
-sensitivities whose candidates underflow FP32."""
+sensitivities whose candidates underflow FP32, designs above their upper bound."""
 import numpy as np
 import pytest
 
@@ -32,3 +32,16 @@ def test_small_sensitivities(cuda, size):
     rng = np.random.default_rng(41)
     n = W.Mesh(*SMALL).n_elem
     _check(cuda, SMALL, rng.uniform(0.05, 0.6, n), -size * rng.uniform(1e-4, 1.0, n), 0.35, 0.2)
+
+
+@pytest.mark.parametrize("over", [0.5, 1e-3])
+@pytest.mark.parametrize("shape", [SMALL, LARGE])
+def test_designs_above_one(cuda, shape, over):
+    """rho - move above 1 (by up to `over`): the lower bound then holds whatever the
+    upper one is.  Steep sensitivities there, so that the candidates lie above both."""
+    rng = np.random.default_rng(42)
+    n = W.Mesh(*shape).n_elem
+    above = rng.random(n) < (0.3 if over > 0.1 else 2e-3)
+    rho = np.where(above, 1.2 + over * rng.random(n), rng.uniform(0.05, 0.6, n))
+    dc = -np.where(above, 100.0, rng.uniform(1e-4, 1.0, n))
+    _check(cuda, shape, rho, dc, 0.6 if over > 0.1 else 0.35, 0.2)
