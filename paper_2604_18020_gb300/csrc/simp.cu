@@ -225,10 +225,11 @@ constexpr size_t energy_smem() {
 //      volume crosses the target within the window, narrows the window by
 //      Newton steps, and replays the bisection from [0, 1e9]: midpoints outside
 //      the window are decided by monotonicity, those inside by evaluation.
-// The replay takes the branches that the step by step bisection takes, so its
-// lambda and its last midpoint are the same.  A target below the sum of the
-// lower bounds, or above all that can be reached, decides every midpoint at
-// once.  Where the crossing is not confirmed (a volume that is flat there,
+// The replay takes the branches that the step by step bisection takes, but where
+// a volume differs from the target by no more than the roundings of its sum, so
+// its lambda and its last midpoint are the same to the bracket's 1e-10.  A target
+// below the sum of the lower bounds, or above all that can be reached, decides
+// every midpoint at once.  Where the crossing is not confirmed (a volume that is flat there,
 // values beyond FP32's range, more undecided elements than the lists hold) the
 // bisection evaluates every midpoint over all elements.
 //
@@ -244,7 +245,6 @@ constexpr int kOcSeg = 64;        // undecided elements a CTA may list
 constexpr int kOcMine = 4;        // ... and a thread
 constexpr int kOcList = 1024;     // ... and the grid
 constexpr float kOcMargin = 3e-5f;
-constexpr float kOcNear = 4e-7f;     // what FP32 may be off by in a bound near 1
 constexpr double kOcWindow = 1.5e-5;
 
 struct OcElem {                   // an undecided element
@@ -421,10 +421,12 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
     const double b0 = block_f32(sum_lo), b1 = block_f32(sum_hi);
     totals(b0, b1, block_f32(sum_a));
   }
-  // the volume exceeds the target at every midpoint, or at none (the FP32
-  // sums are good to far better than 1e-5)
-  const bool always = s_tot[0] * (1.0 - 1e-5) > target && move >= 0.0;
-  const bool never = s_tot[1] * (1.0 + 1e-5) < target && move >= 0.0;
+  // the volume exceeds the target at every midpoint, or at none: the FP32 sums are off
+  // by a rounding per element that a thread adds up, and by the roundings of rho
+  // and move in each bound
+  const double tol = 1e-5 + 6e-8 * (double)((n + stride - 1) / stride), off = 2.4e-7 * move * n;
+  const bool always = s_tot[0] * (1.0 - tol) - off > target && move >= 0.0;
+  const bool never = s_tot[1] * (1.0 + tol) + off < target && move >= 0.0;
 
   // ---- 1. Newton in FP32, kept between the scales known to give too little
   // (slo) and too much volume (shi); uniform over the grid
@@ -500,16 +502,18 @@ oc_kernel(const double* __restrict__ rho, const double* __restrict__ dc,
     int mine = 0;
     OcElem und[kOcMine];
     each([&](int e, double a, float2 f) {
-      const float t = f.x * sf;
-      const float lo = fmaxf(0.f, f.y - movef), hi = fminf(1.f, f.y + movef);
-      // (a lower bound above 1 holds whatever the upper one is; near 1 it is left
-      // to the undecided)
-      const bool crossed = lo > 1.f - kOcNear;
-      if (t * (1.f + kOcMargin) < lo || __double_as_longlong(a) == 0 || lo > 1.f + kOcNear) {
+      // bounds that the FP64 ones are sure to lie between: rho, move and their sum
+      // are rounded to FP32, which of a small lower bound leaves few bits
+      const float off = 1.2e-7f * (fabsf(f.y) + movef), d = f.y - movef, u = f.y + movef;
+      const float lo0 = fmaxf(0.f, d - off), lo1 = d > -off ? fmaxf(0.f, d) + off : 0.f;
+      const float hi0 = u > 1.f + off ? 1.f : u - off, hi1 = fminf(1.f, u + off);
+      // ... and candidates (a below FP32's normal range is 0 here)
+      const float t0 = f.x * sf * (1.f - kOcMargin), t1 = (f.x + 1.2e-38f) * sf * (1.f + kOcMargin);
+      if (t1 < lo0 || __double_as_longlong(a) == 0 || lo0 > hi1) {
         cacc += oc_low(rho[e], move);
-      } else if (t * (1.f - kOcMargin) > hi && !crossed) {
+      } else if (t0 > hi1 && hi0 > lo1) {
         cacc += oc_high(rho[e], move);
-      } else if (t * (1.f - kOcMargin) > lo && t * (1.f + kOcMargin) < hi && t > 1e-30f) {
+      } else if (t0 > lo1 && t1 < hi0 && t0 > 1e-30f) {
         aacc += a;
       } else {
         const double r = rho[e];

@@ -1,6 +1,7 @@
 """The OC update where FP32 copies of its values could mislead it, against the
 oracle's bisection (design 1e-9, multiplier 4e-10, as in test_gpu_design_edges.py):
-sensitivities whose candidates underflow FP32, designs above their upper bound."""
+sensitivities whose candidates underflow FP32, designs above their upper bound,
+lower bounds that FP32 holds to few bits."""
 import numpy as np
 import pytest
 
@@ -45,3 +46,18 @@ def test_designs_above_one(cuda, shape, over):
     rho = np.where(above, 1.2 + over * rng.random(n), rng.uniform(0.05, 0.6, n))
     dc = -np.where(above, 100.0, rng.uniform(1e-4, 1.0, n))
     _check(cuda, shape, rho, dc, 0.6 if over > 0.1 else 0.35, 0.2)
+
+
+@pytest.mark.parametrize("shape", [SMALL, LARGE])
+def test_lower_bounds_of_few_fp32_bits(cuda, shape):
+    """Densities just above the move limit whose candidates meet their lower bounds
+    at the solution: rho - move is known to 1e-8 in FP32, the bounds are 1e-4."""
+    rng = np.random.default_rng(43)
+    n = W.Mesh(*shape).n_elem
+    rho = 0.2 + 10.0 ** rng.uniform(-6.0, -3.0, n)
+    cand = (rho - 0.2) * (1.0 + rng.uniform(-2e-4, 2e-4, n))
+    free = rng.random(n) < 0.3
+    cand[free] = rng.uniform(0.05, 0.35, free.sum())
+    dc = -(cand / rho) ** 2 / n          # the candidates at lambda = 1
+    volume = np.fmax(rho - 0.2, np.fmin(rho + 0.2, cand)).mean()
+    _check(cuda, shape, rho, dc, float(volume), 0.2)
