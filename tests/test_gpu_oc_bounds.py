@@ -61,3 +61,27 @@ def test_lower_bounds_of_few_fp32_bits(cuda, shape):
     dc = -(cand / rho) ** 2 / n          # the candidates at lambda = 1
     volume = np.fmax(rho - 0.2, np.fmin(rho + 0.2, cand)).mean()
     _check(cuda, shape, rho, dc, float(volume), 0.2)
+
+
+@pytest.mark.parametrize("size", [1e8, 1.0, 1e-20, 2.0 ** -510, 2.0 ** -512, 1e-250])
+def test_square_root(cuda, size):
+    """Densities of 1/2 and no bound active: the new ones are sqrt(-dc n) times one
+    number, each rounded once more.  Their ratios to that root in extended precision
+    spread by at most 2 (2^-53 + 1.02 2^-53) if the root is good to 0.51 ulp; on both
+    sides of the exponent (2^-511) below which CUDA's sqrt takes over."""
+    import torch
+    from paper_2604_18020_gb300 import mfto
+    m = W.Mesh(*LARGE)
+    n = m.n_elem
+    cand = np.random.default_rng(44).uniform(0.06, 0.94, n)
+    dc = -(2.0 * cand) ** 2 * size / n
+    with mfto.Handle(*LARGE, np.zeros(m.n_node, np.uint8),
+                     mfto.default_params(volfrac=float(cand.mean()), move=0.45)) as h:
+        out = torch.empty(n, dtype=torch.float64, device=cuda)
+        h.oc_update(torch.full((n,), 0.5, dtype=torch.float64, device=cuda),
+                    torch.tensor(dc, device=cuda), out)
+    got = out.cpu().numpy()
+    assert got.min() > 0.055 and got.max() < 0.945
+    root = np.sqrt((dc * -float(n)).astype(np.longdouble))
+    ratio = got.astype(np.longdouble) / root
+    assert ratio.max() / ratio.min() - 1 <= 2.02 * 2.0 ** -52
