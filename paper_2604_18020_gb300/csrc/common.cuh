@@ -675,6 +675,7 @@ mfto_status gmg_cheb_col_launch(mfto_handle* h, int mode, const float* E, const 
 int64_t gmg_bytes(const mfto_handle* h);
 int64_t learned_bytes(const mfto_handle* h);
 void gmg_release(mfto_handle* h);
+void gmg_graph_release(mfto_handle* h);
 mfto_status gmg_solve(mfto_handle* h, const double* E, const double* f, double* u,
                       mfto_solve_stats* st);
 void mode_coefficients(double nu, double h, ModeCoef<double>* c64, ModeCoef<float>* c32);

@@ -1695,6 +1695,11 @@ mfto_status read_scalars(mfto_handle* h, GmgWs* w) {
 
 }  // namespace
 
+// captured cycles hold the element operator by value
+void gmg_graph_release(mfto_handle* h) {
+  if (h->gmg) drop_graph(h->gmg);
+}
+
 void gmg_release(mfto_handle* h) {
   if (!h || !h->gmg) return;
   GmgWs* w = h->gmg;

@@ -403,6 +403,12 @@ extern "C" mfto_status mfto_set_params(mfto_handle* h, const mfto_params* p) {
   mfto_status s = check_params(h, p);
   if (s != MFTO_OK) return s;
   MFTO_REQUIRE(h, p->max_rhs == h->max_rhs, "mfto_set_params: max_rhs is fixed at mfto_create");
+  // captured launches hold the element operator (and, in FP64, its tiles) by value
+  if (p->nu != h->p.nu) {
+    pcg_graph_release(h);
+    multi_graph_release(h);
+    gmg_graph_release(h);
+  }
   h->p = *p;
   return upload_params(h);
 }
