@@ -131,44 +131,27 @@ conv_bwd_data(const float* __restrict__ dout, int Cout, const __nv_bfloat16* __r
       }
 }
 
-// partial[chunk][co][ci][k] = sum_{v in chunk} dout[co][v] in[ci][v + d_k];
-// one block per (co, ci, chunk), fixed-order block reduction
-template <int K>
+// partial[chunk][co][ci] = sum_{v in chunk} dout[co][v] in[ci][v], the weight gradient
+// of a 1x1x1 layer; one block per (co, ci, chunk), fixed-order block reduction
 __global__ void __launch_bounds__(kNT)
-conv_bwd_weight(const float* __restrict__ in, int Cin, const float* __restrict__ dout, int Cout,
-                Dims d, int chunk, float* __restrict__ partial) {
-  constexpr int KK = K * K * K;
-  __shared__ float red[kNT / 32][KK];
-  const int V = d.V();
+conv1_bwd_weight(const float* __restrict__ in, int Cin, const float* __restrict__ dout, int Cout,
+                 int V, int chunk, float* __restrict__ partial) {
+  __shared__ float red[kNT / 32];
   const int co = blockIdx.x / Cin, ci = blockIdx.x % Cin;
   const int v0 = blockIdx.y * chunk, v1 = min(V, v0 + chunk);
-  float acc[KK];
-#pragma unroll
-  for (int k = 0; k < KK; ++k) acc[k] = 0.f;
   const float* g = dout + (size_t)co * V;
   const float* src = in + (size_t)ci * V;
-  for (int v = v0 + threadIdx.x; v < v1; v += kNT) {
-    const float gv = g[v];
-    const int z = v / (d.H * d.W), y = (v / d.W) % d.H, x = v % d.W;
-#pragma unroll
-    for (int k = 0; k < KK; ++k) {
-      int idx;
-      if (koff_ok(z, y, x, k, K, d, &idx)) acc[k] += gv * src[idx];
-    }
-  }
+  float s = 0.f;
+  for (int v = v0 + threadIdx.x; v < v1; v += kNT) s += g[v] * src[v];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int k = 0; k < KK; ++k) {
-    float s = acc[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) red[warp][k] = s;
-  }
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane == 0) red[warp] = s;
   __syncthreads();
-  for (int k = threadIdx.x; k < KK; k += kNT) {
-    float s = 0.f;
-    for (int q = 0; q < kNT / 32; ++q) s += red[q][k];
-    partial[(((size_t)blockIdx.y * Cout + co) * Cin + ci) * KK + k] = s;
+  if (threadIdx.x == 0) {
+    float t = 0.f;
+    for (int q = 0; q < kNT / 32; ++q) t += red[q];
+    partial[((size_t)blockIdx.y * Cout + co) * Cin + ci] = t;
   }
 }
 
@@ -385,7 +368,8 @@ unsigned cdiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
 // Measured on a GB300 against one plane at a time, its three halo planes staged
 // anew and the CTA waiting for its MMAs: the network's forward pass on 136 x 72 x
 // 72 nodes 944 against 1,442 us (994 with one weight buffer), loss and gradient
-// on 72 x 40 x 40 1,723 against 2,170 us (1,951); the same bits.
+// on 72 x 40 x 40 1,723 against 2,170 us (1,951); the same bits.  With the transfers
+// and weight gradients that came after, 784 and 1,620 us.
 constexpr int kCtTX = 8, kCtTY = 16;                  // output tile (M = 128)
 constexpr int kCtHX = kCtTX + 2, kCtHY = kCtTY + 2;   // staged halo plane
 constexpr int kCtPart = kCtHX * kCtHY * 16;           // one 8-channel part: 2,880 bytes
@@ -841,14 +825,13 @@ mfto_status conv_backward(mfto_nn* n, const NnLayer& L, const float* in, const f
     mfto_status s = wgrad_launch(n, L, in, dout, d);
     if (s != MFTO_OK) return s;
   } else {
-    const int KK = L.k * L.k * L.k;
     const int chunks = n_chunks(V);
     const int chunk = (V + chunks - 1) / chunks;
-    const size_t nw = (size_t)L.cout * L.cin * KK;
+    const size_t nw = (size_t)L.cout * L.cin;
     if ((size_t)chunks * nw > n->wpart_elems)
       return nfail(n, MFTO_INVALID_ARG, "weight partials too small");
     n->launches += 4;
-    conv_bwd_weight<1><<<dim3(L.cout * L.cin, chunks), kNT, 0, n->stream>>>(in, L.cin, dout, L.cout, d, chunk, n->wpart);
+    conv1_bwd_weight<<<dim3(L.cout * L.cin, chunks), kNT, 0, n->stream>>>(in, L.cin, dout, L.cout, V, chunk, n->wpart);
     sum_chunks<<<cdiv(nw, 256), 256, 0, n->stream>>>(n->wpart, (int)nw, chunks, n->grad + L.w_off);
     bias_grad<<<dim3(L.cout, chunks), kNT, 0, n->stream>>>(dout, L.cout, V, chunk, n->wpart);
     sum_chunks<<<cdiv(L.cout, 256), 256, 0, n->stream>>>(n->wpart, L.cout, chunks, n->grad + L.b_off);
@@ -1111,9 +1094,10 @@ extern "C" mfto_status mfto_nn_create(int32_t base, int32_t levels, int64_t max_
       const NnLayer& ly = n->layers[i];
       const int bi = (int)(i / 2);
       const int l = (i == n->layers.size() - 1) ? 0 : (bi < L ? bi : 2 * (L - 1) - bi);
-      const size_t need = (size_t)n_chunks((int)(TV >> (3 * l))) * ((size_t)ly.cout * ly.cin * ly.k * ly.k * ly.k + ly.cout);
-      wp = wp > need ? wp : need;
-      if (ly.k == 3) {
+      if (ly.k == 1) {
+        const size_t need = (size_t)n_chunks((int)(TV >> (3 * l))) * ((size_t)ly.cout * ly.cin + ly.cout);
+        wp = wp > need ? wp : need;
+      } else {
         // the weight gradient's partials: one wave of CTAs, each 128 pairs x 3
         // x its output channels; never more than one task per voxel
         const size_t row = (size_t)ly.cout * (9 * ly.cin + 1) * 3;
