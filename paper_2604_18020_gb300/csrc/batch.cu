@@ -560,7 +560,8 @@ int plan_tiles(const mfto_batch* b, int layers, std::vector<BatchTiles>& out) {
 
 // Tiles of the inner CG: the chunk length with the least time of the busiest
 // SM, a CTA taking its layers, the recomputed one and about two of start and
-// end.  FP64 tiles: whole columns cut into at most four chunks.
+// end.  FP64 tiles: whole columns cut into at most four chunks, whatever the
+// batch's size (a solve applies them once per refinement).
 mfto_status make_tiles(mfto_batch* b) {
   std::vector<BatchTiles> t;
   int best = 0, longest = 1;

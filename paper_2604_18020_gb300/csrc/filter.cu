@@ -6,13 +6,13 @@
 // boundary; W_e = sum_{i in N(e)} w_ei.  Terms are added in stencil order with
 // separate IEEE multiply and add (no fused multiply-add), so the result does
 // not depend on the compiler's contraction choices.  The weight matrix is
-// symmetric, so the transpose visits the same offsets; it divides x by W
-// once per element in a first pass (the same quotients the sum would form
-// once per element (the same quotients the sum would form term by term) and
-// then runs the forward sum on the quotients.
+// symmetric, so the transpose visits the same offsets and runs the forward sum
+// on the quotients x / W, formed once per element (the same quotients the sum
+// would form term by term).
 //
 // Radii in (sqrt 2, 2] (offsets of at most one element, 19 or 27 terms) take the
-// streaming kernel below, others the general one.
+// streaming kernel below, which divides as it stages a layer; others the general
+// one, after a pass that divides.
 #include "common.cuh"
 
 namespace {

@@ -133,7 +133,8 @@ struct FixStream {
 
 // Threads an SM holds at the K.v's launch bounds (at most 128 registers).  The
 // upper outputs of the element below wait in shared memory, each thread's own
-// (24 registers): 388 us at 256 x 128 x 150, against 408 with 12 warps of 168.
+// (24 registers): 31 us at 120 x 60 x 30, against 33 with 12 warps of 168 (52 both
+// at 55 x 55 x 165).
 constexpr int kFixThreads = 512;
 
 // Shared memory of the K.v: the stream, the shares of the other columns' nodes
@@ -326,7 +327,8 @@ __device__ __forceinline__ double kv_column_fixed_body(const double* __restrict_
 }
 
 // Tile shape and z-chunk: an SM's resident CTAs advance a layer in about 1.28 +
-// 0.00625 us per thread (measured: the integer pipes are half busy at 16
+// 0.00625 us per thread (measured, with one exponent for all components; now a
+// tenth more of both: the integer pipes are half busy at 16
 // warps, so a layer's latency counts as much as its work), a CTA takes its
 // layers and about 1.3 more, and the SM with the most CTAs sets the time.
 // copies: launches' worth of tiles in one grid.

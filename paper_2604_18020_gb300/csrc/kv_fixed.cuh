@@ -15,27 +15,27 @@
 //             converted back to FP64 by its owner
 // Sums and differences are exact; alignments, products by constants and the
 // modulus lose a few units of the last place.  So a share of an element carries
-// an error of at most one FP64 rounding (2^-53) of each component's own largest value
-// in the element, and a few 2^-56 of the largest mode difference of any component,
-// times E.  A block without strain shifts nothing of its neighbours away, however
-// stiff it is.
+// an error of at most one FP64 rounding (2^-53) of each component's own largest
+// value in the element, and a few 2^-56 of the largest mode difference of any
+// component, times E.  A block without strain shifts nothing of its neighbours
+// away, however stiff it is.
 //
 // FP64 sums in the mode basis carry 2^-53 E times the components' largest
 // values, but where their sums happen to be exact: against extended precision
 // (relative 2-norm; FP64 column kernel, then this) K u of a bending field over
-// graded moduli 3.3e-15, 1.1e-16, of a solved cantilever's u 5.8e-14, 5.4e-15; the
-// sensitivities 1.4e-15, 1.3e-16 and 2.3e-15, 1.5e-16.  What FP64 keeps and this does not:
-// where one component's exact strain (a simple shear, a rigid rotation) exceeds another
-// component's by more than 2^4, the smaller force keeps 57 bits of the larger, not
-// of itself.  kv_column64.cuh serves callers for whom that matters
-// (mfto_set_kv_variant).
+// graded moduli 3.3e-15, 1.1e-16, of a solved cantilever's u 5.8e-14, 5.4e-15;
+// the sensitivities 1.4e-15, 1.3e-16 and 2.3e-15, 1.5e-16.  What FP64 keeps and
+// this does not: where one component's exact strain (a simple shear, a rigid
+// rotation) exceeds another component's by more than 2^4, the smaller force keeps
+// 57 bits of the larger, not of itself.  kv_column64.cuh serves callers for whom
+// that matters (mfto_set_kv_variant).
 //
-// Measured on a GB300, y = K v, against the FP64 column kernel: 52 (components of one
-// size) to 63 us (components far apart) against 229 at 55 x 55 x 165, 31 to 35
-// against 117 at 120 x 60 x 30, 8 to 10 against 18 at 24 x 12 x 12.  About 1,150
-// instructions per element and layer, 1,350 with components far apart, issued on
-// about half of the cycles; the rest waits for the layer's barrier and for
-// dependent results.
+// Measured on a GB300, y = K v, the FP64 column kernel, then this with components of one
+// size and with components far apart: 1,971, 428 and 481 us at 256 x 128 x 150, 229, 52
+// and 62 at 55 x 55 x 165, 114, 31 and 34 at 120 x 60 x 30, 18.5, 9.3 and 10.3 at 24 x 12
+// x 12.  1,850 and 2,020 warp instructions per 32 elements, the tiles' halos included, issued
+// on 54 % of the cycles; the rest waits for the layer's barrier and for dependent
+// results.  (With one exponent for all components, 393 and 47 us at the first two.)
 #pragma once
 #include <math.h>
 #include <stdint.h>

@@ -137,9 +137,10 @@ compliance_kernel(const double* __restrict__ rho, const double* __restrict__ u,
 // The same on the fixed-point node stream (kv_column_fixed.cuh): the transforms
 // and the energy's squares on the integer pipes, about 12 FP64 operations per
 // element left (one conversion, powers and sums).  Measured on a GB300, p = 3,
-// against the kernel above, which serves the other Poisson's ratios: 303 against
-// 966 us at 256 x 128 x 150, 74 against 150 at 55 x 55 x 165, 49 against 76 at
-// 120 x 60 x 30 (the call, with its host round trip of about 25 us).
+// a displacement whose components lie far apart, against the kernel above, which
+// serves the other Poisson's ratios and variant 2: 337 against 930 us at 256 x 128 x 150,
+// 76 against 140 at 55 x 55 x 165, 43 against 67 at 120 x 60 x 30 (the call, with its host
+// round trip of about 25 us).
 template <int CX, int CY>
 __global__ void __launch_bounds__(CX * CY, kCol64Threads / (CX * CY))
 compliance_fixed_kernel(const double* __restrict__ rho, const double* __restrict__ u,
@@ -229,9 +230,10 @@ constexpr size_t energy_smem() {
 // a volume differs from the target by no more than the roundings of its sum, so
 // its lambda and its last midpoint are the same to the bracket's 1e-10.  A target
 // below the sum of the lower bounds, or above all that can be reached, decides
-// every midpoint at once.  Where the crossing is not confirmed (a volume that is flat there,
-// values beyond FP32's range, more undecided elements than the lists hold) the
-// bisection evaluates every midpoint over all elements.
+// every midpoint at once.  Where the crossing is not confirmed (a volume that is
+// flat there, values beyond FP32's range, more undecided elements than the lists
+// hold) the bisection evaluates every midpoint over all elements, after up to 24
+// passes in FP32.
 //
 // One cooperative grid; a grid barrier counts arrivals (release-add of one per
 // CTA, acquire-polls; bounded), and every CTA adds the per-CTA partials in the
@@ -262,8 +264,7 @@ struct OcUp {                     // the bisection whose every midpoint exceeds 
 // a = r sqrt(max(0, -dc) n), neg_n = -n.  The square root by Goldschmidt's
 // iteration with a final residual (P. Markstein, "Software division and square
 // root using Goldschmidt's algorithms", 2004) from the hardware's
-// approximation: 6 FP64 operations, the result within 0.51 ulp (the residual's
-// correction leaves about 2^-25 ulp before the last rounding); sqrt where the
+// approximation: 6 FP64 operations, the result within 0.51 ulp; sqrt where the
 // argument lies near the ends of the exponent range.
 __device__ __forceinline__ double oc_scale(double r, double dc, double neg_n) {
   const double x = dc * neg_n;
@@ -800,6 +801,8 @@ mfto_status compliance_launch(mfto_handle* h, const double* rho, const double* u
 
 mfto_status simp_init(mfto_handle* h) {
   const Grid g = make_grid(h->mesh);
+  // (the FP64 pipe's rule for both energy kernels: the fixed-point one, bound by issue and
+  // latency, has had none fitted to it)
   col64_choose(0, g.nelx, g.nely, g.nelz, 0.7, h->num_sms, &h->energy_shape, &h->energy_nzc);
   for (int i = 0; i < kCol64Shapes; ++i) {
     const mfto_status s = col64_dispatch(i, [&](auto shape) -> mfto_status {
