@@ -362,7 +362,8 @@ mfto_status mfto_batch_create(int32_t count, const mfto_mesh* meshes, const mfto
 mfto_status mfto_batch_destroy(mfto_batch* b);
 const char* mfto_batch_last_error(const mfto_batch* b);
 mfto_status mfto_batch_layout(const mfto_batch* b, int64_t* h_elem_off, int64_t* h_dof_off);
-/* d_Y = K(E) d_V for every instance, one launch (forms F64, F32). */
+/* d_Y = K(E) d_V for every instance, one launch (forms F64, F32; FP64 with the
+ * precision of mfto_set_kv_variant's 0, as in mfto_batch_solve's residuals). */
 mfto_status mfto_batch_kv(mfto_batch* b, mfto_form form, const void* d_E, const void* d_V,
                           void* d_Y);
 /* Element-block shape of the batch kernels (8x8x4, 8x4x8, 4x8x8, 16x4x4
